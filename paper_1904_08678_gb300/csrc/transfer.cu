@@ -335,6 +335,165 @@ __global__ void __launch_bounds__(8 * TR) k_restrict_gemm(cplx<R>* __restrict__ 
     }
 }
 
+// 4 to 15 FP32 rhs: bound by HBM (the vectors are read once for all rhs) as long as the
+// loads run ahead of the arithmetic.  The CTA's four warps split the aggregate's elements
+// (warp w takes the chunks w, w + 4, ... of RT_KT elements) and each forms the whole M x N
+// tile (M = LX VI vectors, N = LT NT rhs) of its share: lane (ti, tr) of the LX x LT lane
+// grid owns vectors ti + LX q and rhs tr + LT p.  Each warp stages its own chunks with
+// asynchronous 8-byte copies, RT_ST chunks in flight, so there is no block barrier before
+// the sum over the warps at the end; rows of RT_RS entries (80 bytes) put the 16-byte
+// reads of 8 rows on distinct banks, and one such read serves two elements.  12 rhs,
+// Nvec 24, 24^3x48 (2.3 GB): 0.7 ms, against 2.75 ms with one shared read per complex
+// MAC and two block barriers per 256 elements (a 12-rhs solve there: 755 -> 667 ms).  48 columns stay with k_restrict_gemm: there
+// the FMA pipe's register reads bound both (354 us on 16^3x32; this layout 506 us, its
+// 3 CTAs per SM leaving 2.2 waves of 1024).
+constexpr int RT_KT = 8, RT_RS = RT_KT + 2, RT_ST = 3, RT_W = 4;
+
+template <int LX, int VI, int NT>
+constexpr int restrict_tile_smem() {
+  constexpr int M = LX * VI, N = 32 / LX * NT;
+  constexpr int stage = RT_W * RT_ST * (M + N) * RT_RS * 8, red = RT_W * M * N * 8;
+  return stage > red ? stage : red;
+}
+
+// 8-byte asynchronous copy to shared memory; bytes = 0 fills with zeros (src is not read)
+__device__ __forceinline__ void cp_async8(uint32_t dst, const void* src, int bytes) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+}
+
+template <int LX, int VI, int NT>
+__global__ void __launch_bounds__(32 * RT_W)
+    k_restrict_tile(float2* __restrict__ out, const float2* __restrict__ in, const float2* __restrict__ vecs, int Vf,
+                    int nc, int bvol, int nvec, int nrhs, bool fine, FaceSel fs) {
+  constexpr int LT = 32 / LX, M = LX * VI, N = LT * NT, ROWS = M + N;
+  static_assert(ROWS % 4 == 0, "four rows per copy pass");
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int blk = blockIdx.x, s = blockIdx.y, r0 = blockIdx.z * N;
+  const int half = nc >> 1, nb = 2 * nvec;
+  const int nsite = fs.fd < 0 ? bvol : bvol / fs.b[fs.fd >> 1];
+  const int nelem = nsite * half, nchunk = (nelem + RT_KT - 1) / RT_KT;
+  const int Vc = Vf / bvol;
+  const long long fstride = (long long)Vf * nc;
+  float2* st = reinterpret_cast<float2*>(smem_raw) + (long long)warp * RT_ST * ROWS * RT_RS;
+  const int kl = lane & (RT_KT - 1), fl = lane >> 3;  // copy role: element kl of rows fl, fl + 4, ...
+  auto issue = [&](int chunk, int slot) {
+    if (chunk < nchunk) {
+      const int e = chunk * RT_KT + kl;
+      const bool ok = e < nelem;
+      long long a = 0;
+      if (ok) {
+        int c, f;
+        if (fine) { c = s * half + e / nsite; f = e % nsite; }
+        else { f = e / half; c = s * half + e % half; }
+        const int site = blk * bvol + face_site(fs, f);
+        a = fine ? (long long)c * Vf + site : (long long)site * nc + c;
+      }
+      uint32_t dst = smem_u32(st + (slot * ROWS + fl) * RT_RS + kl);
+#pragma unroll
+      for (int j = 0; j < ROWS / 4; ++j) {
+        const int row = fl + 4 * j;
+        const bool isx = row < M;
+        const int f = isx ? row : r0 + row - M;
+        const bool use = ok && f < (isx ? nvec : nrhs);
+        const float2* src = (isx ? vecs : in) + (use ? f * fstride + a : 0);
+        cp_async8(dst, src, use ? 8 : 0);
+        dst += 4 * RT_RS * 8;
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");  // one group per chunk, empty past the end
+  };
+  const int tr = lane % LT, ti = lane / LT;
+  // sums in two levels (a chunk, then the warp's share): one chain of 384 FP32 additions
+  // was 2.3x further from the FP64 result
+  float2 acc[VI][NT], tot[VI][NT];
+#pragma unroll
+  for (int q = 0; q < VI; ++q)
+#pragma unroll
+    for (int p = 0; p < NT; ++p) acc[q][p] = tot[q][p] = make_float2(0.f, 0.f);
+#pragma unroll
+  for (int i = 0; i < RT_ST - 1; ++i) issue(warp + RT_W * i, i);
+  int slot = 0;
+  for (int chunk = warp; chunk < nchunk; chunk += RT_W) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(RT_ST - 2) : "memory");
+    __syncwarp();  // the chunk is in shared memory for every lane; the oldest slot is free again
+    issue(chunk + RT_W * (RT_ST - 1), slot == 0 ? RT_ST - 1 : slot - 1);
+    const float2* xs = st + slot * ROWS * RT_RS;
+    const float2* ts = xs + M * RT_RS;
+#pragma unroll
+    for (int k = 0; k < RT_KT; k += 2) {
+      float4 x[VI], t[NT];
+#pragma unroll
+      for (int q = 0; q < VI; ++q) x[q] = *reinterpret_cast<const float4*>(xs + (ti + LX * q) * RT_RS + k);
+#pragma unroll
+      for (int p = 0; p < NT; ++p) t[p] = *reinterpret_cast<const float4*>(ts + (tr + LT * p) * RT_RS + k);
+#pragma unroll
+      for (int q = 0; q < VI; ++q)
+#pragma unroll
+        for (int p = 0; p < NT; ++p) {
+          cjmac(acc[q][p], make_float2(x[q].x, x[q].y), make_float2(t[p].x, t[p].y));
+          cjmac(acc[q][p], make_float2(x[q].z, x[q].w), make_float2(t[p].z, t[p].w));
+        }
+    }
+    slot = slot == RT_ST - 1 ? 0 : slot + 1;
+#pragma unroll
+    for (int q = 0; q < VI; ++q)
+#pragma unroll
+      for (int p = 0; p < NT; ++p) {
+        tot[q][p] += acc[q][p];
+        acc[q][p] = make_float2(0.f, 0.f);
+      }
+  }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  __syncthreads();
+  // sum over the warps in a fixed order
+  float2* red = reinterpret_cast<float2*>(smem_raw);
+#pragma unroll
+  for (int q = 0; q < VI; ++q)
+#pragma unroll
+    for (int p = 0; p < NT; ++p) red[((long long)warp * M + ti + LX * q) * N + tr + LT * p] = tot[q][p];
+  __syncthreads();
+  for (int k = threadIdx.x; k < M * N; k += 32 * RT_W) {
+    const int i = k % M, r = r0 + k / M;
+    if (i >= nvec || r >= nrhs) continue;
+    const float2* q = red + i * N + k / M;
+    const float2 v = (q[0] + q[M * N]) + (q[2 * M * N] + q[3 * M * N]);
+    out[((long long)r * Vc + blk) * nb + s * nvec + i] = v;
+  }
+}
+
+template <int LX, int VI, int NT>
+static void restrict_tile_v(float2* coarse, const float2* in, const float2* vecs, int Vf, int nc, int bvol, int nvec,
+                            int nrhs, bool fine, const FaceSel& fs, cudaStream_t st) {
+  constexpr int N = 32 / LX * NT, smem = restrict_tile_smem<LX, VI, NT>();
+  auto kern = k_restrict_tile<LX, VI, NT>;
+  if (smem > 48 * 1024) WCMG_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  kern<<<dim3(Vf / bvol, 2, (nrhs + N - 1) / N), 32 * RT_W, smem, st>>>(coarse, in, vecs, Vf, nc, bvol, nvec, nrhs,
+                                                                        fine, fs);
+  WCMG_LAUNCH_CHECK();
+}
+
+// N = 4, 8, 12 or 16 rhs per CTA, M = 8, 16, 24 or 32 vectors: at most three rhs and seven
+// vectors of a tile are padding.
+static void restrict_tile(float2* coarse, const float2* in, const float2* vecs, int Vf, int nc, int bvol, int nvec,
+                          int nrhs, bool fine, const FaceSel& fs, cudaStream_t st) {
+#define WCMG_RT(VI, NT) \
+  restrict_tile_v<8, VI, NT>(coarse, in, vecs, Vf, nc, bvol, nvec, nrhs, fine, fs, st)
+#define WCMG_RTN(VI)                      \
+  do {                                    \
+    if (nrhs <= 4) WCMG_RT(VI, 1);        \
+    else if (nrhs <= 8) WCMG_RT(VI, 2);   \
+    else if (nrhs <= 12) WCMG_RT(VI, 3);  \
+    else WCMG_RT(VI, 4);                  \
+  } while (0)
+  if (nvec <= 8) WCMG_RTN(1);
+  else if (nvec <= 16) WCMG_RTN(2);
+  else if (nvec <= 24) WCMG_RTN(3);
+  else WCMG_RTN(4);
+#undef WCMG_RTN
+#undef WCMG_RT
+}
+
 template <typename R, int VI, int RT>
 static void restrict_gemm_v(cplx<R>* coarse, const cplx<R>* in, const cplx<R>* vecs, int Vf, int nc, int bvol,
                             int nvec, int nrhs, bool fine, const FaceSel& fs, cudaStream_t st) {
@@ -361,6 +520,7 @@ static void restrict_gemm(cplx<R>* coarse, const cplx<R>* in, const cplx<R>* vec
   else restrict_gemm_vi<R, 4>(coarse, in, vecs, Vf, nc, bvol, nvec, nrhs, fine, fs, st);
 }
 
+// 4 to 15 rhs in FP64
 template <typename R, int RR>
 static void restrict_rr(cplx<R>* coarse, const cplx<R>* in, const cplx<R>* vecs, int Vf, int nc, int bvol, int nvec,
                         int nrhs, bool fine, const FaceSel& fs, cudaStream_t st) {
@@ -381,10 +541,14 @@ void launch_restrict(cplx<R>* coarse, const cplx<R>* in, const cplx<R>* vecs, in
   fs.fd = face;
   for (int k = 0; k < 4; ++k) fs.b[k] = block ? block[k] : 1;
   if (face >= 0 && !block) throw Error(-1, "face restriction needs the aggregate extents");
-  if (nrhs >= 16) restrict_gemm<R>(coarse, in, vecs, Vf, nc, bvol, nvec, nrhs, fine, fs, st);
-  else if (sizeof(R) == 4 && nrhs >= 8) restrict_rr<R, 8>(coarse, in, vecs, Vf, nc, bvol, nvec, nrhs, fine, fs, st);
-  else if (nrhs >= 4) restrict_rr<R, 4>(coarse, in, vecs, Vf, nc, bvol, nvec, nrhs, fine, fs, st);
-  else restrict_few<R>(coarse, in, vecs, Vf, nc, bvol, nvec, nrhs, fine, fs, st);
+  if (nrhs >= 16) {
+    restrict_gemm<R>(coarse, in, vecs, Vf, nc, bvol, nvec, nrhs, fine, fs, st);
+  } else if (nrhs >= 4) {
+    if constexpr (sizeof(R) == 4) restrict_tile(coarse, in, vecs, Vf, nc, bvol, nvec, nrhs, fine, fs, st);
+    else restrict_rr<R, 4>(coarse, in, vecs, Vf, nc, bvol, nvec, nrhs, fine, fs, st);
+  } else {
+    restrict_few<R>(coarse, in, vecs, Vf, nc, bvol, nvec, nrhs, fine, fs, st);
+  }
 }
 
 template <typename R>
