@@ -82,6 +82,19 @@ void launch_dslash_mr(cplx<R>* out, const cplx<R>* in, const cplx<R>* gauge, con
 template <typename R>
 void launch_restrict(cplx<R>* coarse, const cplx<R>* in, const cplx<R>* vecs, int Vf, int nc, int bvol, int nvec,
                      int nrhs, bool fine, cudaStream_t st, int face = -1, const int* block = nullptr);
+// Restriction of nrhs operator columns straight into block d of the link rows: rhs r is
+// column first + r (r < nfirst) or second + r.
+struct LinkCols {
+  int ld = 0, d = 0;
+  int first = 0, nfirst = 0, second = 0;
+};
+template <typename R>
+void launch_restrict_links(cplx<R>* links, const cplx<R>* in, const cplx<R>* vecs, int Vf, int nc, int bvol, int nvec,
+                           int nrhs, bool fine, cudaStream_t st, int face, const int* block, const LinkCols& lc);
+// Blocks that follow from sigma3 D_c sigma3 = D_c^dag (sigma3 = +1 on the first nvec basis
+// vectors of a site): A_{-mu}(x) = sigma3 A_{+mu}(x - mu)^dag sigma3 for the four directions.
+template <typename R>
+void launch_mirror_links(cplx<R>* links, const int* nbr, int Vc, int nvec, cudaStream_t st);
 template <typename R>
 void launch_prolong(cplx<R>* out, const cplx<R>* coarse, const cplx<R>* vecs, int Vf, int nc, int bvol, int nvec,
                     int nrhs, bool fine, cudaStream_t st);
@@ -160,9 +173,6 @@ void launch_links_to_5(L* dst, const L* src, int Vc, int nb, cudaStream_t st);
 void launch_links_to_mma(bf16c* dst, const bf16c* src, int Vc, int nb, cudaStream_t st);
 size_t coarse_mma4_smem(int nb, int ntile, int mm, int stages);
 size_t coarse_mma4_scratch_bytes(int Vc, int nb, int nrhs);
-// links[x][a][d*nb + b0 + j] = res[j][x][a] for j < ncols (res: restrict output of the column fields)
-template <typename R, typename L>
-void launch_scatter_links(L* links, const cplx<R>* res, int Vc, int nb, int d, int b0, int ncols, cudaStream_t st);
 template <typename Lin, typename Lout>
 void launch_convert_links(Lout* out, const Lin* in, long long n, cudaStream_t st);
 

@@ -253,10 +253,13 @@ static void restrict_few(cplx<R>* coarse, const cplx<R>* in, const cplx<R>* vecs
 // number of complex entries, so the staging stores (one row entry per lane) hit
 // distinct banks.
 constexpr int RST_KT = 32;
-template <typename R, int VI, int RT, int TR>
+// LINKS (coarsening): rhs r is a column of the coarse operator and the result goes straight
+// to block d of the link rows (lanes on consecutive columns: whole lines), instead of to
+// coarse fields that a second kernel scatters.
+template <typename R, int VI, int RT, int TR, bool LINKS>
 __global__ void __launch_bounds__(8 * TR) k_restrict_gemm(cplx<R>* __restrict__ out, const cplx<R>* __restrict__ in,
                                                           const cplx<R>* __restrict__ vecs, int Vf, int nc, int bvol,
-                                                          int nvec, int nrhs, bool fine, FaceSel fs) {
+                                                          int nvec, int nrhs, bool fine, FaceSel fs, LinkCols lc) {
   using T = cplx<R>;
   constexpr int NTH = 8 * TR;
   constexpr int NT = TR * RT;  // rhs per CTA
@@ -331,7 +334,13 @@ __global__ void __launch_bounds__(8 * TR) k_restrict_gemm(cplx<R>* __restrict__ 
 #pragma unroll
     for (int p = 0; p < RT; ++p) {
       const int i = ti + 8 * q, r = r0 + tr + TR * p;
-      if (i < nvec && r < nrhs) out[((long long)r * Vc + blk) * nb + s * nvec + i] = acc[q][p];
+      if (i < nvec && r < nrhs) {
+        if (LINKS)
+          out[((long long)blk * nb + s * nvec + i) * lc.ld + lc.d * nb + (r < lc.nfirst ? lc.first : lc.second) + r] =
+              acc[q][p];
+        else
+          out[((long long)r * Vc + blk) * nb + s * nvec + i] = acc[q][p];
+      }
     }
 }
 
@@ -494,12 +503,14 @@ static void restrict_tile(float2* coarse, const float2* in, const float2* vecs, 
 #undef WCMG_RT
 }
 
-template <typename R, int VI, int RT>
+template <typename R, int VI, int RT, bool LINKS = false>
 static void restrict_gemm_v(cplx<R>* coarse, const cplx<R>* in, const cplx<R>* vecs, int Vf, int nc, int bvol,
-                            int nvec, int nrhs, bool fine, const FaceSel& fs, cudaStream_t st) {
+                            int nvec, int nrhs, bool fine, const FaceSel& fs, cudaStream_t st,
+                            const LinkCols& lc = LinkCols()) {
   constexpr int TR = 16;
   const dim3 grid(Vf / bvol, 2, (nrhs + TR * RT - 1) / (TR * RT));
-  k_restrict_gemm<R, VI, RT, TR><<<grid, 8 * TR, 0, st>>>(coarse, in, vecs, Vf, nc, bvol, nvec, nrhs, fine, fs);
+  k_restrict_gemm<R, VI, RT, TR, LINKS>
+      <<<grid, 8 * TR, 0, st>>>(coarse, in, vecs, Vf, nc, bvol, nvec, nrhs, fine, fs, lc);
   WCMG_LAUNCH_CHECK();
 }
 
@@ -549,6 +560,31 @@ void launch_restrict(cplx<R>* coarse, const cplx<R>* in, const cplx<R>* vecs, in
   } else {
     restrict_few<R>(coarse, in, vecs, Vf, nc, bvol, nvec, nrhs, fine, fs, st);
   }
+}
+
+// Columns of the Galerkin operator: links(x)[s nvec + i][d nb + col(r)] = <v_i, in_r> over
+// chirality s of aggregate x (column tiles of 16, 32 or 48).
+template <typename R>
+void launch_restrict_links(cplx<R>* links, const cplx<R>* in, const cplx<R>* vecs, int Vf, int nc, int bvol, int nvec,
+                           int nrhs, bool fine, cudaStream_t st, int face, const int* block, const LinkCols& lc) {
+  if (nvec > 32) throw Error(-1, "restrict supports nvec <= 32");
+  FaceSel fs;
+  fs.fd = face;
+  for (int k = 0; k < 4; ++k) fs.b[k] = block[k];
+  const int vi = (nvec + 7) / 8;
+#define WCMG_RL(VI, RT) \
+  restrict_gemm_v<R, VI, RT, true>(links, in, vecs, Vf, nc, bvol, nvec, nrhs, fine, fs, st, lc)
+#define WCMG_RLN(VI)                      \
+  do {                                    \
+    if (nrhs <= 16) WCMG_RL(VI, 1);       \
+    else if (nrhs <= 32) WCMG_RL(VI, 2);  \
+    else WCMG_RL(VI, 3);                  \
+  } while (0)
+  if (vi <= 2) WCMG_RLN(2);
+  else if (vi == 3) WCMG_RLN(3);
+  else WCMG_RLN(4);
+#undef WCMG_RLN
+#undef WCMG_RL
 }
 
 template <typename R>
@@ -1067,6 +1103,8 @@ void launch_make_columns(cplx<R>* cols, const cplx<R>* vecs, int Vf, int nc, int
 #define WCMG_INST(R)                                                                                            \
   template void launch_restrict<R>(cplx<R>*, const cplx<R>*, const cplx<R>*, int, int, int, int, int, bool,     \
                                    cudaStream_t, int, const int*);                                              \
+  template void launch_restrict_links<R>(cplx<R>*, const cplx<R>*, const cplx<R>*, int, int, int, int, int,     \
+                                         bool, cudaStream_t, int, const int*, const LinkCols&);                 \
   template void launch_prolong<R>(cplx<R>*, const cplx<R>*, const cplx<R>*, int, int, int, int, int, bool,      \
                                   cudaStream_t);                                                                \
   template void launch_make_columns<R>(cplx<R>*, const cplx<R>*, int, int, int, int, int, bool, cudaStream_t);

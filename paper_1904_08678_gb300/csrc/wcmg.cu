@@ -161,6 +161,8 @@ struct Level {
   DevBuf<unsigned char> L5[4];
   bool l5_valid[4] = {false, false, false, false};
   bool sigma3 = false;
+  bool herm = false;  // this level's operator is sigma3-hermitian by construction: a Galerkin
+                      // product of D, or of such an operator (links given by a caller are not)
   LevelScalars sc;
   LevelScalars sc_s;  // the GMRES smoother's own Krylov state (it runs inside the outer FGMRES)
   DevBuf<unsigned char> colour;  // SAP: colour (coarse-coordinate parity) of each aggregate
@@ -1308,16 +1310,33 @@ static void coarsen_body(wcmg_ctx* c, int l) {
   WCMG_CUDA(cudaMemsetAsync(links, 0, (size_t)nl * sizeof(cplx<R>), c->st));
   const int chunk = std::min(nb, 48);
   cplx<R>* T = ws<R>(F, "co_T", chunk);
-  cplx<R>* res = ws<R>(C, "co_res", chunk);
+  // A sigma3-hermitian operator (the Wilson-clover D itself: gamma5; a Galerkin product of
+  // one) needs only the self block and the four forward hops: the backward blocks are the
+  // forward ones of the neighbours, sigma3-conjugated and transposed.
+  const bool herm = F.fine || F.herm;
+  const cplx<R>* vecs = Prec<R>::vecs(c, F);
+  LinkCols lc;
+  lc.ld = links_ld(nb);
+  auto columns = [&](int ncols, int dm) {
+    const int face = dm == 0 ? -1 : dm - 1;
+    lc.d = dm;
+    const double s = sizeof(cplx<R>), frac = face < 0 ? 1.0 : 1.0 / F.g.b[face >> 1];
+    KPROF(c, WCMG_K_RESTRICT, frac * (double)F.n() * s * (F.nvec + ncols) + (double)Vc * nb * s * ncols,
+          frac * (double)F.n() * 8.0 * F.nvec * ncols,
+          launch_restrict_links<R>(links, T, vecs, F.g.V, F.nc, F.g.bvol, F.nvec, ncols, F.fine, c->st, face, F.g.b,
+                                   lc));
+  };
   if (F.fine) {
     // fine level: both chirality columns of each vector from one stencil pass
     if (!c->have_gauge) throw Error(WCMG_ERR_STATE, "gauge field not set");
     const int vchunk = chunk / 2;
-    const cplx<R>* vecs = Prec<R>::vecs(c, F);
     const double V = F.g.V, s = sizeof(cplx<R>);
     for (int i0 = 0; i0 < F.nvec; i0 += vchunk) {
       const int nv = std::min(vchunk, F.nvec - i0);
-      for (int dm = 0; dm < 9; ++dm) {
+      lc.first = i0;
+      lc.nfirst = nv;
+      lc.second = F.nvec + i0 - nv;
+      for (int dm = 0; dm < 9; dm += dm == 0 ? 1 : 2) {
         const int mode = dm == 0 ? ST_BLOCK_INTERIOR : ST_FACE_HOP;
         const int hop = dm == 0 ? 0 : dm - 1;
         const double frac = dm == 0 ? 1.0 : 1.0 / F.g.b[hop >> 1];
@@ -1325,30 +1344,27 @@ static void coarsen_body(wcmg_ctx* c, int l) {
               frac * V * 1872.0 * 2 * nv,
               launch_dslash_chiral<R>(T, vecs + (long long)i0 * F.n(), Prec<R>::gauge(c), Prec<R>::clover(c),
                                       F.g.lg(), nv, mode, hop, c->st));
-        restrict_op<R>(c, l, res, T, 2 * nv, dm == 0 ? -1 : hop);
-        const long long half = (long long)nv * Vc * nb;
-        KPROF(c, WCMG_K_COARSEN, (double)Vc * nb * nv * 4.0 * sizeof(cplx<R>), 0.0,
-              (launch_scatter_links<R, cplx<R>>(links, res, Vc, nb, dm == 0 ? 0 : dm, i0, nv, c->st)));
-        KPROF(c, WCMG_K_COARSEN, 0.0, 0.0,
-              (launch_scatter_links<R, cplx<R>>(links, res + half, Vc, nb, dm == 0 ? 0 : dm, F.nvec + i0, nv,
-                                                c->st)));
+        columns(2 * nv, dm);
       }
     }
   }
   cplx<R>* cols = F.fine ? nullptr : ws<R>(F, "co_cols", chunk);
   for (int b0 = 0; !F.fine && b0 < nb; b0 += chunk) {
     const int ncols = std::min(chunk, nb - b0);
+    lc.first = b0;
+    lc.nfirst = ncols;
     KPROF(c, WCMG_K_COARSEN, 2.0 * F.n() * ncols * sizeof(cplx<R>), 0.0,
-          launch_make_columns<R>(cols, Prec<R>::vecs(c, F), F.g.V, F.nc, F.nvec, b0, ncols, F.fine, c->st));
-    for (int dm = 0; dm < 9; ++dm) {
+          launch_make_columns<R>(cols, vecs, F.g.V, F.nc, F.nvec, b0, ncols, F.fine, c->st));
+    for (int dm = 0; dm < 9; dm += herm && dm > 0 ? 2 : 1) {
       const int mode = dm == 0 ? ST_BLOCK_INTERIOR : ST_FACE_HOP;
-      const int hop = dm == 0 ? 0 : dm - 1;
-      apply_op<R>(c, l, T, cols, ncols, mode, hop);
-      restrict_op<R>(c, l, res, T, ncols, dm == 0 ? -1 : hop);
-      KPROF(c, WCMG_K_COARSEN, (double)Vc * nb * ncols * 2.0 * sizeof(cplx<R>), 0.0,
-            (launch_scatter_links<R, cplx<R>>(links, res, Vc, nb, dm == 0 ? 0 : dm, b0, ncols, c->st)));
+      apply_op<R>(c, l, T, cols, ncols, mode, dm == 0 ? 0 : dm - 1);
+      columns(ncols, dm);
     }
   }
+  if (herm)
+    KPROF(c, WCMG_K_COARSEN, (double)Vc * nb * nb * 8.0 * sizeof(cplx<R>), 0.0,
+          launch_mirror_links<R>(links, C.g.d_nbr.p, Vc, F.nvec, c->st));
+  C.herm = herm;
   C.have_op = true;
   C.ainv_valid = false;
   C.low_valid = false;
@@ -2429,6 +2445,7 @@ int wcmg_set_coarse_links(wcmg_ctx* c, int level, const void* A, int where, void
   L.have_op = true;
   L.ainv_valid = false;
   L.sigma3 = false;  // caller's blocks: no symmetry assumed, nine-block kernels only
+  L.herm = false;
   build_links5(c, level);
   if (c->p.coarse_eo && level == c->p.n_levels - 1) ensure_ainv(c, level);
   WCMG_CUDA(cudaStreamSynchronize(c->st));
