@@ -122,76 +122,127 @@ __device__ __forceinline__ Su3 mm(const Su3& a, const Su3& b) {
   return r;
 }
 
-// S[plane][chirality][2x2]: the chiral blocks of sigma_{mu nu} = i gamma_mu gamma_nu
-// (upper: i B_mu B_nu^dag, lower: i B_mu^dag B_nu), planes in the order
-// (0,1) (0,2) (0,3) (1,2) (1,3) (2,3).
-struct CloverSigma { double2 S[6][2][4]; };
+// acc += s a b, acc += s a b^dag, acc += s a^dag b
+template <int S>
+__device__ __forceinline__ void mm_add(Su3& acc, const Su3& a, const Su3& b) {
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int j = 0; j < 3; ++j)
+#pragma unroll
+      for (int k = 0; k < 3; ++k) cmac(acc.m[3 * i + j], S > 0 ? a.m[3 * i + k] : -a.m[3 * i + k], b.m[3 * k + j]);
+}
 
-__global__ void k_clover_build(double2* __restrict__ clov, const double2* __restrict__ g, const int* __restrict__ nbr,
-                               int V, double diag, double half_csw, CloverSigma sig) {
-  int s = blockIdx.x * blockDim.x + threadIdx.x;
+// The clover term in two FP64-bound kernels.  With the staple difference
+//   T(x) = U_nu(x+mu) U_mu(x+nu)^dag U_nu(x)^dag - U_nu(x+mu-nu)^dag U_mu(x-nu)^dag U_nu(x-nu)
+// the four leaves Q of the (mu, nu) plane at x satisfy
+//   Q - Q^dag = X - X^dag,   X = U_mu(x) T(x) + T(x-mu) U_mu(x-mu)
+// (leaf 1 - leaf 4^dag is the first product, leaf 2 - leaf 3^dag the second; only the links'
+// products are used, no unitarity), so T, formed once per site and plane (4 products of
+// 3x3 matrices), serves two sites: 6 products per plane and site instead of 12 for four
+// separate leaves.  The chiral blocks of sigma_{mu nu} are signed Pauli matrices, so the
+// site blocks are sums of the i Fhat (no products).  FP64 units: 2 DFMA per cycle and SM.
+// 24^3x48: 10.4 ms before, 4.4 ms now (2.8 + 1.6).
+// T: [6][9][V], planes in the order (0,1) (0,2) (0,3) (1,2) (1,3) (2,3).
+__global__ void __launch_bounds__(128) k_clover_staple(double2* __restrict__ T, const double2* __restrict__ g,
+                                                       const int* __restrict__ nbr, int V) {
+  const int s = blockIdx.x * blockDim.x + threadIdx.x, plane = blockIdx.y;
   if (s >= V) return;
-  double2 C[2][6][6];
+  const int mu = plane < 3 ? 0 : plane < 5 ? 1 : 2, nu = plane < 3 ? plane + 1 : plane < 5 ? plane - 1 : 3;
+  const int xpm = nbr[(2 * mu) * V + s], xpn = nbr[(2 * nu) * V + s], xmn = nbr[(2 * nu + 1) * V + s];
+  const int xpm_mn = nbr[(2 * nu + 1) * V + xpm];  // x + mu - nu
+  Su3 r = mm(load_u(g, V, nu, xpm), dag(mm(load_u(g, V, nu, s), load_u(g, V, mu, xpn))));
+  mm_add<-1>(r, dag(mm(load_u(g, V, mu, xmn), load_u(g, V, nu, xpm_mn))), load_u(g, V, nu, xmn));
+  double2* t = T + (long long)plane * 9 * V + s;
 #pragma unroll
-  for (int h = 0; h < 2; ++h)
+  for (int k = 0; k < 9; ++k) t[(long long)k * V] = r.m[k];
+}
+
+struct CloverSign { double s[6][2]; };  // [plane][chirality]: sigma_{mu nu} = s sigma_k
+
+// H += sign i (X - X^dag) of one plane for both chiralities, as the Hermitian matrix's
+// diagonal (d) and upper off-diagonal entries (o: 01, 02, 12).  The diagonal needs
+// only the imaginary parts of X's.
+struct Herm3 { double d[3]; double2 o[3]; };
+__device__ __forceinline__ void clover_plane(Herm3 (&h)[2], const double2* __restrict__ T,
+                                             const double2* __restrict__ g, const int* __restrict__ nbr, int V, int s,
+                                             int mu, int plane, double s0, double s1) {
+  const int xmm = nbr[(2 * mu + 1) * V + s];
+  double2 off[6];  // X01, X02, X12, X10, X20, X21
+  double im[3] = {0, 0, 0};
 #pragma unroll
-    for (int i = 0; i < 6; ++i)
+  for (int k = 0; k < 6; ++k) off[k] = make_double2(0, 0);
 #pragma unroll
-      for (int j = 0; j < 6; ++j) C[h][i][j] = make_double2(i == j ? diag : 0.0, 0.0);
-  int plane = 0;
-  for (int mu = 0; mu < 4; ++mu) {
-    for (int nu = mu + 1; nu < 4; ++nu, ++plane) {
-      const int xpm = nbr[(2 * mu) * V + s], xmm = nbr[(2 * mu + 1) * V + s];
-      const int xpn = nbr[(2 * nu) * V + s], xmn = nbr[(2 * nu + 1) * V + s];
-      const int xmm_pn = nbr[(2 * nu) * V + xmm];      // x - mu + nu
-      const int xmm_mn = nbr[(2 * nu + 1) * V + xmm];  // x - mu - nu
-      const int xpm_mn = nbr[(2 * nu + 1) * V + xpm];  // x + mu - nu
-      Su3 Umx = load_u(g, V, mu, s), Unx = load_u(g, V, nu, s);
-      Su3 Um_mm = load_u(g, V, mu, xmm), Un_mn = load_u(g, V, nu, xmn);
-      // leaf 1: U_mu(x) U_nu(x+mu) U_mu(x+nu)^dag U_nu(x)^dag
-      Su3 Q = mm(mm(Umx, load_u(g, V, nu, xpm)), mm(dag(load_u(g, V, mu, xpn)), dag(Unx)));
-      // leaf 2: U_nu(x) U_mu(x-mu+nu)^dag U_nu(x-mu)^dag U_mu(x-mu)
-      Su3 L = mm(mm(Unx, dag(load_u(g, V, mu, xmm_pn))), mm(dag(load_u(g, V, nu, xmm)), Um_mm));
+  for (int half = 0; half < 2; ++half) {
+    const Su3 u = load_u(g, V, mu, half ? xmm : s), t = load_u(T, V, plane, half ? xmm : s);
+    const Su3& a = half ? t : u;
+    const Su3& b = half ? u : t;
 #pragma unroll
-      for (int k = 0; k < 9; ++k) Q.m[k] += L.m[k];
-      // leaf 3: U_mu(x-mu)^dag U_nu(x-mu-nu)^dag U_mu(x-mu-nu) U_nu(x-nu)
-      L = mm(mm(dag(Um_mm), dag(load_u(g, V, nu, xmm_mn))), mm(load_u(g, V, mu, xmm_mn), Un_mn));
+    for (int k = 0; k < 3; ++k) {
 #pragma unroll
-      for (int k = 0; k < 9; ++k) Q.m[k] += L.m[k];
-      // leaf 4: U_nu(x-nu)^dag U_mu(x-nu) U_nu(x+mu-nu) U_mu(x)^dag
-      L = mm(mm(dag(Un_mn), load_u(g, V, mu, xmn)), mm(load_u(g, V, nu, xpm_mn), dag(Umx)));
-#pragma unroll
-      for (int k = 0; k < 9; ++k) Q.m[k] += L.m[k];
-      // i Fhat = i (Q - Q^dag) / 8  (Hermitian)
-      double2 iF[9];
-#pragma unroll
-      for (int a = 0; a < 3; ++a)
-#pragma unroll
-        for (int b = 0; b < 3; ++b) iF[3 * a + b] = mul_i(0.125 * (Q.m[3 * a + b] - conjg(Q.m[3 * b + a])));
-#pragma unroll
-      for (int h = 0; h < 2; ++h)
-#pragma unroll
-        for (int p = 0; p < 2; ++p)
-#pragma unroll
-          for (int q = 0; q < 2; ++q) {
-            const double2 sp = half_csw * sig.S[plane][h][2 * p + q];
-#pragma unroll
-            for (int a = 0; a < 3; ++a)
-#pragma unroll
-              for (int b = 0; b < 3; ++b) cmac(C[h][3 * p + a][3 * q + b], sp, iF[3 * a + b]);
-          }
+      for (int i = 0; i < 3; ++i) im[i] += a.m[3 * i + k].x * b.m[3 * k + i].y + a.m[3 * i + k].y * b.m[3 * k + i].x;
+      cmac(off[0], a.m[k], b.m[3 * k + 1]);
+      cmac(off[1], a.m[k], b.m[3 * k + 2]);
+      cmac(off[2], a.m[3 + k], b.m[3 * k + 2]);
+      cmac(off[3], a.m[3 + k], b.m[3 * k]);
+      cmac(off[4], a.m[6 + k], b.m[3 * k]);
+      cmac(off[5], a.m[6 + k], b.m[3 * k + 1]);
     }
   }
 #pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const double2 o = mul_i(off[i] - conjg(off[3 + i]));
+    h[0].d[i] -= 2.0 * s0 * im[i];
+    h[1].d[i] -= 2.0 * s1 * im[i];
+    h[0].o[i] += s0 * o;
+    h[1].o[i] += s1 * o;
+  }
+}
+
+// C = diag + sum_k sigma_k (x) H_k per chirality: [[d + H_z, H_x - i H_y], [.., d - H_z]]
+__global__ void __launch_bounds__(128) k_clover_build(double2* __restrict__ clov, const double2* __restrict__ T,
+                                                      const double2* __restrict__ g, const int* __restrict__ nbr,
+                                                      int V, double diag, CloverSign sg) {
+  const int s = blockIdx.x * blockDim.x + threadIdx.x;
+  if (s >= V) return;
+  const Herm3 zero = {{0, 0, 0}, {make_double2(0, 0), make_double2(0, 0), make_double2(0, 0)}};
+  {
+    Herm3 z[2] = {zero, zero};  // sigma_z: planes (0,1), (2,3)
+    clover_plane(z, T, g, nbr, V, s, 0, 0, sg.s[0][0], sg.s[0][1]);
+    clover_plane(z, T, g, nbr, V, s, 2, 5, sg.s[5][0], sg.s[5][1]);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      double2* c = clov + (long long)(18 * h) * V + s;
+      // diagonal pairs (0,1) (2,3) (4,5) of the 6x6 block
+      c[0] = make_double2(diag + z[h].d[0], diag + z[h].d[1]);
+      c[(long long)V] = make_double2(diag + z[h].d[2], diag - z[h].d[0]);
+      c[2LL * V] = make_double2(diag - z[h].d[1], diag - z[h].d[2]);
+      // upper entries in rows: 3: (0,1) (0,2) . . .  8: (1,2) . . .  15: (3,4) (3,5) (4,5)
+      c[3LL * V] = z[h].o[0];
+      c[4LL * V] = z[h].o[1];
+      c[8LL * V] = z[h].o[2];
+      c[15LL * V] = -z[h].o[0];
+      c[16LL * V] = -z[h].o[1];
+      c[17LL * V] = -z[h].o[2];
+    }
+  }
+  Herm3 x[2] = {zero, zero}, y[2] = {zero, zero};  // sigma_x: (0,3), (1,2); sigma_y: (0,2), (1,3)
+  clover_plane(x, T, g, nbr, V, s, 0, 2, sg.s[2][0], sg.s[2][1]);
+  clover_plane(x, T, g, nbr, V, s, 1, 3, sg.s[3][0], sg.s[3][1]);
+  clover_plane(y, T, g, nbr, V, s, 0, 1, sg.s[1][0], sg.s[1][1]);
+  clover_plane(y, T, g, nbr, V, s, 1, 4, sg.s[4][0], sg.s[4][1]);
+#pragma unroll
   for (int h = 0; h < 2; ++h) {
+    double2* c = clov + (long long)(18 * h) * V + s;
+    // entries (a, 3 + b) of H_x - i H_y: row 0 at 5, 6, 7, row 1 at 9, 10, 11, row 2 at 12, 13, 14
 #pragma unroll
-    for (int k = 0; k < 3; ++k)
-      clov[(long long)(18 * h + k) * V + s] = make_double2(C[h][2 * k][2 * k].x, C[h][2 * k + 1][2 * k + 1].x);
-    int o = 3;
+    for (int a = 0; a < 3; ++a) c[(long long)(a == 0 ? 5 : a == 1 ? 10 : 14) * V] = make_double2(x[h].d[a], -y[h].d[a]);
 #pragma unroll
-    for (int i = 0; i < 6; ++i)
-#pragma unroll
-      for (int j = i + 1; j < 6; ++j) clov[(long long)(18 * h + o++) * V + s] = C[h][i][j];
+    for (int k = 0; k < 3; ++k) {  // k: (0,1) (0,2) (1,2)
+      const double2 xo = x[h].o[k], yo = y[h].o[k];
+      c[(long long)(k == 0 ? 6 : k == 1 ? 7 : 11) * V] = xo - mul_i(yo);
+      c[(long long)(k == 0 ? 9 : k == 1 ? 12 : 13) * V] = conjg(xo) - mul_i(conjg(yo));
+    }
   }
 }
 
@@ -252,42 +303,28 @@ __global__ void k_clover_pack(double2* __restrict__ clov, const double2* __restr
   }
 }
 
-static CloverSigma make_sigma() {
-  // B_mu as 2x2 complex (row-major)
-  double2 B[4][4];
-  const double2 z = make_double2(0, 0), one = make_double2(1, 0), mi = make_double2(0, -1);
-  // B_x = -i sigma_1 ; B_y = -i sigma_2 ; B_z = -i sigma_3 ; B_t = 1
-  double2 Bx[4] = {z, mi, mi, z};
-  double2 By[4] = {z, make_double2(-1, 0), one, z};
-  double2 Bz[4] = {mi, z, z, make_double2(0, 1)};
-  double2 Bt[4] = {one, z, z, one};
-  for (int k = 0; k < 4; ++k) { B[0][k] = Bx[k]; B[1][k] = By[k]; B[2][k] = Bz[k]; B[3][k] = Bt[k]; }
-  auto mul = [](const double2* a, const double2* b, double2* r, bool dag_a, bool dag_b) {
-    for (int i = 0; i < 2; ++i)
-      for (int j = 0; j < 2; ++j) {
-        double2 acc = make_double2(0, 0);
-        for (int k = 0; k < 2; ++k) {
-          double2 x = dag_a ? conjg(a[2 * k + i]) : a[2 * i + k];
-          double2 y = dag_b ? conjg(b[2 * j + k]) : b[2 * k + j];
-          acc += cmul(x, y);
-        }
-        r[2 * i + j] = mul_i(acc);
-      }
-  };
-  CloverSigma cs;
-  int plane = 0;
-  for (int mu = 0; mu < 4; ++mu)
-    for (int nu = mu + 1; nu < 4; ++nu, ++plane) {
-      mul(B[mu], B[nu], cs.S[plane][0], false, true);   // i B_mu B_nu^dag
-      mul(B[mu], B[nu], cs.S[plane][1], true, false);   // i B_mu^dag B_nu
-    }
-  return cs;
+// Signs of the chiral blocks of sigma_{mu nu} = i gamma_mu gamma_nu (upper: i B_mu
+// B_nu^dag, lower: i B_mu^dag B_nu) with B_k = -i sigma_k, B_t = 1: for spatial planes
+// i sigma_j sigma_k = -eps_{jkl} sigma_l in both; with t, i B_j = sigma_j above and
+// i B_j^dag = -sigma_j below.
+static CloverSign clover_sign(double f) {
+  const double up[6] = {-1, 1, 1, -1, 1, 1};   // (0,1)z (0,2)y (0,3)x (1,2)x (1,3)y (2,3)z
+  const double lo[6] = {-1, 1, -1, -1, -1, -1};
+  CloverSign c;
+  for (int p = 0; p < 6; ++p) {
+    c.s[p][0] = f * up[p];
+    c.s[p][1] = f * lo[p];
+  }
+  return c;
 }
 
+// scratch: 54 V entries (the staples of the six planes)
 void launch_clover_build(double2* clov, const double2* gauge64, const int* nbr, int V, double m0, double csw,
-                         cudaStream_t st) {
-  static const CloverSigma sig = make_sigma();
-  k_clover_build<<<nblk(V, 64), 64, 0, st>>>(clov, gauge64, nbr, V, 4.0 + m0, 0.5 * csw, sig);
+                         double2* scratch, cudaStream_t st) {
+  k_clover_staple<<<dim3(nblk(V, 128), 6), 128, 0, st>>>(scratch, gauge64, nbr, V);
+  WCMG_LAUNCH_CHECK();
+  // C = 4 + m0 + (c_sw / 2) sum sigma (x) i Fhat, i Fhat = i (Q - Q^dag) / 8
+  k_clover_build<<<nblk(V, 128), 128, 0, st>>>(clov, scratch, gauge64, nbr, V, 4.0 + m0, clover_sign(csw / 16.0));
   WCMG_LAUNCH_CHECK();
 }
 void launch_clover_expand(double2* ext, const double2* clov, const int* perm, int V, cudaStream_t st) {

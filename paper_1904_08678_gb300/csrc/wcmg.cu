@@ -2228,6 +2228,18 @@ void wcmg_destroy(wcmg_ctx* ctx) { delete ctx; }
 
 const char* wcmg_last_error(const wcmg_ctx* ctx) { return ctx ? ctx->err.c_str() : "null context"; }
 
+extern "C++" {
+static void clover_build(wcmg_ctx* c) {
+  Level& L = c->L[0];
+  const int V = L.g.V;
+  // the staples (864 bytes per site) live in the coarsening's column workspace, which no
+  // set-up runs concurrently with
+  double2* t = inner64(c) ? ws<double>(L, "co_T", 5) : reinterpret_cast<double2*>(ws<float>(L, "co_T", 9));
+  KPROF(c, WCMG_K_CLOVER, 36.0 * V * 16 * 5, 0,
+        launch_clover_build(c->clover64.p, c->gauge64.p, L.g.d_nbr.p, V, c->p.m0, c->p.csw, t, c->st));
+}
+}  // extern "C++"
+
 int wcmg_set_gauge(wcmg_ctx* c, const void* U, int where, void* stream) {
   API_BEGIN(c)
   c->st = (cudaStream_t)stream;
@@ -2240,8 +2252,7 @@ int wcmg_set_gauge(wcmg_ctx* c, const void* U, int where, void* stream) {
   c->clover32.ensure((size_t)36 * V);
   KPROF(c, WCMG_K_PACK, 36.0 * V * 32, 0, launch_pack_gauge<double>(c->gauge64.p, u, L.g.d_perm.p, V, c->st));
   launch_pack_gauge<float>(c->gauge32.p, u, L.g.d_perm.p, V, c->st);
-  KPROF(c, WCMG_K_CLOVER, 36.0 * V * 16 * 5, 0,
-        launch_clover_build(c->clover64.p, c->gauge64.p, L.g.d_nbr.p, V, c->p.m0, c->p.csw, c->st));
+  clover_build(c);
   clover_derived(c);
   c->have_gauge = true;
   WCMG_CUDA(cudaStreamSynchronize(c->st));
@@ -2255,10 +2266,7 @@ int wcmg_set_clover(wcmg_ctx* c, double csw, void* stream) {
   if (!c->have_gauge) throw Error(WCMG_ERR_STATE, "gauge field not set");
   if (!std::isfinite(csw)) throw Error(WCMG_ERR_ARG, "csw must be finite");
   c->p.csw = csw;
-  Level& L = c->L[0];
-  const int V = L.g.V;
-  KPROF(c, WCMG_K_CLOVER, 36.0 * V * 16 * 5, 0,
-        launch_clover_build(c->clover64.p, c->gauge64.p, L.g.d_nbr.p, V, c->p.m0, c->p.csw, c->st));
+  clover_build(c);
   clover_derived(c);
   WCMG_CUDA(cudaStreamSynchronize(c->st));
   c->prof.flush();
