@@ -235,39 +235,137 @@ void launch_scale_dev(cplx<R>* y, const cplx<R>* x, const double* s, int inv_sqr
   WCMG_LAUNCH_CHECK();
 }
 
-// The step reads the residual from rin and writes the new one to r (rin = r in place;
-// the first step reads b itself).  X_ZERO: x is known to be 0 (first step: not read);
-// R_NEXT = false: the new r is not needed (last step: not written).  Same arithmetic in
-// every variant.
+// ---- minimal-residual updates ----
+// Bound by HBM: what counts is how often the fields are read and written.  A pair of steps
+// k, k + 1 shares one update of x: x += alpha_k r_k + alpha_{k+1} r_{k+1}, with r_{k+1}
+// written over p_k so that r_k survives.  Four steps from x = 0 then move 15 fields (17
+// with one update of x per step), and 16 when they are added to a given x (18, and 3 more
+// for a separate addition).  16-byte accesses: n is even on every level and the fields
+// start on 16 bytes, so an FP32 thread takes two entries.
+template <typename R> struct MrVec;
+template <> struct MrVec<double> { using type = double2; static constexpr int n = 1; };
+template <> struct MrVec<float> { using type = float4; static constexpr int n = 2; };
+__device__ __forceinline__ void vmac(double2& a, double2 s, double2 v) { cmac(a, s, v); }
+__device__ __forceinline__ void vmac(float4& a, float2 s, float4 v) {
+  float2 lo = make_float2(a.x, a.y), hi = make_float2(a.z, a.w);
+  cmac(lo, s, make_float2(v.x, v.y));
+  cmac(hi, s, make_float2(v.z, v.w));
+  a = make_float4(lo.x, lo.y, hi.x, hi.y);
+}
+__device__ __forceinline__ double2 vsub(double2 a, double2 s, double2 v) { return a - cmul(s, v); }
+__device__ __forceinline__ float4 vsub(float4 a, float2 s, float4 v) {
+  const float2 lo = make_float2(a.x, a.y) - cmul(s, make_float2(v.x, v.y));
+  const float2 hi = make_float2(a.z, a.w) - cmul(s, make_float2(v.z, v.w));
+  return make_float4(lo.x, lo.y, hi.x, hi.y);
+}
+template <typename V> __device__ __forceinline__ V vzero() {
+  V v;
+  memset(&v, 0, sizeof(V));
+  return v;
+}
+template <typename R>
+__device__ __forceinline__ cplx<R> mr_alpha(const double2* pr, const double* pp, int q) {
+  const double d = pp[q];
+  return d != 0.0 ? cmk((R)(pr[q].x / d), (R)(pr[q].y / d)) : czero<R>();
+}
+
 template <typename R, bool X_ZERO, bool R_NEXT>
-__global__ void k_mr_update(cplx<R>* __restrict__ x, cplx<R>* r, const cplx<R>* rin, const cplx<R>* __restrict__ p,
-                            const double2* __restrict__ pr, const double* __restrict__ pp, long long n) {
+__global__ void k_mr_update(cplx<R>* __restrict__ x, cplx<R>* __restrict__ r, const cplx<R>* __restrict__ p,
+                            const double2* __restrict__ pr, const double* __restrict__ pp, long long nv) {
+  using V = typename MrVec<R>::type;
   __shared__ cplx<R> a_s;
   const int q = blockIdx.y;
-  if (threadIdx.x == 0) {
-    const double d = pp[q];
-    a_s = d != 0.0 ? cmk((R)(pr[q].x / d), (R)(pr[q].y / d)) : czero<R>();
-  }
+  if (threadIdx.x == 0) a_s = mr_alpha<R>(pr, pp, q);
   __syncthreads();
   const long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (e >= n) return;
-  const cplx<R> a = a_s;
-  const long long o = (long long)q * n + e;
-  const cplx<R> rv = rin[o];
-  cplx<R> xv = X_ZERO ? czero<R>() : x[o];
-  cmac(xv, a, rv);
-  x[o] = xv;
-  if (R_NEXT) r[o] = rv - cmul(a, p[o]);
+  if (e >= nv) return;
+  const long long o = (long long)q * nv + e;
+  const V rv = reinterpret_cast<V*>(r)[o];
+  V xv = X_ZERO ? vzero<V>() : reinterpret_cast<V*>(x)[o];
+  vmac(xv, a_s, rv);
+  reinterpret_cast<V*>(x)[o] = xv;
+  if (R_NEXT) reinterpret_cast<V*>(r)[o] = vsub(rv, a_s, reinterpret_cast<const V*>(p)[o]);
+}
+template <typename R>
+__global__ void k_mr_residual(cplx<R>* __restrict__ p, const cplx<R>* __restrict__ r, const double2* __restrict__ pr,
+                              const double* __restrict__ pp, long long nv) {
+  using V = typename MrVec<R>::type;
+  __shared__ cplx<R> a_s;
+  const int q = blockIdx.y;
+  if (threadIdx.x == 0) a_s = mr_alpha<R>(pr, pp, q);
+  __syncthreads();
+  const long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (e >= nv) return;
+  const long long o = (long long)q * nv + e;
+  V* pv = reinterpret_cast<V*>(p) + o;
+  *pv = vsub(reinterpret_cast<const V*>(r)[o], a_s, *pv);
+}
+template <typename R, bool X_ZERO, bool R_NEXT>
+__global__ void k_mr_pair(cplx<R>* __restrict__ x, const cplx<R>* __restrict__ r0, cplx<R>* __restrict__ r1,
+                          const cplx<R>* __restrict__ p1, const double2* __restrict__ pr0,
+                          const double* __restrict__ pp0, const double2* __restrict__ pr1,
+                          const double* __restrict__ pp1, long long nv) {
+  using V = typename MrVec<R>::type;
+  __shared__ cplx<R> a_s[2];
+  const int q = blockIdx.y;
+  if (threadIdx.x == 0) a_s[0] = mr_alpha<R>(pr0, pp0, q);
+  if (threadIdx.x == 32) a_s[1] = mr_alpha<R>(pr1, pp1, q);
+  __syncthreads();
+  const long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (e >= nv) return;
+  const long long o = (long long)q * nv + e;
+  const V rv = reinterpret_cast<V*>(r1)[o];
+  V xv = X_ZERO ? vzero<V>() : reinterpret_cast<V*>(x)[o];
+  vmac(xv, a_s[0], reinterpret_cast<const V*>(r0)[o]);
+  vmac(xv, a_s[1], rv);
+  reinterpret_cast<V*>(x)[o] = xv;
+  if (R_NEXT) reinterpret_cast<V*>(r1)[o] = vsub(rv, a_s[1], reinterpret_cast<const V*>(p1)[o]);
+}
+
+template <typename R>
+static long long mr_vectors(long long n) {
+  if (n % MrVec<R>::n) throw Error(-1, "MR update: odd field length");
+  return n / MrVec<R>::n;
 }
 template <typename R>
 void launch_mr_update(cplx<R>* x, cplx<R>* r, const cplx<R>* p, const double2* pr, const double* pp, long long n,
-                      int nrhs, cudaStream_t st, bool x_zero, bool r_next, const cplx<R>* rin) {
-  const dim3 grid(nblk(n, 256), nrhs);
-  if (!rin) rin = r;
-  if (x_zero && r_next) k_mr_update<R, true, true><<<grid, 256, 0, st>>>(x, r, rin, p, pr, pp, n);
-  else if (x_zero) k_mr_update<R, true, false><<<grid, 256, 0, st>>>(x, r, rin, p, pr, pp, n);
-  else if (r_next) k_mr_update<R, false, true><<<grid, 256, 0, st>>>(x, r, rin, p, pr, pp, n);
-  else k_mr_update<R, false, false><<<grid, 256, 0, st>>>(x, r, rin, p, pr, pp, n);
+                      int nrhs, cudaStream_t st, bool x_zero, bool r_next) {
+  const long long nv = mr_vectors<R>(n);
+  const dim3 grid(nblk(nv, 256), nrhs);
+  if (x_zero && r_next) k_mr_update<R, true, true><<<grid, 256, 0, st>>>(x, r, p, pr, pp, nv);
+  else if (x_zero) k_mr_update<R, true, false><<<grid, 256, 0, st>>>(x, r, p, pr, pp, nv);
+  else if (r_next) k_mr_update<R, false, true><<<grid, 256, 0, st>>>(x, r, p, pr, pp, nv);
+  else k_mr_update<R, false, false><<<grid, 256, 0, st>>>(x, r, p, pr, pp, nv);
+  WCMG_LAUNCH_CHECK();
+}
+template <typename R>
+void launch_mr_residual(cplx<R>* p, const cplx<R>* r, const double2* pr, const double* pp, long long n, int nrhs,
+                        cudaStream_t st) {
+  const long long nv = mr_vectors<R>(n);
+  k_mr_residual<R><<<dim3(nblk(nv, 256), nrhs), 256, 0, st>>>(p, r, pr, pp, nv);
+  WCMG_LAUNCH_CHECK();
+}
+template <typename R>
+void launch_mr_pair(cplx<R>* x, const cplx<R>* r0, cplx<R>* r1, const cplx<R>* p1, const double2* pr0,
+                    const double* pp0, const double2* pr1, const double* pp1, long long n, int nrhs, cudaStream_t st,
+                    bool x_zero, bool r_next) {
+  const long long nv = mr_vectors<R>(n);
+  const dim3 grid(nblk(nv, 256), nrhs);
+#define WCMG_MP(XZ, RN) k_mr_pair<R, XZ, RN><<<grid, 256, 0, st>>>(x, r0, r1, p1, pr0, pp0, pr1, pp1, nv)
+  if (x_zero && r_next) WCMG_MP(true, true);
+  else if (x_zero) WCMG_MP(true, false);
+  else if (r_next) WCMG_MP(false, true);
+  else WCMG_MP(false, false);
+#undef WCMG_MP
+  WCMG_LAUNCH_CHECK();
+}
+
+__global__ void k_add_widened(double2* __restrict__ y, const float2* __restrict__ x, long long n) {
+  const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (i < n) y[i] += to_c64(x[i]);
+}
+void launch_add_widened(double2* y, const float2* x, long long n, cudaStream_t st) {
+  k_add_widened<<<nblk(n, 256), 256, 0, st>>>(y, x, n);
   WCMG_LAUNCH_CHECK();
 }
 
@@ -673,7 +771,12 @@ void launch_counter_gaussian(double2* out, long long n, int nfields, unsigned lo
   template void launch_scale_dev<R>(cplx<R>*, const cplx<R>*, const double*, int, long long, int, cudaStream_t,  \
                                     const int*, int, long long);                                                 \
   template void launch_mr_update<R>(cplx<R>*, cplx<R>*, const cplx<R>*, const double2*, const double*, long long, \
-                                    int, cudaStream_t, bool, bool, const cplx<R>*);                              \
+                                    int, cudaStream_t, bool, bool);                                              \
+  template void launch_mr_residual<R>(cplx<R>*, const cplx<R>*, const double2*, const double*, long long, int,   \
+                                      cudaStream_t);                                                             \
+  template void launch_mr_pair<R>(cplx<R>*, const cplx<R>*, cplx<R>*, const cplx<R>*, const double2*,            \
+                                  const double*, const double2*, const double*, long long, int, cudaStream_t,    \
+                                  bool, bool);                                                                   \
   template void launch_mask_rhs<R>(cplx<R>*, const int*, long long, int, cudaStream_t);                          \
   template void launch_fill_zero<R>(cplx<R>*, long long, cudaStream_t);
 WCMG_INST(double)

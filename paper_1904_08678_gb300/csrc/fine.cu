@@ -468,16 +468,19 @@ __device__ __forceinline__ bool on_face(const BlockInfo& bi, int s, int d) {
   return (d & 1) ? (l[mu] == 0) : (l[mu] == bi.b[mu] - 1);
 }
 
+// RSD: the result is the residual rsd - D in, formed in the epilogue (a pass of its own
+// would read the product and write it once more).
 // MR epilogue (DOTS): the CTA also sums <out, in> = sum conj(out) in and <out, out>
 // over its sites (FP32/FP64 per thread, FP64 across the CTA) into one partial per
 // (rhs, CTA): the minimal-residual step p = D r, alpha = <p, r>/<p, p> then needs
-// no extra pass over p and r.
-template <typename R, int MODE, bool DOTS, int NR>
+// no extra pass over p and r.  A null `out` keeps the sums only (the last step of a
+// fixed-step MR, whose new residual nobody reads).
+template <typename R, int MODE, bool DOTS, int NR, bool RSD = false>
 __global__ void __launch_bounds__(128, (sizeof(R) == 4 && NR == 1) ? 6 : (sizeof(R) == 4 ? 4 : 1))
     k_dslash(cplx<R>* __restrict__ out, const cplx<R>* __restrict__ in, const cplx<R>* __restrict__ U,
              const cplx<R>* __restrict__ clov, const int* __restrict__ nbr, int V, BlockInfo bi, int hopdir, int nrhs,
              double2* __restrict__ pr_part, double* __restrict__ pp_part,
-             const unsigned char* __restrict__ colour, int col) {
+             const unsigned char* __restrict__ colour, int col, const cplx<R>* __restrict__ rsd) {
   using T = cplx<R>;
   // rhs groups fastest in the grid: the CTAs running together cover the same sites
   // for every rhs, so links and clover are fetched from HBM once
@@ -548,10 +551,14 @@ __global__ void __launch_bounds__(128, (sizeof(R) == 4 && NR == 1) ? 6 : (sizeof
       }
 #pragma unroll
       for (int q = 0; q < NR; ++q)
-        if (q < nq) {
+        if (q < nq && !(DOTS && !out)) {
           cplx<R>* oq = out + off + q * rstride;
+          const cplx<R>* bq = RSD ? rsd + off + q * rstride : nullptr;
 #pragma unroll
-          for (int i = 0; i < 6; ++i) oq[(long long)(6 * h + i) * V + s] = acc[q][6 * h + i];
+          for (int i = 0; i < 6; ++i) {
+            const long long a = (long long)(6 * h + i) * V + s;
+            oq[a] = RSD ? bq[a] - acc[q][6 * h + i] : acc[q][6 * h + i];
+          }
         }
     }
   }
@@ -581,7 +588,9 @@ static int dslash_nr(int nrhs) { return (sizeof(R) == 4 && nrhs > 1) ? 2 : 1; }
 
 template <typename R>
 void launch_dslash(cplx<R>* out, const cplx<R>* in, const cplx<R>* gauge, const cplx<R>* clov, const LevelGeom& g,
-                   int nrhs, int mode, int hopdir, cudaStream_t st, const unsigned char* colour, int col) {
+                   int nrhs, int mode, int hopdir, cudaStream_t st, const unsigned char* colour, int col,
+                   const cplx<R>* rsd) {
+  if (rsd && mode != ST_FULL) throw Error(-1, "residual epilogue: full stencil only");
   BlockInfo bi;
   for (int k = 0; k < 4; ++k) bi.b[k] = g.b[k];
   bi.bvol = g.bvol;
@@ -589,10 +598,14 @@ void launch_dslash(cplx<R>* out, const cplx<R>* in, const cplx<R>* gauge, const 
   const dim3 grid((unsigned)(nblk(g.V, 128) * (long long)((nrhs + nr - 1) / nr)));
 #define WCMG_DS(MODE, NR) \
   k_dslash<R, MODE, false, NR><<<grid, 128, 0, st>>>(out, in, gauge, clov, g.nbr, g.V, bi, hopdir, nrhs, nullptr, \
-                                                     nullptr, colour, col)
+                                                     nullptr, colour, col, nullptr)
+#define WCMG_DS_RSD(NR)                                                                                             \
+  k_dslash<R, ST_FULL, false, NR, true><<<grid, 128, 0, st>>>(out, in, gauge, clov, g.nbr, g.V, bi, hopdir, nrhs,   \
+                                                              nullptr, nullptr, colour, col, rsd)
   if constexpr (sizeof(R) == 4) {
     if (nr == 2) {
-      if (mode == ST_FULL) WCMG_DS(ST_FULL, 2);
+      if (rsd) WCMG_DS_RSD(2);
+      else if (mode == ST_FULL) WCMG_DS(ST_FULL, 2);
       else if (mode == ST_BLOCK_INTERIOR) WCMG_DS(ST_BLOCK_INTERIOR, 2);
       else WCMG_DS(ST_FACE_HOP, 2);
       WCMG_LAUNCH_CHECK();
@@ -600,10 +613,12 @@ void launch_dslash(cplx<R>* out, const cplx<R>* in, const cplx<R>* gauge, const 
     }
   }
   {
-    if (mode == ST_FULL) WCMG_DS(ST_FULL, 1);
+    if (rsd) WCMG_DS_RSD(1);
+    else if (mode == ST_FULL) WCMG_DS(ST_FULL, 1);
     else if (mode == ST_BLOCK_INTERIOR) WCMG_DS(ST_BLOCK_INTERIOR, 1);
     else WCMG_DS(ST_FACE_HOP, 1);
   }
+#undef WCMG_DS_RSD
 #undef WCMG_DS
   WCMG_LAUNCH_CHECK();
 }
@@ -1206,13 +1221,13 @@ void launch_dslash_mr(cplx<R>* out, const cplx<R>* in, const cplx<R>* gauge, con
   if constexpr (sizeof(R) == 4) {
     if (nr == 2) {
       k_dslash<R, ST_FULL, true, 2><<<grid, 128, 0, st>>>(out, in, gauge, clov, g.nbr, g.V, bi, 0, nrhs, pr_part,
-                                                           pp_part, nullptr, 0);
+                                                           pp_part, nullptr, 0, nullptr);
       done = true;
     }
   }
   if (!done)
     k_dslash<R, ST_FULL, true, 1><<<grid, 128, 0, st>>>(out, in, gauge, clov, g.nbr, g.V, bi, 0, nrhs, pr_part,
-                                                         pp_part, nullptr, 0);
+                                                         pp_part, nullptr, 0, nullptr);
   WCMG_LAUNCH_CHECK();
   k_mr_final<<<nrhs, 256, 0, st>>>(pr, pp, pr_part, pp_part, nsb);
   WCMG_LAUNCH_CHECK();
@@ -1223,7 +1238,7 @@ void launch_dslash_mr(cplx<R>* out, const cplx<R>* in, const cplx<R>* gauge, con
   template void launch_unpack_fine<R>(double2*, const cplx<R>*, const int*, int, int, cudaStream_t);          \
   template void launch_pack_gauge<R>(cplx<R>*, const double2*, const int*, int, cudaStream_t);                \
   template void launch_dslash<R>(cplx<R>*, const cplx<R>*, const cplx<R>*, const cplx<R>*, const LevelGeom&, \
-                                 int, int, int, cudaStream_t, const unsigned char*, int);                    \
+                                 int, int, int, cudaStream_t, const unsigned char*, int, const cplx<R>*);    \
   template void launch_sap_fine<R>(cplx<R>*, const cplx<R>*, const cplx<R>*, const cplx<R>*, const cplx<R>*,  \
                                    const LevelGeom&, const int*, int, int, int, cudaStream_t);                \
   template void launch_sap_fine_eo<R>(cplx<R>*, const cplx<R>*, const cplx<R>*, const cplx<R>*,              \

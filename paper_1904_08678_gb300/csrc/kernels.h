@@ -42,7 +42,7 @@ void launch_clover_pack(double2* clov, const double2* ext, const int* perm, int 
 template <typename R>
 void launch_dslash(cplx<R>* out, const cplx<R>* in, const cplx<R>* gauge, const cplx<R>* clov, const LevelGeom& g,
                    int nrhs, int mode, int hopdir, cudaStream_t st, const unsigned char* colour = nullptr,
-                   int col = 0);
+                   int col = 0, const cplx<R>* rsd = nullptr);
 // One SAP colour pass on the fine level, fused: for each aggregate B in blocks[0 ..
 // nblocks) and every rhs, r = b - Dx on B (Dx null: b), `steps` MR steps of the
 // block-local D_B from e = 0 with alpha_B = <p, r>_B / <p, p>_B, then x += e on B.
@@ -63,7 +63,8 @@ void launch_sap_fine_eo(cplx<R>* x, const cplx<R>* b, const cplx<R>* Dx, const c
                         int nblocks, int steps, int nrhs, cudaStream_t st);
 // out = D in (full stencil) and, per rhs r, pr[r] = <out_r, in_r> = sum conj(out) in,
 // pp[r] = <out_r, out_r> (the minimal-residual step's two reductions, fused into the
-// stencil).  pr_part / pp_part: scratch of nrhs * dslash_partials(V) entries.
+// stencil); out may be null: the sums only.  pr_part / pp_part: scratch of nrhs *
+// dslash_partials(V) entries.
 int dslash_partials(int V);
 // Masked stencil (ST_BLOCK_INTERIOR or ST_FACE_HOP) of both chirality projections of
 // nv vectors: out[i] = D_mode(Pi_+ v_i), out[nv + i] = D_mode(Pi_- v_i) (CoarsenOperator).
@@ -200,6 +201,8 @@ template <typename R>
 void launch_copy_idx(cplx<R>* dst, const cplx<R>* src, long long n, const int* idx, long long dmul, long long smul,
                      cudaStream_t st);
 void launch_fill_int(int* x, int v, int n, cudaStream_t st);
+// y += x widened to FP64
+void launch_add_widened(double2* y, const float2* x, long long n, cudaStream_t st);
 template <typename R>
 void launch_axpby(cplx<R>* y, double a, const cplx<R>* x, double b, long long n, int nrhs, cudaStream_t st);
 // y[r] = x[r] * s[r] (s real, device; 1/sqrt(s) with inv_sqrt).  ydev (nullable):
@@ -207,15 +210,21 @@ void launch_axpby(cplx<R>* y, double a, const cplx<R>* x, double b, long long n,
 template <typename R>
 void launch_scale_dev(cplx<R>* y, const cplx<R>* x, const double* s, int inv_sqrt, long long n, int nrhs,
                       cudaStream_t st, const int* ydev = nullptr, int yadd = 0, long long ystride = 0);
-// MR update with alpha[r] = pr[r] / pp[r] (0 if pp = 0), pr = <p, r>, pp = <p, p>:
-//   x += alpha r ; r -= alpha p
-// x_zero: x is taken as 0 and not read; r_next = false: r is not written (the last step
-// of a fixed-step MR, whose residual nobody reads); rin (nullable): read the residual
-// from rin instead of r (the first step reads b) and write the new one to r.
+// MR updates with alpha = pr[q] / pp[q] (0 if pp = 0), pr = <p, r>, pp = <p, p> of rhs q;
+// x_zero: x is taken as 0 and not read.
+// One step: x += alpha r; r_next: r -= alpha p in place.
 template <typename R>
 void launch_mr_update(cplx<R>* x, cplx<R>* r, const cplx<R>* p, const double2* pr, const double* pp, long long n,
-                      int nrhs, cudaStream_t st, bool x_zero = false, bool r_next = true,
-                      const cplx<R>* rin = nullptr);
+                      int nrhs, cudaStream_t st, bool x_zero, bool r_next);
+// First half of a pair of steps: p <- r - alpha p (the next residual takes p's place, r is kept).
+template <typename R>
+void launch_mr_residual(cplx<R>* p, const cplx<R>* r, const double2* pr, const double* pp, long long n, int nrhs,
+                        cudaStream_t st);
+// Second half: x += alpha0 r0 + alpha1 r1; r_next: r1 -= alpha1 p1 in place.
+template <typename R>
+void launch_mr_pair(cplx<R>* x, const cplx<R>* r0, cplx<R>* r1, const cplx<R>* p1, const double2* pr0,
+                    const double* pp0, const double2* pr1, const double* pp1, long long n, int nrhs, cudaStream_t st,
+                    bool x_zero, bool r_next);
 // x[r] = mask[r] ? 0 : x[r]
 template <typename R>
 void launch_mask_rhs(cplx<R>* x, const int* mask, long long n, int nrhs, cudaStream_t st);

@@ -91,7 +91,7 @@ static inline void coords(int s, const int* d, int* x) {
 // Scalars of one level's Krylov loops (device) and its (F)GMRES state.
 struct LevelScalars {
   int cap_rhs = 0, cap_m = 0;
-  DevBuf<double2> c2;  // h1, h2 [2][rhs][m+1]; pr [rhs]
+  DevBuf<double2> c2;  // h1, h2 [2][rhs][m+1]; pr [2][rhs] (steps of a pair)
   DevBuf<double> d;    // hn2, nrm2, inv_beta, inv_h, pp, bnorm, resid, cs... [slots][rhs]
   DevBuf<double2> H, sn, g, y;
   DevBuf<double> cs;
@@ -100,8 +100,8 @@ struct LevelScalars {
     if (rhs <= cap_rhs && m <= cap_m) return;
     rhs = std::max(rhs, cap_rhs);
     m = std::max(m, cap_m);
-    c2.ensure((size_t)rhs * (2 * (m + 1) + 1));
-    d.ensure((size_t)rhs * 8);
+    c2.ensure((size_t)rhs * (2 * (m + 1) + 2));
+    d.ensure((size_t)rhs * 9);
     H.ensure((size_t)rhs * (m + 1) * m);
     sn.ensure((size_t)rhs * m);
     g.ensure((size_t)rhs * (m + 1));
@@ -117,7 +117,8 @@ struct LevelScalars {
   }
   double2* h1() { need(); return c2.p; }
   double2* h2() { need(); return c2.p + (size_t)cap_rhs * (cap_m + 1); }
-  double2* pr() { need(); return c2.p + (size_t)2 * cap_rhs * (cap_m + 1); }
+  double2* pr(int k = 0) { need(); return c2.p + (size_t)2 * cap_rhs * (cap_m + 1) + (size_t)(k & 1) * cap_rhs; }
+  double* pp(int k = 0) { return slot(k & 1 ? 8 : 4); }
   double* slot(int k) { need(); return d.p + (size_t)k * cap_rhs; }
   GmresState state(int m) {
     need();
@@ -130,7 +131,7 @@ struct LevelScalars {
     return s;
   }
 };
-// slot map: 0 hn2, 1 nrm2, 2 inv_beta, 3 inv_h, 4 pp, 5 bnorm, 6 resid, 7 misc
+// slot map: 0 hn2, 1 nrm2, 2 inv_beta, 3 inv_h, 4 pp, 5 bnorm, 6 resid, 7 misc, 8 pp of odd MR steps
 
 struct Level {
   HostGeom g;
@@ -727,25 +728,44 @@ static void dot_op(wcmg_ctx* c, double2* out, const cplx<R>* a, const cplx<R>* b
         launch_dot<R>(out, a, b, n, nrhs, c->partial.p, c->st));
 }
 
-// ---------------- MR (smoother) ----------------
-// Sec. 2.1 MinimalResidual, zero initial guess, fixed number of steps:
-//   r = b; k times: p = A r, alpha = <p, r>/<p, p>, x += alpha r, r -= alpha p.
+// out = b - D_level x
 template <typename R>
-static void mr(wcmg_ctx* c, int l, cplx<R>* x, const cplx<R>* b, int nrhs, int steps) {
+static void residual_op(wcmg_ctx* c, int l, cplx<R>* out, const cplx<R>* b, const cplx<R>* x, int nrhs) {
   Level& L = c->L[l];
-  const long long n = L.n();
-  cplx<R>* r = ws<R>(L, "mr_r", nrhs);
-  cplx<R>* p = ws<R>(L, "mr_p", nrhs);
-  L.sc.ensure(max_rhs_all(c), std::max(c->p.outer_restart, c->p.coarse_restart));
-  if (steps == 0) {
-    launch_fill_zero<R>(x, n * nrhs, c->st);
+  if (l != 0) {
+    apply_op<R>(c, l, out, x, nrhs);
+    launch_axpby<R>(out, 1.0, b, -1.0, L.n(), nrhs, c->st);
     return;
   }
-  // the first step reads b as its residual and sets x = alpha r; the last one leaves r
-  for (int k = 0; k < steps; ++k) {
-    const cplx<R>* rk = k == 0 ? b : r;
+  if (!c->have_gauge) throw Error(WCMG_ERR_STATE, "gauge field not set");
+  if (!c->capturing) c->opc[WCMG_OPC_APPLY][0] += nrhs;
+  const double V = L.g.V, s = sizeof(cplx<R>);
+  KPROF(c, sizeof(R) == 8 ? WCMG_K_DSLASH64 : WCMG_K_DSLASH, V * s * (36.0 * nrhs + 72.0), V * (1872.0 + 24.0) * nrhs,
+        launch_dslash<R>(out, x, Prec<R>::gauge(c), Prec<R>::clover(c), L.g.lg(), nrhs, ST_FULL, 0, c->st, nullptr, 0,
+                         b));
+}
+
+// ---------------- MR (smoother) ----------------
+// Sec. 2.1 MinimalResidual, zero initial guess, fixed number of steps:
+//   r = b; k times: p = A r, alpha = <p, r>/<p, p>, x += alpha r, r -= alpha p;
+// add: the result is added to x instead of replacing it.  Steps 0 and 1 and, on the fine
+// level, the last two (whose second p is never formed: only its sums are) share one
+// update of x (see the update kernels).
+template <typename R>
+static void mr(wcmg_ctx* c, int l, cplx<R>* x, const cplx<R>* b, int nrhs, int steps, bool add = false) {
+  Level& L = c->L[l];
+  const long long n = L.n();
+  cplx<R>* A = ws<R>(L, "mr_r", nrhs);
+  cplx<R>* B = ws<R>(L, "mr_p", nrhs);
+  L.sc.ensure(max_rhs_all(c), std::max(c->p.outer_restart, c->p.coarse_restart));
+  if (steps == 0) {
+    if (!add) launch_fill_zero<R>(x, n * nrhs, c->st);
+    return;
+  }
+  // p = A r and the sums of step k; on the fine level the sums come out of the stencil's
+  // epilogue and p may be null
+  auto stencil = [&](int k, cplx<R>* p, const cplx<R>* r) {
     if (l == 0) {
-      // fine level: the two reductions come out of the Dslash epilogue
       if (!c->have_gauge) throw Error(WCMG_ERR_STATE, "gauge field not set");
       const long long np = (long long)max_rhs_all(c) * dslash_partials(L.g.V);
       c->mr_pr.ensure(np);
@@ -753,18 +773,44 @@ static void mr(wcmg_ctx* c, int l, cplx<R>* x, const cplx<R>* b, int nrhs, int s
       const double V = L.g.V, s = sizeof(cplx<R>);
       const int cls = sizeof(R) == 8 ? WCMG_K_DSLASH64 : WCMG_K_DSLASH;
       if (!c->capturing) c->opc[WCMG_OPC_APPLY][0] += nrhs;
-      KPROF(c, cls, V * s * (24.0 * nrhs + 72.0), V * (1872.0 + 16.0) * nrhs,
-            launch_dslash_mr<R>(p, rk, Prec<R>::gauge(c), Prec<R>::clover(c), L.g.lg(), nrhs, L.sc.pr(),
-                                L.sc.slot(4), c->mr_pr.p, c->mr_pp.p, c->st));
+      KPROF(c, cls, V * s * ((p ? 24.0 : 12.0) * nrhs + 72.0), V * (1872.0 + 16.0) * nrhs,
+            launch_dslash_mr<R>(p, r, Prec<R>::gauge(c), Prec<R>::clover(c), L.g.lg(), nrhs, L.sc.pr(k), L.sc.pp(k),
+                                c->mr_pr.p, c->mr_pp.p, c->st));
     } else {
-      apply_op<R>(c, l, p, rk, nrhs);
-      dot_op<R>(c, L.sc.pr(), p, rk, n, nrhs);
-      norm2_op<R>(c, L.sc.slot(4), p, n, nrhs);
+      apply_op<R>(c, l, p, r, nrhs);
+      dot_op<R>(c, L.sc.pr(k), p, r, n, nrhs);
+      norm2_op<R>(c, L.sc.pp(k), p, n, nrhs);
     }
-    const bool first = k == 0, last = k + 1 == steps;
-    KPROF(c, WCMG_K_BLAS, ((first ? 2.0 : 3.0) + (last ? 0.0 : 2.0)) * n * nrhs * sizeof(cplx<R>),
-          16.0 * n * nrhs,
-          launch_mr_update<R>(x, r, p, L.sc.pr(), L.sc.slot(4), n, nrhs, c->st, first, !last, rk));
+  };
+  const double fb = (double)n * nrhs * sizeof(cplx<R>), fl = 8.0 * n * nrhs;
+  bool x_zero = !add;
+  const cplx<R>* r = b;  // r_k: b itself, then A
+  for (int k = 0; k < steps;) {
+    const bool last = k + 1 == steps;
+    if (!last && (k == 0 || (l == 0 && k + 2 == steps))) {
+      cplx<R>* p = k == 0 ? A : B;
+      stencil(k, p, r);
+      KPROF(c, WCMG_K_BLAS, 3.0 * fb, fl, launch_mr_residual<R>(p, r, L.sc.pr(k), L.sc.pp(k), n, nrhs, c->st));
+      const bool fin = k + 2 == steps;
+      cplx<R>* q = fin && l == 0 ? nullptr : B;  // k == 0 whenever q is needed
+      stencil(k + 1, q, p);
+      KPROF(c, WCMG_K_BLAS, ((x_zero ? 3.0 : 4.0) + (fin ? 0.0 : 2.0)) * fb, (fin ? 2.0 : 3.0) * fl,
+            launch_mr_pair<R>(x, r, p, q, L.sc.pr(k), L.sc.pp(k), L.sc.pr(k + 1), L.sc.pp(k + 1), n, nrhs, c->st,
+                              x_zero, !fin));
+      r = p;
+      k += 2;
+    } else if (k == 0) {  // a single step: its p is not needed on the fine level
+      stencil(0, l == 0 ? nullptr : B, r);
+      KPROF(c, WCMG_K_BLAS, (x_zero ? 2.0 : 3.0) * fb, fl,
+            launch_mr_update<R>(x, const_cast<cplx<R>*>(r), B, L.sc.pr(0), L.sc.pp(0), n, nrhs, c->st, x_zero, false));
+      k += 1;
+    } else {
+      stencil(k, last && l == 0 ? nullptr : B, r);
+      KPROF(c, WCMG_K_BLAS, (last ? 3.0 : 5.0) * fb, (last ? 1.0 : 2.0) * fl,
+            launch_mr_update<R>(x, A, B, L.sc.pr(k), L.sc.pp(k), n, nrhs, c->st, x_zero, !last));
+      k += 1;
+    }
+    x_zero = false;
   }
 }
 
@@ -806,8 +852,7 @@ static KrylovOut fgmres(wcmg_ctx* c, int l, cplx<R>* x, const cplx<R>* b, int nr
     launch_fill_zero<R>(x, n * nrhs, c->st);
     copy_fields<R>(c, r, b, n * nrhs);
   } else {
-    apply_op<R>(c, l, r, x, nrhs);
-    launch_axpby<R>(r, 1.0, b, -1.0, n, nrhs, c->st);  // r = b - A x
+    residual_op<R>(c, l, r, b, x, nrhs);
   }
   KrylovOut out;
   int cycles = 0;
@@ -884,8 +929,7 @@ static KrylovOut fgmres(wcmg_ctx* c, int l, cplx<R>* x, const cplx<R>* b, int nr
     bool all = true;
     for (int q = 0; q < nrhs; ++q) all &= dn[q] != 0;
     if (all && !verify) { out.converged = true; return out; }
-    apply_op<R>(c, l, r, x, nrhs);
-    launch_axpby<R>(r, 1.0, b, -1.0, n, nrhs, c->st);
+    residual_op<R>(c, l, r, b, x, nrhs);
     norm2_op<R>(c, SC.slot(1), r, n, nrhs);
     launch_gmres_mark_done(S, SC.slot(1), tol, nrhs, c->st);
     const double* nr = read_doubles(c, SC.slot(1), nrhs);
@@ -995,8 +1039,7 @@ static void fgmres_g(wcmg_ctx* c, int l, cplx<R>* x, const cplx<R>* b, int nrhs,
     launch_fill_zero<R>(x, n * nrhs, c->st);
     copy_fields<R>(c, r, b, n * nrhs);
   } else {
-    apply_op<R>(c, l, r, x, nrhs);
-    launch_axpby<R>(r, 1.0, b, -1.0, n, nrhs, c->st);  // r = b - A x
+    residual_op<R>(c, l, r, b, x, nrhs);
   }
   norm2_op<R>(c, SC.slot(1), r, n, nrhs);
   const bool single = max_cycles == 1;
@@ -1053,8 +1096,7 @@ static void fgmres_g(wcmg_ctx* c, int l, cplx<R>* x, const cplx<R>* b, int nrhs,
     int slot_if = -1;
     cond_node(c, h_if, cudaGraphCondTypeIf, [&](int slot_i) {
       slot_if = slot_i;
-      apply_op<R>(c, l, r, x, nrhs);
-      launch_axpby<R>(r, 1.0, b, -1.0, n, nrhs, c->st);
+      residual_op<R>(c, l, r, b, x, nrhs);
       norm2_op<R>(c, SC.slot(1), r, n, nrhs);
       launch_gmres_mark_done(S, SC.slot(1), tol, nrhs, c->st);
     });
@@ -1283,9 +1325,12 @@ static void cycle(wcmg_ctx* c, int l, cplx<R>* e, const cplx<R>* r, int nrhs) {
     prolong_op<R>(c, l, e, ec, nrhs);
   }
   cplx<R>* t = ws<R>(L, "cyc_t", nrhs);
+  residual_op<R>(c, l, t, r, e, nrhs);  // t = r - D e
+  if (c->p.smoother == WCMG_SMOOTHER_MR || c->p.smoother_steps == 0) {
+    mr<R>(c, l, e, t, nrhs, c->p.smoother_steps, true);
+    return;
+  }
   cplx<R>* s = ws<R>(L, "cyc_s", nrhs);
-  apply_op<R>(c, l, t, e, nrhs);
-  launch_axpby<R>(t, 1.0, r, -1.0, n, nrhs, c->st);  // t = r - D e
   smooth<R>(c, l, s, t, nrhs);
   launch_axpby<R>(e, 1.0, s, 1.0, n, nrhs, c->st);
 }
@@ -1513,12 +1558,10 @@ static void solve_f64(wcmg_ctx* c, double2* x, const double2* b, int nrhs, wcmg_
 constexpr double kInnerTol = 1e-5;
 
 // r = b - D x for the caller's initial guess (c->guess), else x = 0 and r = b (FP64).
-static void start_residual(wcmg_ctx* c, double2* x, double2* r, double2* t, const double2* b, int nrhs) {
+static void start_residual(wcmg_ctx* c, double2* x, double2* r, const double2* b, int nrhs) {
   const long long n = c->L[0].n();
   if (c->guess) {
-    apply_op<double>(c, 0, t, x, nrhs);
-    copy_fields<double>(c, r, b, n * nrhs);
-    launch_axpby<double>(r, -1.0, t, 1.0, n, nrhs, c->st);
+    residual_op<double>(c, 0, r, b, x, nrhs);
   } else {
     launch_fill_zero<double>(x, n * nrhs, c->st);
     copy_fields<double>(c, r, b, n * nrhs);
@@ -1531,7 +1574,6 @@ static void solve_mixed(wcmg_ctx* c, double2* x, const double2* b, int nrhs, wcm
   Level& L = c->L[0];
   const long long n = L.n();
   double2* r64 = ws<double>(L, "mx_r", nrhs);
-  double2* t64 = ws<double>(L, "mx_t", nrhs);
   float2* r32 = ws<float>(L, "mx_r32", nrhs);
   float2* e32 = ws<float>(L, "mx_e32", nrhs);
   L.sc.ensure(max_rhs_all(c), std::max(c->p.outer_restart, c->p.coarse_restart));
@@ -1542,7 +1584,7 @@ static void solve_mixed(wcmg_ctx* c, double2* x, const double2* b, int nrhs, wcm
     const double* h = read_doubles(c, bn2, nrhs);
     for (int q = 0; q < nrhs; ++q) bnorm[q] = std::sqrt(h[q]);
   }
-  start_residual(c, x, r64, t64, b, nrhs);
+  start_residual(c, x, r64, b, nrhs);
   DevBuf<int>& mask = c->errflag;  // errflag has room for max rhs + 1
   std::vector<int> done(nrhs, 0);
   int its = 0, restarts = 0;
@@ -1570,11 +1612,8 @@ static void solve_mixed(wcmg_ctx* c, double2* x, const double2* b, int nrhs, wcm
     its += k.iterations;
     ++restarts;
     if (k.iterations == 0) { st->converged = 0; break; }  // FP32 cycle could not move (no progress)
-    launch_convert<float, double>(t64, e32, n * nrhs, c->st);
-    launch_axpby<double>(x, 1.0, t64, 1.0, n, nrhs, c->st);
-    apply_op<double>(c, 0, t64, x, nrhs);
-    copy_fields<double>(c, r64, b, n * nrhs);
-    launch_axpby<double>(r64, -1.0, t64, 1.0, n, nrhs, c->st);
+    launch_add_widened(x, e32, n * nrhs, c->st);
+    residual_op<double>(c, 0, r64, b, x, nrhs);
   }
   st->outer_iterations = its;
   st->restarts = restarts - 1 > 0 ? restarts - 1 : 0;
@@ -1589,7 +1628,6 @@ static void solve_mixed_body(wcmg_ctx* c, double2* x, const double2* b, int nrhs
   Level& L = c->L[0];
   const long long n = L.n();
   double2* r64 = ws<double>(L, "mx_r", nrhs);
-  double2* t64 = ws<double>(L, "mx_t", nrhs);
   float2* r32 = ws<float>(L, "mx_r32", nrhs);
   float2* e32 = ws<float>(L, "mx_e32", nrhs);
   L.sc.ensure(max_rhs_all(c), std::max(c->p.outer_restart, c->p.coarse_restart));
@@ -1597,7 +1635,7 @@ static void solve_mixed_body(wcmg_ctx* c, double2* x, const double2* b, int nrhs
   KCtl* Kmx = c->kctl.p;
   KCtl* Kfg = c->kctl.p + 1;
   norm2_op<double>(c, bn2, b, n, nrhs);
-  start_residual(c, x, r64, t64, b, nrhs);
+  start_residual(c, x, r64, b, nrhs);
   norm2_op<double>(c, L.sc.slot(1), r64, n, nrhs);
   const cudaGraphConditionalHandle h = cond_handle(c);
   launch_kctl_init(Kmx, c->p.outer_maxiter, nullptr, 0, h, 0, c->st);
@@ -1608,11 +1646,8 @@ static void solve_mixed_body(wcmg_ctx* c, double2* x, const double2* b, int nrhs
     launch_mask_rhs<float>(r32, c->mx_done.p, n, nrhs, c->st);
     fgmres_g<float>(c, 0, e32, r32, nrhs, c->p.outer_restart, kInnerTol, c->p.outer_restart, true, false, true, 1,
                     Kfg, &Kmx->its, c->p.outer_maxiter, nullptr);
-    launch_convert<float, double>(t64, e32, n * nrhs, c->st);
-    launch_axpby<double>(x, 1.0, t64, 1.0, n, nrhs, c->st);
-    apply_op<double>(c, 0, t64, x, nrhs);
-    copy_fields<double>(c, r64, b, n * nrhs);
-    launch_axpby<double>(r64, -1.0, t64, 1.0, n, nrhs, c->st);
+    launch_add_widened(x, e32, n * nrhs, c->st);
+    residual_op<double>(c, 0, r64, b, x, nrhs);
     norm2_op<double>(c, L.sc.slot(1), r64, n, nrhs);
     launch_mx_check(Kmx, Kfg, L.sc.slot(1), bn2, c->p.outer_tol, c->mx_done.p, c->mx_worst.p, nrhs,
                     body_count(c, slot), h, c->st);
@@ -1777,8 +1812,7 @@ static double true_residual(wcmg_ctx* c, const double2* x, const double2* b, int
   Level& L = c->L[0];
   const long long n = L.n();
   double2* t = ws<double>(L, "tr_t", nrhs);
-  apply_op<double>(c, 0, t, x, nrhs);
-  launch_axpby<double>(t, 1.0, b, -1.0, n, nrhs, c->st);
+  residual_op<double>(c, 0, t, b, x, nrhs);
   L.sc.ensure(max_rhs_all(c), std::max(c->p.outer_restart, c->p.coarse_restart));
   norm2_op<double>(c, L.sc.slot(1), t, n, nrhs);
   norm2_op<double>(c, L.sc.slot(7), b, n, nrhs);
