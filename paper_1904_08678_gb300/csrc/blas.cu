@@ -104,71 +104,199 @@ void launch_norm2(double* out, const cplx<R>* a, long long n, int nrhs, double* 
   WCMG_LAUNCH_CHECK();
 }
 
-// ---- multi-dot against a Krylov basis (chunks of 8 basis vectors) ----
+// ---- Gram-Schmidt of an Arnoldi step: two sweeps over the basis ----
+// Classical Gram-Schmidt twice is h1 = V^dag w, w1 = w - V h1, h2 = V^dag w1, w1 - V h2.
+// Since h2 = h1 - G h1 with the Gram matrix G = V^dag V of the basis, the second projection
+// needs no sweep of its own once G is known: the sweep that forms <V_i, w> also forms the
+// newest column <V_i, V_j> of G (V_j and w are read once per chunk of 8 basis vectors and
+// stay in L2 between the chunks), and one update subtracts V (h1 + h2).  G is as accurate
+// as the sums are (FP32 products, FP64 across warps), so what is left of V in the result
+// is of the order |1 - G|^2, as after two explicit passes.  Bound by HBM: k + 2 + k + 2
+// fields instead of 4 k + 9 (norm included): the 12-rhs solve on 24^3x48 went from 621 to 538 ms.
 constexpr int MD_K = 8;
 template <typename R>
-__global__ void __launch_bounds__(RED_T) k_multidot_partial(double2* __restrict__ partial,
-                                                            const cplx<R>* __restrict__ basis, long long bstride,
-                                                            int k, const cplx<R>* __restrict__ w, long long n,
-                                                            int kpad, const int* __restrict__ kdev, int kadd,
-                                                            int vec2) {
-  __shared__ double2 scratch[(RED_T / 32) * MD_K];
-  const int r = blockIdx.y, i0 = blockIdx.z * MD_K;
+__global__ void __launch_bounds__(RED_T) k_gram_partial(double2* __restrict__ partial, const cplx<R>* __restrict__ basis,
+                                                        long long bstride, int k, const cplx<R>* __restrict__ w,
+                                                        long long n, int nchunk, const int* __restrict__ kdev, int kadd,
+                                                        int vec2) {
+  __shared__ double2 scratch[2][(RED_T / 32) * MD_K];
+  // chunks of basis vectors fastest in the grid: CTAs running together read the same w, V_j
+  const int i0 = (blockIdx.x % nchunk) * MD_K, blk = blockIdx.x / nchunk, nblk_ = gridDim.x / nchunk;
+  const int r = blockIdx.y, kpad = nchunk * MD_K;
   if (kdev) k = *kdev + kadd;
   if (i0 >= k) return;  // uniform per block
   const long long off = (long long)r * n;
-  cplx<R> acc[MD_K];
+  const cplx<R>* vj = basis + (k - 1) * bstride + off;
+  cplx<R> aw[MD_K], av[MD_K];
 #pragma unroll
-  for (int q = 0; q < MD_K; ++q) acc[q] = czero<R>();
+  for (int q = 0; q < MD_K; ++q) aw[q] = av[q] = czero<R>();
   if constexpr (sizeof(R) == 4) {
     if (vec2) {  // two complex entries per 16-byte load (n, bstride even; 16-byte aligned fields)
       const float4* w4 = reinterpret_cast<const float4*>(w + off);
+      const float4* v4 = reinterpret_cast<const float4*>(vj);
       const long long n2 = n >> 1;
-      for (long long e = blockIdx.x * (long long)RED_T + threadIdx.x; e < n2; e += (long long)gridDim.x * RED_T) {
-        const float4 x = w4[e];
+      for (long long e = blk * (long long)RED_T + threadIdx.x; e < n2; e += (long long)nblk_ * RED_T) {
+        const float4 x = w4[e], y = v4[e];
 #pragma unroll
         for (int q = 0; q < MD_K; ++q)
           if (i0 + q < k) {
             const float4 v = reinterpret_cast<const float4*>(basis + (i0 + q) * bstride + off)[e];
-            cjmac(acc[q], make_float2(v.x, v.y), make_float2(x.x, x.y));
-            cjmac(acc[q], make_float2(v.z, v.w), make_float2(x.z, x.w));
+            cjmac(aw[q], make_float2(v.x, v.y), make_float2(x.x, x.y));
+            cjmac(aw[q], make_float2(v.z, v.w), make_float2(x.z, x.w));
+            cjmac(av[q], make_float2(v.x, v.y), make_float2(y.x, y.y));
+            cjmac(av[q], make_float2(v.z, v.w), make_float2(y.z, y.w));
           }
       }
-      vec2 = -1;  // done
     }
   }
-  if (vec2 >= 0)
-    for (long long e = blockIdx.x * (long long)RED_T + threadIdx.x; e < n; e += (long long)gridDim.x * RED_T) {
-      const cplx<R> x = w[off + e];
+  if (sizeof(R) == 8 || !vec2)
+    for (long long e = blk * (long long)RED_T + threadIdx.x; e < n; e += (long long)nblk_ * RED_T) {
+      const cplx<R> x = w[off + e], y = vj[e];
 #pragma unroll
       for (int q = 0; q < MD_K; ++q)
-        if (i0 + q < k) cjmac(acc[q], basis[(i0 + q) * bstride + off + e], x);
+        if (i0 + q < k) {
+          const cplx<R> v = basis[(i0 + q) * bstride + off + e];
+          cjmac(aw[q], v, x);
+          cjmac(av[q], v, y);
+        }
     }
-  // warp sums in the working precision (one transposing butterfly for the 8 values),
-  // then FP64 across the warps of the CTA and across CTAs
+  // warp sums in the working precision (one transposing butterfly for 8 values), then
+  // FP64 across the warps of the CTA and across CTAs
   static_assert(MD_K == 8, "transposing warp reduction of 8 values");
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  warp_sum8_transposed(acc, lane);
-  if ((lane & 3) == 0) scratch[warp * MD_K + warp_sum8_index(lane)] = to_c64(acc[0]);
+  warp_sum8_transposed(aw, lane);
+  warp_sum8_transposed(av, lane);
+  if ((lane & 3) == 0) {
+    scratch[0][warp * MD_K + warp_sum8_index(lane)] = to_c64(aw[0]);
+    scratch[1][warp * MD_K + warp_sum8_index(lane)] = to_c64(av[0]);
+  }
   __syncthreads();
-  if (threadIdx.x < MD_K && i0 + threadIdx.x < k) {
-    double2 t = scratch[threadIdx.x];
-    for (int w = 1; w < RED_T / 32; ++w) t += scratch[w * MD_K + threadIdx.x];
-    partial[((long long)r * kpad + i0 + threadIdx.x) * gridDim.x + blockIdx.x] = t;
+  const int q = threadIdx.x % MD_K, z = threadIdx.x / MD_K;
+  if (z < 2 && i0 + q < k) {
+    double2 t = scratch[z][q];
+    for (int u = 1; u < RED_T / 32; ++u) t += scratch[z][u * MD_K + q];
+    partial[(((long long)r * 2 + z) * kpad + i0 + q) * nblk_ + blk] = t;
   }
 }
-// k basis vectors; with kdev the count is *kdev + kadd (<= k) read on the device.
+// Row i, z = 0: <V_i, w> -> h[r][i]; z = 1: <V_i, V_j> -> column j = k - 1 and row j of G[r]
+__global__ void __launch_bounds__(RED_T) k_gram_final(double2* __restrict__ h, double2* __restrict__ G,
+                                                      const double2* __restrict__ partial, int count, int kpad, int ld,
+                                                      int k, const int* __restrict__ kdev, int kadd) {
+  __shared__ double2 scratch[RED_T / 32];
+  __shared__ double2 red[1];
+  const int r = blockIdx.x, i = blockIdx.y, z = blockIdx.z;
+  if (kdev) k = *kdev + kadd;
+  if (i >= k) return;  // uniform per block
+  const double2* p = partial + (((long long)r * 2 + z) * kpad + i) * count;
+  double2 acc = make_double2(0, 0);
+  for (int b = threadIdx.x; b < count; b += RED_T) acc += p[b];
+  block_sum_many<double2>(&acc, 1, scratch, red);
+  if (threadIdx.x == 0) {
+    if (z == 0) {
+      h[(long long)r * ld + i] = red[0];
+    } else {
+      double2* g = G + (long long)r * ld * ld;
+      g[(long long)(k - 1) * ld + i] = conjg(red[0]);
+      g[(long long)i * ld + k - 1] = red[0];
+    }
+  }
+}
+// h <- h + (h - G h): the coefficients of both projections (one CTA per rhs, k <= 65)
+constexpr int GC_T = 96;
+__global__ void __launch_bounds__(GC_T) k_gram_coef(double2* __restrict__ h, const double2* __restrict__ G, int ld,
+                                                    int k, const int* __restrict__ kdev, int kadd) {
+  __shared__ double2 hs[GC_T];
+  const int r = blockIdx.x, i = threadIdx.x;
+  if (kdev) k = *kdev + kadd;
+  double2* hr = h + (long long)r * ld;
+  if (i < k) hs[i] = hr[i];
+  __syncthreads();
+  if (i >= k) return;
+  const double2* g = G + (long long)r * ld * ld;
+  double2 t = hs[i];
+  for (int l = 0; l < k; ++l) t -= cjmul(g[(long long)l * ld + i], hs[l]);  // G_il = conj(G_li)
+  hr[i] = hs[i] + t;
+}
+// k basis vectors, the newest one V_{k-1}; with kdev the count is *kdev + kadd (<= k) read on
+// the device.  h: [nrhs][ld] coefficients of both projections, G: [nrhs][ld][ld].
 template <typename R>
-void launch_multidot(double2* out, const cplx<R>* basis, long long bstride, int k, int ldo, const cplx<R>* w,
-                     long long n, int nrhs, double2* partial, cudaStream_t st, const int* kdev, int kadd) {
+void launch_gram_project(double2* h, double2* G, const cplx<R>* basis, long long bstride, int k, int ld,
+                         const cplx<R>* w, long long n, int nrhs, double2* partial, cudaStream_t st, const int* kdev,
+                         int kadd) {
   const int nchunk = (k + MD_K - 1) / MD_K, kpad = nchunk * MD_K;
+  if (k > GC_T) throw Error(-1, "Gram-Schmidt supports k <= 96");
   const int nb = red_blocks(n, nrhs);  // independent of k: a captured graph sums in the same order
   const int vec2 = sizeof(R) == 4 && n % 2 == 0 && bstride % 2 == 0 && reinterpret_cast<uintptr_t>(basis) % 16 == 0 &&
                    reinterpret_cast<uintptr_t>(w) % 16 == 0;
-  k_multidot_partial<R><<<dim3(nb, nrhs, nchunk), RED_T, 0, st>>>(partial, basis, bstride, k, w, n, kpad, kdev, kadd,
-                                                                  vec2);
-  k_final<double2><<<dim3(nrhs, k), RED_T, 0, st>>>(out, partial, nb, (long long)kpad * nb, nb, ldo, kdev, kadd);
-  ++launch_counter();
+  k_gram_partial<R><<<dim3(nb * nchunk, nrhs), RED_T, 0, st>>>(partial, basis, bstride, k, w, n, nchunk, kdev, kadd,
+                                                               vec2);
+  WCMG_LAUNCH_CHECK();
+  k_gram_final<<<dim3(nrhs, k, 2), RED_T, 0, st>>>(h, G, partial, nb, kpad, ld, k, kdev, kadd);
+  WCMG_LAUNCH_CHECK();
+  k_gram_coef<<<nrhs, GC_T, 0, st>>>(h, G, ld, k, kdev, kadd);
+  WCMG_LAUNCH_CHECK();
+}
+
+// w -= V h and ||w||^2 in one pass: AN_T threads x at most 608 CTAs per rhs stride over the
+// field (two entries per 16-byte access when vec2), four basis vectors in flight.
+constexpr int AN_T = 512;
+template <typename R>
+__global__ void __launch_bounds__(AN_T) k_project_norm(cplx<R>* __restrict__ w, const cplx<R>* __restrict__ basis,
+                                                       long long bstride, int k, const double2* __restrict__ h, int ld,
+                                                       long long n, double* __restrict__ partial,
+                                                       const int* __restrict__ kdev, int kadd, int vec2) {
+  __shared__ cplx<R> cf[GC_T];
+  __shared__ double scratch[AN_T / 32];
+  __shared__ double red[1];
+  const int r = blockIdx.y;
+  if (kdev) k = min(*kdev + kadd, k);
+  for (int i = threadIdx.x; i < k; i += AN_T) {
+    const double2 c = h[(long long)r * ld + i];
+    cf[i] = cmk(R(-c.x), R(-c.y));
+  }
+  __syncthreads();
+  w += (long long)r * n;
+  basis += (long long)r * n;
+  R nn = 0;
+  if (sizeof(R) == 4 && vec2) {
+    const long long n2 = n >> 1;
+    for (long long e = blockIdx.x * (long long)AN_T + threadIdx.x; e < n2; e += (long long)gridDim.x * AN_T) {
+      float4 x = reinterpret_cast<float4*>(w)[e];
+      float2 lo = make_float2(x.x, x.y), hi = make_float2(x.z, x.w);
+#pragma unroll 4
+      for (int i = 0; i < k; ++i) {
+        const float4 v = reinterpret_cast<const float4*>(basis + i * bstride)[e];
+        const float2 c = make_float2((float)cf[i].x, (float)cf[i].y);
+        cmac(lo, c, make_float2(v.x, v.y));
+        cmac(hi, c, make_float2(v.z, v.w));
+      }
+      reinterpret_cast<float4*>(w)[e] = make_float4(lo.x, lo.y, hi.x, hi.y);
+      nn += (R)(cnorm2(lo) + cnorm2(hi));
+    }
+  } else {
+    for (long long e = blockIdx.x * (long long)AN_T + threadIdx.x; e < n; e += (long long)gridDim.x * AN_T) {
+      cplx<R> x = w[e];
+#pragma unroll 4
+      for (int i = 0; i < k; ++i) cmac(x, cf[i], basis[i * bstride + e]);
+      w[e] = x;
+      nn += cnorm2(x);
+    }
+  }
+  const R v[1] = {nn};
+  block_sum_mixed<R, 1>(v, scratch, red);
+  if (threadIdx.x == 0) partial[(long long)r * gridDim.x + blockIdx.x] = red[0];
+}
+template <typename R>
+void launch_project_norm(double* norm2, cplx<R>* w, const cplx<R>* basis, long long bstride, int k, const double2* h,
+                         int ld, long long n, int nrhs, double* partial, cudaStream_t st, const int* kdev, int kadd) {
+  if (k > GC_T) throw Error(-1, "Gram-Schmidt supports k <= 96");
+  const int vec2 = sizeof(R) == 4 && n % 2 == 0 && bstride % 2 == 0 && reinterpret_cast<uintptr_t>(basis) % 16 == 0 &&
+                   reinterpret_cast<uintptr_t>(w) % 16 == 0;
+  const long long per = (long long)AN_T * (vec2 ? 2 : 1);
+  const int nb = (int)std::max(1LL, std::min(608LL, (n + per - 1) / per));
+  k_project_norm<R><<<dim3(nb, nrhs), AN_T, 0, st>>>(w, basis, bstride, k, h, ld, n, partial, kdev, kadd, vec2);
+  WCMG_LAUNCH_CHECK();
+  k_final<double><<<dim3(nrhs, 1), RED_T, 0, st>>>(norm2, partial, nb, nb, 0, 1);
   WCMG_LAUNCH_CHECK();
 }
 
@@ -213,8 +341,9 @@ void launch_axpby(cplx<R>* y, double a, const cplx<R>* x, double b, long long n,
 }
 
 template <typename R>
-__global__ void k_scale_dev(cplx<R>* __restrict__ y, const cplx<R>* __restrict__ x, const double* __restrict__ s,
-                            int inv_sqrt, long long n, const int* __restrict__ ydev, int yadd, long long ystride) {
+__global__ void k_scale_dev(cplx<R>* y, const cplx<R>* x, const double* __restrict__ s,
+                            int inv_sqrt, long long n, const int* __restrict__ ydev, int yadd, long long ystride,
+                            cplx<R>* __restrict__ y2) {
   __shared__ R f_s;
   const int r = blockIdx.y;
   if (ydev) y += (long long)(*ydev + yadd) * ystride;
@@ -226,12 +355,14 @@ __global__ void k_scale_dev(cplx<R>* __restrict__ y, const cplx<R>* __restrict__
   __syncthreads();
   const long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (e >= n) return;
-  y[(long long)r * n + e] = f_s * x[(long long)r * n + e];
+  const cplx<R> v = f_s * x[(long long)r * n + e];
+  y[(long long)r * n + e] = v;
+  if (y2) y2[(long long)r * n + e] = v;
 }
 template <typename R>
 void launch_scale_dev(cplx<R>* y, const cplx<R>* x, const double* s, int inv_sqrt, long long n, int nrhs,
-                      cudaStream_t st, const int* ydev, int yadd, long long ystride) {
-  k_scale_dev<R><<<dim3(nblk(n, 256), nrhs), 256, 0, st>>>(y, x, s, inv_sqrt, n, ydev, yadd, ystride);
+                      cudaStream_t st, const int* ydev, int yadd, long long ystride, cplx<R>* y2) {
+  k_scale_dev<R><<<dim3(nblk(n, 256), nrhs), 256, 0, st>>>(y, x, s, inv_sqrt, n, ydev, yadd, ystride, y2);
   WCMG_LAUNCH_CHECK();
 }
 
@@ -484,139 +615,187 @@ __device__ double gmres_column(GmresState S, int r, int j, const double2* hcol, 
   return h > 0.0 ? 1.0 / h : 0.0;
 }
 
-__global__ void k_gmres_step(GmresState S, int j, const double2* __restrict__ h1, const double2* __restrict__ h2,
-                             const double* __restrict__ hnorm2, double tol, int final_done, int nrhs,
+// The same for one rhs (row 0 of the state) from shared copies: hcol [j + 1] is overwritten,
+// cs and sn hold the rotations of columns 0 .. j - 1.
+__device__ void gmres_rotate(GmresState S, int j, double2* hcol, const double* cs, const double2* sn, double hn2,
+                             double tol, int final_done) {
+  const int m = S.m;
+  for (int i = 0; i < j; ++i) {
+    const double2 a = hcol[i], b = hcol[i + 1];
+    S.H[i * m + j] = cs[i] * a + cmul(sn[i], b);
+    hcol[i + 1] = cs[i] * b - cmul(conjg(sn[i]), a);
+  }
+  double c; double2 s, rho;
+  givens(hcol[j], make_double2(sqrt(hn2), 0), c, s, rho);
+  S.cs[j] = c; S.sn[j] = s;
+  S.H[j * m + j] = rho;
+  S.H[(j + 1) * m + j] = make_double2(0, 0);
+  const double2 gj = S.g[j];
+  S.g[j + 1] = -cmul(conjg(s), gj);
+  S.g[j] = c * gj;
+  const double res = sqrt(cnorm2(S.g[j + 1]));
+  S.resid[0] = res;
+  S.jdone[0] = j + 1;
+  if (res <= tol * S.bnorm[0]) {
+    S.active[0] = 0;
+    if (final_done) S.done[0] = 1;
+  }
+}
+
+__global__ void k_gmres_step(GmresState S, int j, const double2* __restrict__ h, const double* __restrict__ hnorm2, double tol, int final_done, int nrhs,
                              double* __restrict__ inv_h, const int* __restrict__ jdev) {
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= nrhs) return;
   if (jdev) j = *jdev;
   const int m = S.m;
   if (!S.active[r]) { inv_h[r] = 0.0; return; }
-  double2 hcol[65];
-  for (int i = 0; i <= j; ++i) hcol[i] = h1[(long long)r * (m + 1) + i] + h2[(long long)r * (m + 1) + i];
-  inv_h[r] = gmres_column(S, r, j, hcol, hnorm2[r], tol, final_done);
+  inv_h[r] = gmres_column(S, r, j, h + (long long)r * (m + 1), hnorm2[r], tol, final_done);
 }
 
 // ---- fused Arnoldi step for short vectors (one rhs) ----
 // Everything of one (F)GMRES Arnoldi step after the operator application, for
 // vectors short enough that a single thread-block cluster streams them from L2:
-// both classical Gram-Schmidt passes h1 = V^dag w, w -= V h1, h2 = V^dag w,
-// w -= V h2, the norm ||w||^2, the Givens update of Hessenberg column j and
-// V_{j+1} = w / ||w||.  CTA c of the C-CTA cluster owns a contiguous range of the
-// vector; its partial sums (warp sums in the working precision, FP64 across
-// warps) are exchanged through distributed shared memory, and every CTA adds the C
-// partials in the same order, so all CTAs hold identical coefficients.  One
-// launch replaces ten (three two-stage reductions, two updates, Givens, scaling).
-constexpr int AC_T = 256, AC_MAXK = 65;
-
-template <typename R>
-__device__ __forceinline__ void ac_reduce8(cplx<R> (&acc)[8], double2* __restrict__ scr, double2* __restrict__ out,
-                                           int i0, int k) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  warp_sum8_transposed(acc, lane);
-  if ((lane & 3) == 0) scr[warp * 8 + warp_sum8_index(lane)] = to_c64(acc[0]);
-  __syncthreads();
-  if (threadIdx.x < 8 && i0 + threadIdx.x < k) {
-    double2 t = scr[threadIdx.x];
-    for (int w = 1; w < AC_T / 32; ++w) t += scr[w * 8 + threadIdx.x];
-    out[i0 + threadIdx.x] = t;
-  }
-  __syncthreads();
-}
+// the sweep of <V_i, w> and <V_i, V_j> (the newest column of the Gram matrix), the
+// coefficients h + (h - G h) of both Gram-Schmidt passes, w - V h, its norm, the Givens
+// update of Hessenberg column j and V_{j+1} = w / ||w||.  CTA c of the C-CTA cluster owns
+// a contiguous range of the vector.  Bound by latency, so: one warp per basis vector in
+// the sweep (warp sums only, no block barrier per chunk of vectors), the updated elements
+// stay in registers until the norm is known, everything the coefficients and the rotation
+// need (G, cs, sn, g) is requested before the sweep, and the rotation runs from shared
+// memory while the cluster writes V_{j+1}.  Partial sums are exchanged through distributed
+// shared memory and every CTA adds the C partials in the same order, so all CTAs hold
+// identical coefficients.  24.6k entries, 16 CTAs: 34 us before (two sweeps and two updates,
+// four cluster barriers, the rotation from global memory).
+constexpr int AC_T = 512, AC_MAXK = 65, AC_W = AC_T / 32;
+constexpr int AC_EL = 16;  // elements per thread: n <= 2^17 over at least 8 CTAs ... 16 x 512 each
 
 template <typename R>
 __global__ void __launch_bounds__(AC_T) k_arnoldi_cluster(cplx<R>* __restrict__ Vb, long long bstride,
-                                                          cplx<R>* __restrict__ w, long long n, GmresState S, int j,
-                                                          const int* __restrict__ jdev, double tol, int final_done) {
+                                                          const cplx<R>* __restrict__ w, long long n, GmresState S,
+                                                          double2* __restrict__ G, int j, const int* __restrict__ jdev,
+                                                          double tol, int final_done, cplx<R>* __restrict__ vnext) {
   namespace cg = cooperative_groups;
   cg::cluster_group cl = cg::this_cluster();
   const int C = (int)cl.num_blocks(), crank = (int)cl.block_rank();
-  __shared__ double2 pA[AC_MAXK], pB[AC_MAXK];  // this CTA's partial sums (read by the whole cluster)
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  __shared__ double2 pA[AC_MAXK], pV[AC_MAXK];  // this CTA's partial sums (read by the whole cluster)
   __shared__ double pN;
-  __shared__ double2 h1s[AC_MAXK], hcol[AC_MAXK];
-  __shared__ double2 scr[(AC_T / 32) * 8];
-  __shared__ double dscr[AC_T / 32];
+  __shared__ double2 hs[AC_MAXK], gs[AC_MAXK], hcol[AC_MAXK];
+  __shared__ cplx<R> cf[AC_MAXK];
+  __shared__ double csn[AC_MAXK];
+  __shared__ double2 snn[AC_MAXK];
+  __shared__ double dscr[AC_W];
+  __shared__ double dred[1];
   if (jdev) j = *jdev;
-  const int k = j + 1;
+  const int k = j + 1, m = S.m, ld = m + 1;
   const bool act = S.active[0] != 0;  // before this step (CTA 0 may change it below)
-  const long long per = (n + C - 1) / C;
-  const long long e0 = (long long)crank * per, e1 = e0 + per < n ? e0 + per : n;
-  // pass 1: <V_i, w>
-  for (int i0 = 0; i0 < k; i0 += 8) {
-    cplx<R> acc[8];
+  const int per = (int)((n + C - 1) / C);
+  const int e0 = crank * per, cnt = max(0, min(per, (int)n - e0));
+  // row i of G without its newest entry: 8 lanes per row
+  const int gi = threadIdx.x >> 3, gl = threadIdx.x & 7;
+  double2 gr[8];
 #pragma unroll
-    for (int g = 0; g < 8; ++g) acc[g] = czero<R>();
-    for (long long e = e0 + threadIdx.x; e < e1; e += AC_T) {
-      const cplx<R> x = w[e];
-#pragma unroll
-      for (int g = 0; g < 8; ++g)
-        if (i0 + g < k) cjmac(acc[g], Vb[(i0 + g) * bstride + e], x);
+  for (int t = 0; t < 8; ++t) {
+    const int l = gl + 8 * t;
+    gr[t] = gi < k && l < k && l != j && gi != j ? G[(long long)l * ld + gi] : make_double2(0, 0);
+  }
+  if (crank == 0)
+    for (int i = threadIdx.x; i < j; i += AC_T) {
+      csn[i] = S.cs[i];
+      snn[i] = S.sn[i];
     }
-    ac_reduce8<R>(acc, scr, pA, i0, k);
+  // sweep: <V_i, w> and <V_i, V_j>, one warp per i
+  const cplx<R>* wv = w + e0;
+  const cplx<R>* vj = Vb + (long long)j * bstride + e0;
+  for (int i = warp; i < k; i += AC_W) {
+    const cplx<R>* vi = Vb + (long long)i * bstride + e0;
+    cplx<R> aw = czero<R>(), av = czero<R>();
+#pragma unroll 8
+    for (int e = lane; e < cnt; e += 32) {
+      const cplx<R> v = vi[e];
+      cjmac(aw, v, wv[e]);
+      cjmac(av, v, vj[e]);
+    }
+    const cplx<R> tw = warp_sum(aw), tv = warp_sum(av);
+    if (lane == 0) {
+      pA[i] = to_c64(tw);
+      pV[i] = to_c64(tv);
+    }
   }
   cl.sync();
-  for (int i = threadIdx.x; i < k; i += AC_T) {
+  for (int i = threadIdx.x; i < 2 * k; i += AC_T) {
+    const bool second = i >= k;
+    const int q = second ? i - k : i;
     double2 t = make_double2(0, 0);
-    for (int c = 0; c < C; ++c) t += cl.map_shared_rank(pA, c)[i];
-    h1s[i] = t;
+#pragma unroll 8
+    for (int c = 0; c < C; ++c) t += cl.map_shared_rank(second ? pV : pA, c)[q];
+    (second ? gs : hs)[q] = t;
   }
   __syncthreads();
-  // w -= V h1, then pass 2: <V_i, w>  (each thread revisits only its own elements)
-  for (long long e = e0 + threadIdx.x; e < e1; e += AC_T) {
-    cplx<R> x = w[e];
-    for (int i = 0; i < k; ++i) {
-      const double2 h = h1s[i];
-      cnmac(x, cmk(R(h.x), R(h.y)), Vb[i * bstride + e]);
-    }
-    w[e] = x;
-  }
-  for (int i0 = 0; i0 < k; i0 += 8) {
-    cplx<R> acc[8];
-#pragma unroll
-    for (int g = 0; g < 8; ++g) acc[g] = czero<R>();
-    for (long long e = e0 + threadIdx.x; e < e1; e += AC_T) {
-      const cplx<R> x = w[e];
-#pragma unroll
-      for (int g = 0; g < 8; ++g)
-        if (i0 + g < k) cjmac(acc[g], Vb[(i0 + g) * bstride + e], x);
-    }
-    ac_reduce8<R>(acc, scr, pB, i0, k);
-  }
-  cl.sync();
-  for (int i = threadIdx.x; i < k; i += AC_T) {
+  // h + (h - G h), G's newest column gs: G_{l j} = gs_l, G_{j l} = conj(gs_l)
+  {
     double2 t = make_double2(0, 0);
-    for (int c = 0; c < C; ++c) t += cl.map_shared_rank(pB, c)[i];
-    hcol[i] = h1s[i] + t;
-    h1s[i] = t;  // h2
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int l = gl + 8 * q;
+      if (gi < k && l < k) {
+        // gr holds G_{l gi}; the sum needs G_{gi l} = conj(G_{l gi})
+        const double2 g = l == j ? conjg(gs[gi]) : gi == j ? gs[l] : gr[q];
+        t += cjmul(g, hs[l]);
+      }
+    }
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) t += shfl_xor2(t, o);
+    if (gi < k && gl == 0) {
+      const double2 h = hs[gi] + (hs[gi] - t);
+      hcol[gi] = h;
+      cf[gi] = cmk(R(h.x), R(h.y));
+      if (crank == 0) {
+        G[(long long)j * ld + gi] = conjg(gs[gi]);
+        G[(long long)gi * ld + j] = gs[gi];
+      }
+    }
   }
   __syncthreads();
-  // w -= V h2 and ||w||^2
+  // w - V h in registers, and its norm
+  cplx<R> x[AC_EL];
   R nn = 0;
-  for (long long e = e0 + threadIdx.x; e < e1; e += AC_T) {
-    cplx<R> x = w[e];
-    for (int i = 0; i < k; ++i) {
-      const double2 h = h1s[i];
-      cnmac(x, cmk(R(h.x), R(h.y)), Vb[i * bstride + e]);
+#pragma unroll
+  for (int u = 0; u < AC_EL; ++u) {
+    const int e = threadIdx.x + u * AC_T;
+    if (e < cnt) {
+      cplx<R> t = wv[e];
+      const cplx<R>* v = Vb + e0 + e;
+#pragma unroll 8
+      for (int i = 0; i < k; ++i) cnmac(t, cf[i], v[i * bstride]);
+      x[u] = t;
+      nn += cnorm2(t);
     }
-    w[e] = x;
-    nn += cnorm2(x);
   }
   {
     const R v[1] = {nn};
-    double red[1];
-    block_sum_mixed<R, 1>(v, dscr, red);
-    if (threadIdx.x == 0) pN = red[0];
+    block_sum_mixed<R, 1>(v, dscr, dred);
+    if (threadIdx.x == 0) pN = dred[0];
   }
   cl.sync();
   double hn2 = 0.0;
+#pragma unroll 8
   for (int c = 0; c < C; ++c) hn2 += *cl.map_shared_rank(&pN, c);
-  // V_{j+1} = w / ||w|| and, on one thread, the Givens update of column j
+  cl.barrier_arrive();  // done with the others' shared memory
+  if (crank == 0 && threadIdx.x == 0 && act) gmres_rotate(S, j, hcol, csn, snn, hn2, tol, final_done);
   const double h = sqrt(hn2);
   const R inv = (R)(act && h > 0.0 ? 1.0 / h : 0.0);
-  cplx<R>* vn = Vb + (long long)(j + 1) * bstride;
-  for (long long e = e0 + threadIdx.x; e < e1; e += AC_T) vn[e] = inv * w[e];
-  if (crank == 0 && threadIdx.x == 0 && act) gmres_column(S, 0, j, hcol, hn2, tol, final_done);
-  cl.sync();  // no CTA leaves while another may still read its shared memory
+  cplx<R>* vn = Vb + (long long)(j + 1) * bstride + e0;
+#pragma unroll
+  for (int u = 0; u < AC_EL; ++u) {
+    const int e = threadIdx.x + u * AC_T;
+    if (e < cnt) {
+      const cplx<R> t = inv * x[u];
+      vn[e] = t;
+      if (vnext) vnext[e0 + e] = t;
+    }
+  }
+  cl.barrier_wait();  // no CTA leaves while another may still read its shared memory
 }
 
 static int arnoldi_cluster_size() {
@@ -654,12 +833,13 @@ static int arnoldi_cluster_size() {
 // entries) but not for fine-level ones (a 16^4 lattice, 7.9 x 10^5 entries: 300 us per
 // step against about 60 us), so it takes vectors of at most 2^17 entries.
 bool arnoldi_fused_ok(long long n, int nrhs, int m) {
-  return nrhs == 1 && m + 1 <= AC_MAXK && n <= (1LL << 17) && arnoldi_cluster_size() > 0;
+  return nrhs == 1 && m + 1 <= AC_MAXK && n <= (1LL << 17) && arnoldi_cluster_size() > 0 &&
+         (n + arnoldi_cluster_size() - 1) / arnoldi_cluster_size() <= AC_EL * AC_T;
 }
 
 template <typename R>
-void launch_arnoldi_fused(cplx<R>* Vb, long long bstride, cplx<R>* w, long long n, const GmresState& S, int j,
-                          const int* jdev, double tol, int final_done, cudaStream_t st) {
+void launch_arnoldi_fused(cplx<R>* Vb, long long bstride, cplx<R>* w, long long n, const GmresState& S, double2* G,
+                          int j, const int* jdev, double tol, int final_done, cudaStream_t st, cplx<R>* vnext) {
   const int C = arnoldi_cluster_size();
   if (C <= 0) throw Error(-1, "no thread-block cluster available for the fused Arnoldi step");
   auto kern = k_arnoldi_cluster<R>;
@@ -675,13 +855,13 @@ void launch_arnoldi_fused(cplx<R>* Vb, long long bstride, cplx<R>* w, long long 
   at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  WCMG_CUDA(cudaLaunchKernelEx(&cfg, kern, Vb, bstride, w, n, S, j, jdev, tol, final_done));
+  WCMG_CUDA(cudaLaunchKernelEx(&cfg, kern, Vb, bstride, (const cplx<R>*)w, n, S, G, j, jdev, tol, final_done, vnext));
   WCMG_LAUNCH_CHECK();
 }
-template void launch_arnoldi_fused<float>(float2*, long long, float2*, long long, const GmresState&, int, const int*,
-                                          double, int, cudaStream_t);
-template void launch_arnoldi_fused<double>(double2*, long long, double2*, long long, const GmresState&, int,
-                                           const int*, double, int, cudaStream_t);
+template void launch_arnoldi_fused<float>(float2*, long long, float2*, long long, const GmresState&, double2*, int,
+                                          const int*, double, int, cudaStream_t, float2*);
+template void launch_arnoldi_fused<double>(double2*, long long, double2*, long long, const GmresState&, double2*, int,
+                                           const int*, double, int, cudaStream_t, double2*);
 
 __global__ void k_gmres_solve_y(GmresState S, int nrhs) {
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
@@ -712,9 +892,9 @@ void launch_gmres_start(const GmresState& s, const double* nrm2, double tol, int
   k_gmres_start<<<nblk(nrhs, 64), 64, 0, st>>>(s, nrm2, tol, nrhs, inv_beta);
   WCMG_LAUNCH_CHECK();
 }
-void launch_gmres_step(const GmresState& s, int j, const double2* h1, const double2* h2, const double* hnorm2,
-                       double tol, int final_done, int nrhs, double* inv_h, cudaStream_t st, const int* jdev) {
-  k_gmres_step<<<nblk(nrhs, 64), 64, 0, st>>>(s, j, h1, h2, hnorm2, tol, final_done, nrhs, inv_h, jdev);
+void launch_gmres_step(const GmresState& s, int j, const double2* h, const double* hnorm2, double tol,
+                       int final_done, int nrhs, double* inv_h, cudaStream_t st, const int* jdev) {
+  k_gmres_step<<<nblk(nrhs, 64), 64, 0, st>>>(s, j, h, hnorm2, tol, final_done, nrhs, inv_h, jdev);
   WCMG_LAUNCH_CHECK();
 }
 void launch_gmres_solve_y(const GmresState& s, int nrhs, cudaStream_t st) {
@@ -761,15 +941,17 @@ void launch_counter_gaussian(double2* out, long long n, int nfields, unsigned lo
 #define WCMG_INST(R)                                                                                             \
   template void launch_dot<R>(double2*, const cplx<R>*, const cplx<R>*, long long, int, double2*, cudaStream_t); \
   template void launch_norm2<R>(double*, const cplx<R>*, long long, int, double*, cudaStream_t);                 \
-  template void launch_multidot<R>(double2*, const cplx<R>*, long long, int, int, const cplx<R>*, long long, int, \
-                                   double2*, cudaStream_t, const int*, int);                                     \
+  template void launch_gram_project<R>(double2*, double2*, const cplx<R>*, long long, int, int, const cplx<R>*,  \
+                                       long long, int, double2*, cudaStream_t, const int*, int);                 \
+  template void launch_project_norm<R>(double*, cplx<R>*, const cplx<R>*, long long, int, const double2*, int,   \
+                                       long long, int, double*, cudaStream_t, const int*, int);                  \
   template void launch_multiaxpy<R>(cplx<R>*, const cplx<R>*, long long, int, const double2*, int, double,       \
                                     long long, int, cudaStream_t, const int*, int);                              \
   template void launch_copy_idx<R>(cplx<R>*, const cplx<R>*, long long, const int*, long long, long long,        \
                                    cudaStream_t);                                                                \
   template void launch_axpby<R>(cplx<R>*, double, const cplx<R>*, double, long long, int, cudaStream_t);         \
   template void launch_scale_dev<R>(cplx<R>*, const cplx<R>*, const double*, int, long long, int, cudaStream_t,  \
-                                    const int*, int, long long);                                                 \
+                                    const int*, int, long long, cplx<R>*);                                       \
   template void launch_mr_update<R>(cplx<R>*, cplx<R>*, const cplx<R>*, const double2*, const double*, long long, \
                                     int, cudaStream_t, bool, bool);                                              \
   template void launch_mr_residual<R>(cplx<R>*, const cplx<R>*, const double2*, const double*, long long, int,   \

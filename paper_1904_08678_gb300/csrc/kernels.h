@@ -185,13 +185,20 @@ void launch_dot(double2* out, const cplx<R>* a, const cplx<R>* b, long long n, i
                 cudaStream_t st);
 template <typename R>
 void launch_norm2(double* out, const cplx<R>* a, long long n, int nrhs, double* partial, cudaStream_t st);
-// out[r][i] = <basis_i, w> for i < k; basis_i at basis + i * bstride (each [nrhs][n]).
+// Arnoldi Gram-Schmidt against V_0 .. V_{k-1} (V_i at basis + i * bstride, each [nrhs][n]):
+// h[r][i] = the coefficients of two classical passes, from one sweep that forms <V_i, w> and
+// the newest column of the Gram matrix G[r] = V^dag V (h: [nrhs][ld], G: [nrhs][ld][ld]);
+// partial: nrhs * 2 * roundup(k, 8) * 608 entries.  Then w -= V h and norm2[r] = ||w||^2.
 // kdev (nullable, device): the count is *kdev + kadd instead (at most k, which sizes
 // the grid) -- the Arnoldi step number of a device-driven loop.
 template <typename R>
-void launch_multidot(double2* out, const cplx<R>* basis, long long bstride, int k, int ldo, const cplx<R>* w,
-                     long long n, int nrhs, double2* partial, cudaStream_t st, const int* kdev = nullptr,
-                     int kadd = 0);
+void launch_gram_project(double2* h, double2* G, const cplx<R>* basis, long long bstride, int k, int ld,
+                         const cplx<R>* w, long long n, int nrhs, double2* partial, cudaStream_t st,
+                         const int* kdev = nullptr, int kadd = 0);
+template <typename R>
+void launch_project_norm(double* norm2, cplx<R>* w, const cplx<R>* basis, long long bstride, int k, const double2* h,
+                         int ld, long long n, int nrhs, double* partial, cudaStream_t st, const int* kdev = nullptr,
+                         int kadd = 0);
 // w[r] += sign * sum_{i<k} coef[r*ldc + i] * basis_i[r]; kdev as for launch_multidot
 template <typename R>
 void launch_multiaxpy(cplx<R>* w, const cplx<R>* basis, long long bstride, int k, const double2* coef, int ldc,
@@ -206,10 +213,11 @@ void launch_add_widened(double2* y, const float2* x, long long n, cudaStream_t s
 template <typename R>
 void launch_axpby(cplx<R>* y, double a, const cplx<R>* x, double b, long long n, int nrhs, cudaStream_t st);
 // y[r] = x[r] * s[r] (s real, device; 1/sqrt(s) with inv_sqrt).  ydev (nullable):
-// y is offset by (*ydev + yadd) * ystride on the device.
+// y is offset by (*ydev + yadd) * ystride on the device.  y2 (nullable): a second copy.
 template <typename R>
 void launch_scale_dev(cplx<R>* y, const cplx<R>* x, const double* s, int inv_sqrt, long long n, int nrhs,
-                      cudaStream_t st, const int* ydev = nullptr, int yadd = 0, long long ystride = 0);
+                      cudaStream_t st, const int* ydev = nullptr, int yadd = 0, long long ystride = 0,
+                      cplx<R>* y2 = nullptr);
 // MR updates with alpha = pr[q] / pp[q] (0 if pp = 0), pr = <p, r>, pp = <p, p> of rhs q;
 // x_zero: x is taken as 0 and not read.
 // One step: x += alpha r; r_next: r -= alpha p in place.
@@ -264,20 +272,21 @@ struct GmresState {
   int m;
 };
 // h column j is in H (entries 0..j from multidot); hnorm holds ||w||.
-// h1, h2: the two CGS passes' coefficients [nrhs][m+1]; hnorm2 = ||w||^2 after both.
+// h: the coefficients of both Gram-Schmidt passes [nrhs][m+1]; hnorm2 = ||w||^2 after both.
 // `final_done`: a recurrence convergence also marks the rhs done (no true-residual check).
 // One fused Arnoldi step after the operator application, for one short rhs
-// (n <= 2^17, restart <= 64): CGS2 projections of w against V_0..V_j, the norm,
-// the Givens update of Hessenberg column j and V_{j+1} = w / ||w||, in one launch
-// of a thread-block cluster (16 CTAs, else 8).  jdev (nullable): step on the device.
+// (n <= 2^17, restart <= 64): both projections of w against V_0..V_j (G: Gram matrix of the
+// basis, [m+1][m+1]), the norm, the Givens update of Hessenberg column j and V_{j+1} =
+// w / ||w||, in one launch of a thread-block cluster (16 CTAs, else 8).  jdev (nullable):
+// step on the device.  vnext (nullable): a second copy of V_{j+1}.
 bool arnoldi_fused_ok(long long n, int nrhs, int m);
 template <typename R>
-void launch_arnoldi_fused(cplx<R>* Vb, long long bstride, cplx<R>* w, long long n, const GmresState& S, int j,
-                          const int* jdev, double tol, int final_done, cudaStream_t st);
+void launch_arnoldi_fused(cplx<R>* Vb, long long bstride, cplx<R>* w, long long n, const GmresState& S, double2* G,
+                          int j, const int* jdev, double tol, int final_done, cudaStream_t st,
+                          cplx<R>* vnext = nullptr);
 // jdev (nullable, device): the step number is *jdev instead of j.
-void launch_gmres_step(const GmresState& s, int j, const double2* h1, const double2* h2, const double* hnorm2,
-                       double tol, int final_done, int nrhs, double* inv_h, cudaStream_t st,
-                       const int* jdev = nullptr);
+void launch_gmres_step(const GmresState& s, int j, const double2* h, const double* hnorm2, double tol,
+                       int final_done, int nrhs, double* inv_h, cudaStream_t st, const int* jdev = nullptr);
 // done[r] |= nrm2[r] <= (tol * bnorm[r])^2
 void launch_gmres_mark_done(const GmresState& s, const double* nrm2, double tol, int nrhs, cudaStream_t st);
 void launch_gmres_solve_y(const GmresState& s, int nrhs, cudaStream_t st);
