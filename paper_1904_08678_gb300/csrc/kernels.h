@@ -106,7 +106,11 @@ void launch_block_ortho(double2* vecs, int Vf, int nc, int bvol, int nvec, bool 
 // input is vecs itself, or the FP32 field in32 when given; out32 (nullable) receives
 // the FP32 rounding of the result as well.
 void launch_block_ortho_df(double2* vecs, float4* qdf, int Vf, int nc, int bvol, int nvec, bool fine, int* err,
-                           cudaStream_t st, const float2* in32 = nullptr, float2* out32 = nullptr);
+                           cudaStream_t st, const int* only, const float2* in32 = nullptr, float2* out32 = nullptr);
+// Cholesky QR of the same panels (ortho.cu): W: panels x nvec^2 entries of scratch; flag[2 blk +
+// s] = 1 leaves a panel (ill-conditioned) to launch_block_ortho_df, *nflag += their number.
+void launch_cholqr(double2* vecs, double2* W, int* flag, int* nflag, int Vf, int nc, int bvol, int nvec, bool fine,
+                   cudaStream_t st, const float2* in32 = nullptr, float2* out32 = nullptr);
 // cols[b] = Pi_s v_i with (s, i) = divmod(b0 + b, nvec), for b < ncols.
 template <typename R>
 void launch_make_columns(cplx<R>* cols, const cplx<R>* vecs, int Vf, int nc, int nvec, int b0, int ncols, bool fine,

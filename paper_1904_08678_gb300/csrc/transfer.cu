@@ -703,7 +703,8 @@ __global__ void __launch_bounds__(256, 2) k_block_ortho(double2* __restrict__ ve
 }
 
 // ---------------- block orthonormalisation in double-float arithmetic ----------------
-// The same Gram-Schmidt (classical, with the selective second pass and the
+// For the panels that the Cholesky QR of ortho.cu flags as too ill-conditioned (`only`, one
+// word per (aggregate, chirality); the other CTAs end at once).  The same Gram-Schmidt (classical, with the selective second pass and the
 // normalisation of k_block_ortho) with every multiply-add on the FP32 pipe in
 // double-float ("DF") form: a value is the unevaluated sum h + l of two floats
 // (|l| <= ulp(h) / 2 once normalised: 48 significand bits).  Error-free
@@ -744,11 +745,13 @@ template <int MAXE, int NT, int MINB, int GS>
 __global__ void __launch_bounds__(NT, MINB) k_block_ortho_df(double2* __restrict__ vecs, float4* __restrict__ qdf,
                                                              int Vf, int nc, int bvol, int nvec, bool fine,
                                                              int* __restrict__ err, const float2* __restrict__ in32,
-                                                             float2* __restrict__ out32) {
+                                                             float2* __restrict__ out32,
+                                                             const int* __restrict__ only) {
   constexpr int MV = 33;  // nvec <= 32, slot 32: squared norm
   __shared__ dfc scratch[NT / 32][MV];
   __shared__ dfc red[MV];
   const int blk = blockIdx.x, s = blockIdx.y;
+  if (!only[2 * blk + s]) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int nelem = bvol * (nc >> 1);
   const long long fstride = (long long)Vf * nc;
@@ -859,11 +862,13 @@ template <int MAXE, int NT, int MINB, int GS>
 __global__ void __launch_bounds__(NT, MINB) k_block_ortho_df2(double2* __restrict__ vecs, float4* __restrict__ qdf,
                                                               int Vf, int nc, int bvol, int nvec, bool fine,
                                                               int* __restrict__ err, const float2* __restrict__ in32,
-                                                              float2* __restrict__ out32) {
+                                                              float2* __restrict__ out32,
+                                                              const int* __restrict__ only) {
   constexpr int MV = 33;  // nvec <= 32, slot 32: squared norm
   __shared__ dfc scratch[2][NT / 32][MV];
   __shared__ dfc red[2][MV];
   const int blk = blockIdx.x, s = blockIdx.y;
+  if (!only[2 * blk + s]) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int nelem = bvol * (nc >> 1);
   const long long fstride = (long long)Vf * nc;
@@ -1045,7 +1050,7 @@ __global__ void __launch_bounds__(NT, MINB) k_block_ortho_df2(double2* __restric
 
 
 void launch_block_ortho_df(double2* vecs, float4* qdf, int Vf, int nc, int bvol, int nvec, bool fine, int* err,
-                           cudaStream_t st, const float2* in32, float2* out32) {
+                           cudaStream_t st, const int* only, const float2* in32, float2* out32) {
   const int nelem = bvol * (nc / 2);
   if (nvec > 32) throw Error(-1, "block orthonormalisation supports nvec <= 32");
   if (nelem > 256 * 8) throw Error(-1, "aggregate too large for block orthonormalisation");
@@ -1058,11 +1063,11 @@ void launch_block_ortho_df(double2* vecs, float4* qdf, int Vf, int nc, int bvol,
   // 61 ms.  Columns in pairs, 512 x 3, 2 CTAs (64 registers), groups of 2: 47 ms (16^3x32:
   // 3.5 against 3.8 ms).  The kernels wait on their re-reads of earlier Q columns.
   if (nelem <= 256 * 2)
-    k_block_ortho_df<2, 256, 3, 8><<<grid, 256, 0, st>>>(vecs, qdf, Vf, nc, bvol, nvec, fine, err, in32, out32);
+    k_block_ortho_df<2, 256, 3, 8><<<grid, 256, 0, st>>>(vecs, qdf, Vf, nc, bvol, nvec, fine, err, in32, out32, only);
   else if (nelem <= 512 * 3)
-    k_block_ortho_df2<3, 512, 2, 2><<<grid, 512, 0, st>>>(vecs, qdf, Vf, nc, bvol, nvec, fine, err, in32, out32);
+    k_block_ortho_df2<3, 512, 2, 2><<<grid, 512, 0, st>>>(vecs, qdf, Vf, nc, bvol, nvec, fine, err, in32, out32, only);
   else
-    k_block_ortho_df<8, 256, 3, 8><<<grid, 256, 0, st>>>(vecs, qdf, Vf, nc, bvol, nvec, fine, err, in32, out32);
+    k_block_ortho_df<8, 256, 3, 8><<<grid, 256, 0, st>>>(vecs, qdf, Vf, nc, bvol, nvec, fine, err, in32, out32, only);
   WCMG_LAUNCH_CHECK();
 }
 

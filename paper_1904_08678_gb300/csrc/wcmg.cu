@@ -237,6 +237,8 @@ struct wcmg_ctx {
   DevBuf<double> mr_pp;
   DevBuf<unsigned char> stage[3];
   DevBuf<int> errflag;
+  DevBuf<double2> cqW;       // Cholesky QR: the inverse factor of each (aggregate, chirality) panel
+  DevBuf<int> cqFlag;        // panels left to Gram-Schmidt, then their number
   DevBuf<int> tma_err;       // nonzero after a bounded device-side wait gave up
   int* h_flags = nullptr;   // pinned host mirror of per-rhs flags
   double* h_vals = nullptr; // pinned host mirror of per-rhs values
@@ -1448,10 +1450,20 @@ static void ortho_level(wcmg_ctx* c, int l, const float2* in32 = nullptr, float2
   // algorithmic work: one Gram-Schmidt pass, nvec (nvec - 1) complex MAC per panel row
   // (dots + updates); a second pass, when the cancellation test asks for it, is extra.
   if (c->p.ortho_df) {
-    float4* qdf = reinterpret_cast<float4*>(ws<double>(L, "ortho_qdf", L.nvec));
+    // Cholesky QR; what it flags (none on near-null candidates) goes to the Gram-Schmidt
+    // kernel, whose double-float copy of Q is allocated only then
+    const int panels = 2 * (L.g.V / L.g.bvol);
+    c->cqW.ensure((size_t)panels * L.nvec * L.nvec);
+    c->cqFlag.ensure((size_t)panels + 1);
+    WCMG_CUDA(cudaMemsetAsync(c->cqFlag.p + panels, 0, sizeof(int), c->st));
     KPROF(c, WCMG_K_ORTHO, 2.0 * n * 16.0, 8.0 * n * (L.nvec - 1),
-          launch_block_ortho_df(L.v64.p, qdf, L.g.V, L.nc, L.g.bvol, L.nvec, L.fine, c->errflag.p, c->st, in32,
-                                out32));
+          launch_cholqr(L.v64.p, c->cqW.p, c->cqFlag.p, c->cqFlag.p + panels, L.g.V, L.nc, L.g.bvol, L.nvec, L.fine,
+                        c->st, in32, out32));
+    if (!read_ints(c, c->cqFlag.p + panels, 1)[0]) return;
+    float4* qdf = reinterpret_cast<float4*>(ws<double>(L, "ortho_qdf", L.nvec));
+    KPROF(c, WCMG_K_ORTHO, 0.0, 0.0,
+          launch_block_ortho_df(L.v64.p, qdf, L.g.V, L.nc, L.g.bvol, L.nvec, L.fine, c->errflag.p, c->st, c->cqFlag.p,
+                                in32, out32));
   } else {
     KPROF(c, WCMG_K_ORTHO, 2.0 * n * 16.0, 8.0 * n * (L.nvec - 1),
           launch_block_ortho(L.v64.p, L.g.V, L.nc, L.g.bvol, L.nvec, L.fine, c->errflag.p, c->st));
@@ -2386,22 +2398,13 @@ int wcmg_set_nullvecs(wcmg_ctx* c, int level, const void* vecs, int where, void*
   Level& L = c->L[level];
   const size_t bytes = (size_t)L.nvec * L.n() * 16;
   const double2* v = in_dev(c, vecs, bytes, where, 0);
-  if (inner64(c)) {
-    L.raw64.ensure((size_t)L.nvec * L.n());
-    pack_level<double>(c, level, L.raw64.p, v, L.nvec);
-    build_P<double>(c, level);
-  } else {
-    L.raw32.ensure((size_t)L.nvec * L.n());
-    L.raw64.ensure((size_t)L.nvec * L.n());
-    pack_level<double>(c, level, L.raw64.p, v, L.nvec);
-    // orthonormalise from the FP64 input directly
-    L.v64.ensure((size_t)L.nvec * L.n());
-    copy_fields<double>(c, L.v64.p, L.raw64.p, (long long)L.nvec * L.n());
-    ortho_level(c, level);
-    launch_convert<double, float>(L.raw32.p, L.raw64.p, (long long)L.nvec * L.n(), c->st);
-    L.v32_valid = false;
-    L.have_P = true;
-  }
+  // orthonormalised in place from the FP64 input (the set-up's own raw vectors start from the
+  // vectors it is given, never from these)
+  L.v64.ensure((size_t)L.nvec * L.n());
+  pack_level<double>(c, level, L.v64.p, v, L.nvec);
+  ortho_level(c, level);
+  L.v32_valid = false;
+  L.have_P = true;
   WCMG_CUDA(cudaStreamSynchronize(c->st));
   c->prof.flush();
   API_END(c)

@@ -1,0 +1,73 @@
+"""Double-float block orthonormalisation: Cholesky QR and the panels it leaves to Gram-Schmidt."""
+import numpy as np
+import pytest
+
+from paper_1904_08678_gb300 import inputs
+from tests.gpu_util import dev, host, rel
+
+pytestmark = pytest.mark.gpu
+
+
+def q_factor(dims, block, nvec, vecs, df, level=0):
+    from paper_1904_08678_gb300 import wcmg
+    if level == 0:
+        p = wcmg.default_params(dims=dims, blocks=[block], nvec=[nvec], ortho_df=df)
+    else:  # a coarse level of `dims` sites with 6 components
+        fine = [2 * d for d in dims]
+        p = wcmg.default_params(dims=fine, n_levels=3, blocks=[(2, 2, 2, 2), block], nvec=[3, nvec], ortho_df=df)
+    ctx = wcmg.Context(p)
+    ctx.set_nullvecs(level, dev(vecs))
+    out = dev(np.full(vecs.shape, np.nan, dtype=complex))
+    ctx.get_nullvecs(level, out)
+    return host(out)
+
+
+# column counts around the 3 x 3 blocks and the groups of 4; panels of less than one tile,
+# a ragged last tile, 1536 and 2048 rows
+CASES = [((2, 4, 2, 2), (1, 2, 1, 1), 1), ((4, 2, 2, 2), (2, 1, 1, 1), 2), ((2, 2, 3, 3), (2, 2, 3, 3), 3),
+         ((4, 4, 4, 4), (2, 2, 2, 2), 4), ((6, 3, 3, 3), (3, 3, 3, 3), 23), ((4, 4, 4, 8), (4, 4, 4, 4), 24),
+         ((4, 4, 4, 4), (4, 4, 4, 2), 25), ((4, 4, 4, 5), (4, 4, 4, 5), 32)]
+
+
+@pytest.mark.parametrize("dims,block,nvec", CASES)
+def test_same_factor_as_fp64_gram_schmidt(dims, block, nvec):
+    """The positive-diagonal Q factor is unique; both agree to a few hundred units of 2^-48."""
+    v = inputs.complex_gaussian(31, nvec, (nvec, int(np.prod(dims)), 4, 3))
+    v[nvec // 2:] += 0.5 * v[0]
+    assert rel(q_factor(dims, block, nvec, v, 1), q_factor(dims, block, nvec, v, 0)) < 1e-12
+
+
+def test_coarse_level_layout():
+    dims, block, nvec = (4, 2, 4, 6), (2, 2, 2, 3), 5
+    v = inputs.complex_gaussian(32, 1, (nvec, int(np.prod(dims)), 6))
+    assert rel(q_factor(dims, block, nvec, v, 1, level=1), q_factor(dims, block, nvec, v, 0, level=1)) < 1e-12
+
+
+def test_ill_conditioned_aggregate_among_good_ones():
+    """One aggregate's columns nearly parallel (condition 1e4 and more): its panels go to
+    Gram-Schmidt (error condition x 1e-14, columns orthonormal), its neighbours do not."""
+    dims, block, nvec = (4, 4, 4, 4), (2, 2, 2, 2), 6
+    v = inputs.complex_gaussian(33, 1, (nvec, 4, 4, 4, 4, 4, 3))
+    bad = (slice(None), slice(0, 2), slice(2, 4), slice(0, 2), slice(2, 4))
+    w = v[bad]
+    v[bad] = w[:1] + 1e-4 * w
+    v = v.reshape(nvec, 256, 4, 3)
+    a, b = q_factor(dims, block, nvec, v, 1), q_factor(dims, block, nvec, v, 0)
+    a, b = (q.reshape((nvec, 4, 4, 4, 4, 4, 3)) for q in (a, b))
+    assert rel(a[bad], b[bad]) < 1e-9
+    panel = a[bad].reshape(nvec, -1, 4, 3)
+    for s in (slice(0, 2), slice(2, 4)):
+        q = panel[:, :, s].reshape(nvec, -1)
+        assert np.abs(q.conj() @ q.T - np.eye(nvec)).max() < 1e-13
+    a[bad], b[bad] = 0, 0
+    assert rel(a, b) < 1e-12
+
+
+def test_rank_deficient_aggregate_is_refused():
+    from paper_1904_08678_gb300 import wcmg
+    v = inputs.complex_gaussian(34, 1, (3, 256, 4, 3))
+    v[2] = 0
+    ctx = wcmg.Context(wcmg.default_params(dims=(4, 4, 4, 4), blocks=[(2, 2, 2, 2)], nvec=[3], ortho_df=1))
+    with pytest.raises(wcmg.WcmgError) as e:
+        ctx.set_nullvecs(0, dev(v))
+    assert e.value.code == wcmg.ERR_NAN
