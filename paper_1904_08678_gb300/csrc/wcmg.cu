@@ -1188,12 +1188,15 @@ static void sap(wcmg_ctx* c, int l, cplx<R>* x, const cplx<R>* b, int nrhs, int 
 constexpr int PTC_NW1 = WCMG_PTC_HIDDEN * 1 * 9 * 16;
 constexpr int PTC_NW2 = 1 * WCMG_PTC_HIDDEN * 9 * 16;
 
-static void ptc_layer_fwd(wcmg_ctx* c, float2* out, const float2* in, const float2* W, int nin, int nout, int nrhs) {
+// One network layer over nrhs samples: expanding (1 -> 12 fields) or contracting (12 -> 1);
+// adj: the other one's backward pass with respect to its input.
+static void ptc_layer(wcmg_ctx* c, bool expand, bool adj, float2* out, const float2* in, const float2* W, int nrhs) {
   Level& L = c->L[0];
   const double V = L.g.V;
-  KPROF(c, WCMG_K_PTC, V * 96.0 * (nin + nout) * nrhs + 8.0 * V * 72.0 * 4,
-        V * 8.0 * (double)nin * nout * 9 * (48 + 36) * nrhs,
-        launch_ptc_forward(out, in, W, c->gauge32.p, L.g.d_nbr.p, L.g.V, nin, nout, nrhs, c->st));
+  const int H = WCMG_PTC_HIDDEN;
+  KPROF(c, WCMG_K_PTC, V * 96.0 * (H + 1) * nrhs + 8.0 * V * 72.0 * 4, V * 8.0 * 9 * (H * 48.0 + 36.0) * nrhs,
+        (expand ? launch_ptc_expand : launch_ptc_contract)(out, in, W, c->gauge32.p, L.g.d_nbr.p, L.g.V, H, nrhs, adj,
+                                                           c->st));
 }
 
 // out = N(in), FP32, nrhs fields in the internal fine layout
@@ -1201,8 +1204,8 @@ static void ptc_forward(wcmg_ctx* c, float2* out, const float2* in, int nrhs) {
   if (!c->have_ptc) throw Error(WCMG_ERR_STATE, "PTC weights not set");
   if (!c->have_gauge) throw Error(WCMG_ERR_STATE, "gauge field not set");
   float2* hid = ws<float>(c->L[0], "ptc_hid", (long long)WCMG_PTC_HIDDEN * nrhs);
-  ptc_layer_fwd(c, hid, in, c->ptcW.p, 1, WCMG_PTC_HIDDEN, nrhs);
-  ptc_layer_fwd(c, out, hid, c->ptcW.p + PTC_NW1, WCMG_PTC_HIDDEN, 1, nrhs);
+  ptc_layer(c, true, false, hid, in, c->ptcW.p, nrhs);
+  ptc_layer(c, false, false, out, hid, c->ptcW.p + PTC_NW1, nrhs);
 }
 
 // Gradients dL/d conj(W) into ptcG (summed over the fields) and, if gin is not
@@ -1212,19 +1215,16 @@ static void ptc_backward(wcmg_ctx* c, const float2* in, const float2* gout, floa
   const int V = L.g.V, H = WCMG_PTC_HIDDEN;
   float2* hid = ws<float>(L, "ptc_hid", (long long)H * nrhs);
   float2* ghid = ws<float>(L, "ptc_ghid", (long long)H * nrhs);
-  ptc_layer_fwd(c, hid, in, c->ptcW.p, 1, H, nrhs);
-  c->ptcPartial.ensure((size_t)std::max(ptc_wgrad_partial_size(V, H, 1, nrhs), ptc_wgrad_partial_size(V, 1, H, nrhs)));
-  const double flops = (double)V * 8.0 * H * 9 * (48 + 36) * nrhs;
+  ptc_layer(c, true, false, hid, in, c->ptcW.p, nrhs);
+  c->ptcPartial.ensure((size_t)ptc_wgrad_partial_size(V, H, nrhs));
+  const double flops = (double)V * 8.0 * 9 * (H * 48.0 + 36.0) * nrhs;
   KPROF(c, WCMG_K_PTC, (double)V * 96.0 * (H + 1) * nrhs, flops,
-        launch_ptc_wgrad(c->ptcG.p + PTC_NW1, c->ptcPartial.p, gout, hid, c->gauge32.p, L.g.d_nbr.p, V, H, 1, nrhs,
+        launch_ptc_wgrad(c->ptcG.p + PTC_NW1, c->ptcPartial.p, hid, gout, c->gauge32.p, L.g.d_nbr.p, V, H, nrhs, true,
                          c->st));
+  ptc_layer(c, true, true, ghid, gout, c->ptcW.p + PTC_NW1, nrhs);
   KPROF(c, WCMG_K_PTC, (double)V * 96.0 * (H + 1) * nrhs, flops,
-        launch_ptc_backward_data(ghid, gout, c->ptcW.p + PTC_NW1, c->gauge32.p, L.g.d_nbr.p, V, H, 1, nrhs, c->st));
-  KPROF(c, WCMG_K_PTC, (double)V * 96.0 * (H + 1) * nrhs, flops,
-        launch_ptc_wgrad(c->ptcG.p, c->ptcPartial.p, ghid, in, c->gauge32.p, L.g.d_nbr.p, V, 1, H, nrhs, c->st));
-  if (gin)
-    KPROF(c, WCMG_K_PTC, (double)V * 96.0 * (H + 1) * nrhs, flops,
-          launch_ptc_backward_data(gin, ghid, c->ptcW.p, c->gauge32.p, L.g.d_nbr.p, V, 1, H, nrhs, c->st));
+        launch_ptc_wgrad(c->ptcG.p, c->ptcPartial.p, ghid, in, c->gauge32.p, L.g.d_nbr.p, V, H, nrhs, false, c->st));
+  if (gin) ptc_layer(c, false, true, gin, ghid, c->ptcW.p, nrhs);
 }
 
 static void ptc_alloc(wcmg_ctx* c) {
