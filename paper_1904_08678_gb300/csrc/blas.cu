@@ -658,18 +658,33 @@ __global__ void k_gmres_step(GmresState S, int j, const double2* __restrict__ h,
 // the sweep of <V_i, w> and <V_i, V_j> (the newest column of the Gram matrix), the
 // coefficients h + (h - G h) of both Gram-Schmidt passes, w - V h, its norm, the Givens
 // update of Hessenberg column j and V_{j+1} = w / ||w||.  CTA c of the C-CTA cluster owns
-// a contiguous range of the vector.  Bound by latency, so: one warp per basis vector in
-// the sweep (warp sums only, no block barrier per chunk of vectors), the updated elements
-// stay in registers until the norm is known, everything the coefficients and the rotation
-// need (G, cs, sn, g) is requested before the sweep, and the rotation runs from shared
-// memory while the cluster writes V_{j+1}.  Partial sums are exchanged through distributed
+// a contiguous range of the vector.  Bound by latency, so: the warps share the basis vectors
+// of the sweep evenly (warp sums only, no block barrier per chunk of vectors), the updated
+// elements stay in registers until the norm is known, everything the coefficients and the
+// rotation need (G, cs, sn) is requested before the sweep, remote sums are read all at once,
+// FP64 work is left to as few warps as it has values (a warp's FP64 instruction takes 16
+// cycles of the SM's unit), and the rotation runs from shared memory while the cluster writes
+// V_{j+1}.  Partial sums are exchanged through distributed
 // shared memory and every CTA adds the C partials in the same order, so all CTAs hold
-// identical coefficients.  24.6k entries, 16 CTAs: 34 us before (two sweeps and two updates,
-// four cluster barriers, the rotation from global memory).
+// identical coefficients.  24.6k entries, 16 CTAs, in a solve under ncu: 36 us with one warp
+// per basis vector and every thread adding the remote norms in FP64, 22 us now.
 constexpr int AC_T = 512, AC_MAXK = 65, AC_W = AC_T / 32;
-constexpr int AC_EL = 16;  // elements per thread: n <= 2^17 over at least 8 CTAs ... 16 x 512 each
+constexpr int AC_EL = 16;  // most elements per thread
 
-template <typename R>
+// sum over the cluster's ranks of one shared double2, all remote reads in flight
+__device__ __forceinline__ double2 ac_cluster_sum(cooperative_groups::cluster_group& cl, double2* p, int C) {
+  double2 v[16];
+#pragma unroll
+  for (int c = 0; c < 16; ++c) v[c] = c < C ? *cl.map_shared_rank(p, c) : make_double2(0, 0);
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1)
+#pragma unroll
+    for (int c = 0; c < o; ++c) v[c] += v[c + o];
+  return v[0];
+}
+
+// NE: elements per thread (power of two; the vector has at most C x AC_T x NE entries)
+template <typename R, int NE>
 __global__ void __launch_bounds__(AC_T) k_arnoldi_cluster(cplx<R>* __restrict__ Vb, long long bstride,
                                                           const cplx<R>* __restrict__ w, long long n, GmresState S,
                                                           double2* __restrict__ G, int j, const int* __restrict__ jdev,
@@ -678,20 +693,22 @@ __global__ void __launch_bounds__(AC_T) k_arnoldi_cluster(cplx<R>* __restrict__ 
   cg::cluster_group cl = cg::this_cluster();
   const int C = (int)cl.num_blocks(), crank = (int)cl.block_rank();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  __shared__ double2 pA[AC_MAXK], pV[AC_MAXK];  // this CTA's partial sums (read by the whole cluster)
-  __shared__ double pN;
-  __shared__ double2 hs[AC_MAXK], gs[AC_MAXK], hcol[AC_MAXK];
+  __shared__ double2 pA[2 * AC_MAXK];  // this CTA's sums <V_i, w>, then <V_i, V_j> (read by the whole cluster)
+  __shared__ cplx<R> pw[AC_W][2];      // per warp, when several warps share a basis vector
+  __shared__ double2 pN;
+  __shared__ double2 hs[2 * AC_MAXK], hcol[AC_MAXK];
   __shared__ cplx<R> cf[AC_MAXK];
   __shared__ double csn[AC_MAXK];
   __shared__ double2 snn[AC_MAXK];
-  __shared__ double dscr[AC_W];
-  __shared__ double dred[1];
+  __shared__ R wsum[AC_W];
+  __shared__ double hn_s;
+  __shared__ R inv_s;
   if (jdev) j = *jdev;
   const int k = j + 1, m = S.m, ld = m + 1;
   const bool act = S.active[0] != 0;  // before this step (CTA 0 may change it below)
   const int per = (int)((n + C - 1) / C);
   const int e0 = crank * per, cnt = max(0, min(per, (int)n - e0));
-  // row i of G without its newest entry: 8 lanes per row
+  // row gi of G without its newest entry: 8 lanes per row
   const int gi = threadIdx.x >> 3, gl = threadIdx.x & 7;
   double2 gr[8];
 #pragma unroll
@@ -704,36 +721,46 @@ __global__ void __launch_bounds__(AC_T) k_arnoldi_cluster(cplx<R>* __restrict__ 
       csn[i] = S.cs[i];
       snn[i] = S.sn[i];
     }
-  // sweep: <V_i, w> and <V_i, V_j>, one warp per i
+  // sweep: <V_i, w> and <V_i, V_j>; the 16 warps split into one group of P per basis vector
+  // (P = 16, 8, .. 1: as many as there are vectors for), each warp a P-th of the range
   const cplx<R>* wv = w + e0;
   const cplx<R>* vj = Vb + (long long)j * bstride + e0;
-  for (int i = warp; i < k; i += AC_W) {
+  const int P = k == 1 ? 16 : k == 2 ? 8 : k <= 4 ? 4 : k <= 8 ? 2 : 1;
+  for (int i = warp / P; i < k; i += AC_W / P) {
     const cplx<R>* vi = Vb + (long long)i * bstride + e0;
     cplx<R> aw = czero<R>(), av = czero<R>();
 #pragma unroll 8
-    for (int e = lane; e < cnt; e += 32) {
+    for (int e = lane + 32 * (warp % P); e < cnt; e += 32 * P) {
       const cplx<R> v = vi[e];
       cjmac(aw, v, wv[e]);
       cjmac(av, v, vj[e]);
     }
     const cplx<R> tw = warp_sum(aw), tv = warp_sum(av);
     if (lane == 0) {
-      pA[i] = to_c64(tw);
-      pV[i] = to_c64(tv);
+      if (P == 1) {
+        pA[i] = to_c64(tw);
+        pA[k + i] = to_c64(tv);
+      } else {
+        pw[warp][0] = tw;
+        pw[warp][1] = tv;
+      }
+    }
+  }
+  if (P > 1) {
+    __syncthreads();
+    if (threadIdx.x < 2 * k) {
+      const int i = threadIdx.x % k, z = threadIdx.x / k;
+      double2 t = to_c64(pw[i * P][z]);
+      for (int u = 1; u < P; ++u) t += to_c64(pw[i * P + u][z]);
+      pA[threadIdx.x] = t;
     }
   }
   cl.sync();
-  for (int i = threadIdx.x; i < 2 * k; i += AC_T) {
-    const bool second = i >= k;
-    const int q = second ? i - k : i;
-    double2 t = make_double2(0, 0);
-#pragma unroll 8
-    for (int c = 0; c < C; ++c) t += cl.map_shared_rank(second ? pV : pA, c)[q];
-    (second ? gs : hs)[q] = t;
-  }
+  if (threadIdx.x < 2 * k) hs[threadIdx.x] = ac_cluster_sum(cl, pA + threadIdx.x, C);
   __syncthreads();
+  const double2* gs = hs + k;
   // h + (h - G h), G's newest column gs: G_{l j} = gs_l, G_{j l} = conj(gs_l)
-  {
+  if (gi < (k + 3) / 4 * 4) {  // whole warps
     double2 t = make_double2(0, 0);
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
@@ -757,37 +784,50 @@ __global__ void __launch_bounds__(AC_T) k_arnoldi_cluster(cplx<R>* __restrict__ 
     }
   }
   __syncthreads();
-  // w - V h in registers, and its norm
-  cplx<R> x[AC_EL];
-  R nn = 0;
+  // w - V h in registers (all of a thread's elements per basis vector: loads in flight),
+  // and its norm: warp sums in R, the warps' in FP64
+  cplx<R> x[NE];
 #pragma unroll
-  for (int u = 0; u < AC_EL; ++u) {
+  for (int u = 0; u < NE; ++u) {
     const int e = threadIdx.x + u * AC_T;
-    if (e < cnt) {
-      cplx<R> t = wv[e];
-      const cplx<R>* v = Vb + e0 + e;
-#pragma unroll 8
-      for (int i = 0; i < k; ++i) cnmac(t, cf[i], v[i * bstride]);
-      x[u] = t;
-      nn += cnorm2(t);
+    x[u] = e < cnt ? wv[e] : czero<R>();
+  }
+  constexpr int UI = NE >= 8 ? 1 : 8 / NE;
+#pragma unroll UI
+  for (int i = 0; i < k; ++i) {
+    const cplx<R>* v = Vb + (long long)i * bstride + e0;
+    const cplx<R> c = cf[i];
+#pragma unroll
+    for (int u = 0; u < NE; ++u) {
+      const int e = threadIdx.x + u * AC_T;
+      if (e < cnt) cnmac(x[u], c, v[e]);
     }
   }
-  {
-    const R v[1] = {nn};
-    block_sum_mixed<R, 1>(v, dscr, dred);
-    if (threadIdx.x == 0) pN = dred[0];
+  R nn = 0;
+#pragma unroll
+  for (int u = 0; u < NE; ++u) nn += cnorm2(x[u]);
+  nn = warp_sum(nn);
+  if (lane == 0) wsum[warp] = nn;
+  __syncthreads();
+  if (warp == 0) {
+    double t = lane < AC_W ? (double)wsum[lane] : 0.0;
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (lane == 0) pN = make_double2(t, 0);
   }
   cl.sync();
-  double hn2 = 0.0;
-#pragma unroll 8
-  for (int c = 0; c < C; ++c) hn2 += *cl.map_shared_rank(&pN, c);
+  if (threadIdx.x == 0) {  // one thread: FP64 runs at two lanes per cycle on an SM
+    const double hn2 = ac_cluster_sum(cl, &pN, C).x, h = sqrt(hn2);
+    hn_s = hn2;
+    inv_s = (R)(act && h > 0.0 ? 1.0 / h : 0.0);
+  }
+  __syncthreads();
   cl.barrier_arrive();  // done with the others' shared memory
-  if (crank == 0 && threadIdx.x == 0 && act) gmres_rotate(S, j, hcol, csn, snn, hn2, tol, final_done);
-  const double h = sqrt(hn2);
-  const R inv = (R)(act && h > 0.0 ? 1.0 / h : 0.0);
+  if (crank == 0 && threadIdx.x == AC_T - 32 && act) gmres_rotate(S, j, hcol, csn, snn, hn_s, tol, final_done);
+  const R inv = inv_s;
   cplx<R>* vn = Vb + (long long)(j + 1) * bstride + e0;
 #pragma unroll
-  for (int u = 0; u < AC_EL; ++u) {
+  for (int u = 0; u < NE; ++u) {
     const int e = threadIdx.x + u * AC_T;
     if (e < cnt) {
       const cplx<R> t = inv * x[u];
@@ -803,7 +843,7 @@ static int arnoldi_cluster_size() {
   if (cached >= 0) return cached;
   cached = 0;
   for (int C : {16, 8}) {
-    auto kern = k_arnoldi_cluster<float>;
+    auto kern = k_arnoldi_cluster<float, AC_EL>;
     if (C > 8 && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
       cudaGetLastError();
       continue;
@@ -842,7 +882,12 @@ void launch_arnoldi_fused(cplx<R>* Vb, long long bstride, cplx<R>* w, long long 
                           int j, const int* jdev, double tol, int final_done, cudaStream_t st, cplx<R>* vnext) {
   const int C = arnoldi_cluster_size();
   if (C <= 0) throw Error(-1, "no thread-block cluster available for the fused Arnoldi step");
-  auto kern = k_arnoldi_cluster<R>;
+  const long long per = ((n + C - 1) / C + AC_T - 1) / AC_T;  // elements per thread
+  auto kern = per <= 1   ? k_arnoldi_cluster<R, 1>
+              : per <= 2 ? k_arnoldi_cluster<R, 2>
+              : per <= 4 ? k_arnoldi_cluster<R, 4>
+              : per <= 8 ? k_arnoldi_cluster<R, 8>
+                         : k_arnoldi_cluster<R, AC_EL>;
   if (C > 8) WCMG_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(C);
