@@ -468,8 +468,10 @@ __device__ __forceinline__ bool on_face(const BlockInfo& bi, int s, int d) {
   return (d & 1) ? (l[mu] == 0) : (l[mu] == bi.b[mu] - 1);
 }
 
-// RSD: the result is the residual rsd - D in, formed in the epilogue (a pass of its own
-// would read the product and write it once more).
+// RSD: the result is the residual rsd - D in (a pass of its own would read the product and
+// write it once more).  In FP32 the hop sums start from 2 rsd and the result is negated, so
+// that rsd's loads overlap the first hop's; in the epilogue, where FP64 keeps them, they were
+// exposed (two rhs per thread, 12 rhs on 24^3x48: 984 us, now 820 us; without rsd 683 us).
 // MR epilogue (DOTS): the CTA also sums <out, in> = sum conj(out) in and <out, out>
 // over its sites (FP32/FP64 per thread, FP64 across the CTA) into one partial per
 // (rhs, CTA): the minimal-residual step p = D r, alpha = <p, r>/<p, p> then needs
@@ -508,7 +510,8 @@ __global__ void __launch_bounds__(128, (sizeof(R) == 4 && NR == 1) ? 6 : (sizeof
 #pragma unroll
     for (int q = 0; q < NR; ++q)
 #pragma unroll
-      for (int c = 0; c < 12; ++c) acc[q][c] = czero<R>();
+      for (int c = 0; c < 12; ++c)
+        acc[q][c] = RSD && sizeof(R) == 4 ? R(2) * rsd[off + q * rs + (long long)c * V + s] : czero<R>();
     auto use = [&](int d) -> bool {
       if (MODE == ST_FULL) return true;
       if (MODE == ST_BLOCK_INTERIOR) return !on_face(bi, s, d);
@@ -557,7 +560,7 @@ __global__ void __launch_bounds__(128, (sizeof(R) == 4 && NR == 1) ? 6 : (sizeof
 #pragma unroll
           for (int i = 0; i < 6; ++i) {
             const long long a = (long long)(6 * h + i) * V + s;
-            oq[a] = RSD ? bq[a] - acc[q][6 * h + i] : acc[q][6 * h + i];
+            oq[a] = !RSD ? acc[q][6 * h + i] : sizeof(R) == 4 ? -acc[q][6 * h + i] : bq[a] - acc[q][6 * h + i];
           }
         }
     }
