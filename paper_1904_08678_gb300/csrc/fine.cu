@@ -585,6 +585,93 @@ __global__ void __launch_bounds__(128, (sizeof(R) == 4 && NR == 1) ? 6 : (sizeof
   }
 }
 
+// The full FP64 stencil on a small lattice: one CTA per 32 sites and rhs, one warp per direction
+// (both hops), whose sums meet in shared memory; warp h then finishes chirality half h.  An
+// SM retires one FP64 instruction of a warp in 16 cycles, so 32 sites are 10 us of its time
+// however they are cut; with one warp per 32 sites that time and the ten load latencies
+// of a site lie in a row on the few SMs that have a warp.  8^3x16: 44 us before, 27 us now.
+// Taken up to DS64_SITES sites x rhs (six CTAs per SM): a whole apply of 27,648 sites 92 against
+// 78 us, of 36,864 sites 92 against 102 us, where k_dslash's own warps fill the SMs.
+constexpr long long DS64_SITES = 152 * 32 * 6;
+template <int MU>
+__device__ __forceinline__ void hop_pair(double2 (&acc)[1][12], const double2* __restrict__ in,
+                                         const double2* __restrict__ U, const int* __restrict__ nbr, int V, int s) {
+  hop<double, MU, true, 1>(acc, in, 0, U, V, s, nbr[(2 * MU) * V + s]);
+  hop<double, MU, false, 1>(acc, in, 0, U, V, s, nbr[(2 * MU + 1) * V + s]);
+}
+template <bool DOTS, bool RSD>
+__global__ void __launch_bounds__(128) k_dslash_split(double2* __restrict__ out, const double2* __restrict__ in,
+                                                      const double2* __restrict__ U, const double2* __restrict__ clov,
+                                                      const int* __restrict__ nbr, int V, int nrhs,
+                                                      double2* __restrict__ pr_part, double* __restrict__ pp_part,
+                                                      const double2* __restrict__ rsd) {
+  __shared__ double2 part[4][12][32];
+  __shared__ double dots[2][3];
+  const int r = blockIdx.x % nrhs, sb = blockIdx.x / nrhs, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int s = sb * 32 + lane;
+  const bool valid = s < V;
+  const long long off = (long long)r * 12 * V;
+  in += off;
+  double2 acc[1][12];
+#pragma unroll
+  for (int c = 0; c < 12; ++c) acc[0][c] = make_double2(0, 0);
+  if (valid) {
+    if (warp == 0) hop_pair<0>(acc, in, U, nbr, V, s);
+    else if (warp == 1) hop_pair<1>(acc, in, U, nbr, V, s);
+    else if (warp == 2) hop_pair<2>(acc, in, U, nbr, V, s);
+    else hop_pair<3>(acc, in, U, nbr, V, s);
+  }
+#pragma unroll
+  for (int c = 0; c < 12; ++c) part[warp][c][lane] = acc[0][c];
+  __syncthreads();
+  if (warp < 2) {
+    const int h = warp;
+    double dr = 0, di = 0, nn = 0;
+    if (valid) {
+      double2 p[1][6];
+#pragma unroll
+      for (int i = 0; i < 6; ++i) {
+        p[0][i] = in[(long long)(6 * h + i) * V + s];
+        const int c = 6 * h + i;
+        const double2 t = (part[0][c][lane] + part[1][c][lane]) + (part[2][c][lane] + part[3][c][lane]);
+        if (h == 0) acc[0][i] = t;
+        else acc[0][6 + i] = t;
+      }
+      if (h == 0) clover_half<double, 1>(acc, clov, p, 0, V, s);
+      else clover_half<double, 1>(acc, clov, p, 1, V, s);
+#pragma unroll
+      for (int i = 0; i < 6; ++i) {
+        const double2 o = h == 0 ? acc[0][i] : acc[0][6 + i];
+        if (DOTS) {
+          dr += o.x * p[0][i].x + o.y * p[0][i].y;
+          di += o.x * p[0][i].y - o.y * p[0][i].x;
+          nn += o.x * o.x + o.y * o.y;
+        }
+        const long long a = off + (long long)(6 * h + i) * V + s;
+        if (!DOTS || out) out[a] = RSD ? rsd[a] - o : o;
+      }
+    }
+    if (DOTS) {
+      dr = warp_sum(dr);
+      di = warp_sum(di);
+      nn = warp_sum(nn);
+      if (lane == 0) {
+        dots[h][0] = dr;
+        dots[h][1] = di;
+        dots[h][2] = nn;
+      }
+    }
+  }
+  if (DOTS) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      const int nsb = gridDim.x / nrhs;
+      pr_part[(long long)r * nsb + sb] = make_double2(dots[0][0] + dots[1][0], dots[0][1] + dots[1][1]);
+      pp_part[(long long)r * nsb + sb] = dots[0][2] + dots[1][2];
+    }
+  }
+}
+
 // rhs per thread: 2 for FP32 with several rhs, else 1
 template <typename R>
 static int dslash_nr(int nrhs) { return (sizeof(R) == 4 && nrhs > 1) ? 2 : 1; }
@@ -594,6 +681,19 @@ void launch_dslash(cplx<R>* out, const cplx<R>* in, const cplx<R>* gauge, const 
                    int nrhs, int mode, int hopdir, cudaStream_t st, const unsigned char* colour, int col,
                    const cplx<R>* rsd) {
   if (rsd && mode != ST_FULL) throw Error(-1, "residual epilogue: full stencil only");
+  if constexpr (sizeof(R) == 8) {
+    if (mode == ST_FULL && !colour && (long long)g.V * nrhs <= DS64_SITES) {
+      const unsigned grid = nblk(g.V, 32) * nrhs;
+      if (rsd)
+        k_dslash_split<false, true>
+            <<<grid, 128, 0, st>>>(out, in, gauge, clov, g.nbr, g.V, nrhs, nullptr, nullptr, rsd);
+      else
+        k_dslash_split<false, false>
+            <<<grid, 128, 0, st>>>(out, in, gauge, clov, g.nbr, g.V, nrhs, nullptr, nullptr, nullptr);
+      WCMG_LAUNCH_CHECK();
+      return;
+    }
+  }
   BlockInfo bi;
   for (int k = 0; k < 4; ++k) bi.b[k] = g.b[k];
   bi.bvol = g.bvol;
@@ -1209,7 +1309,7 @@ __global__ void __launch_bounds__(256) k_mr_final(double2* __restrict__ pr, doub
   }
 }
 
-int dslash_partials(int V) { return (int)nblk(V, 128); }
+int dslash_partials(int V) { return (int)nblk(V, 32); }  // the most: 32 sites each
 
 template <typename R>
 void launch_dslash_mr(cplx<R>* out, const cplx<R>* in, const cplx<R>* gauge, const cplx<R>* clov, const LevelGeom& g,
@@ -1217,7 +1317,18 @@ void launch_dslash_mr(cplx<R>* out, const cplx<R>* in, const cplx<R>* gauge, con
   BlockInfo bi;
   for (int k = 0; k < 4; ++k) bi.b[k] = g.b[k];
   bi.bvol = g.bvol;
-  const int nsb = dslash_partials(g.V);
+  if constexpr (sizeof(R) == 8) {
+    if ((long long)g.V * nrhs <= DS64_SITES) {
+      const int nsb = (int)nblk(g.V, 32);
+      k_dslash_split<true, false>
+          <<<nsb * nrhs, 128, 0, st>>>(out, in, gauge, clov, g.nbr, g.V, nrhs, pr_part, pp_part, nullptr);
+      WCMG_LAUNCH_CHECK();
+      k_mr_final<<<nrhs, 256, 0, st>>>(pr, pp, pr_part, pp_part, nsb);
+      WCMG_LAUNCH_CHECK();
+      return;
+    }
+  }
+  const int nsb = (int)nblk(g.V, 128);
   const int nr = dslash_nr<R>(nrhs);
   const unsigned grid = (unsigned)((long long)nsb * ((nrhs + nr - 1) / nr));
   bool done = false;
