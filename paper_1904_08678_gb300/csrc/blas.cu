@@ -287,8 +287,8 @@ __global__ void __launch_bounds__(AN_T) k_project_norm(cplx<R>* __restrict__ w, 
   if (threadIdx.x == 0) partial[(long long)r * gridDim.x + blockIdx.x] = red[0];
 }
 template <typename R>
-void launch_project_norm(double* norm2, cplx<R>* w, const cplx<R>* basis, long long bstride, int k, const double2* h,
-                         int ld, long long n, int nrhs, double* partial, cudaStream_t st, const int* kdev, int kadd) {
+int launch_project_norm(double* partial, cplx<R>* w, const cplx<R>* basis, long long bstride, int k, const double2* h,
+                        int ld, long long n, int nrhs, cudaStream_t st, const int* kdev, int kadd) {
   if (k > GC_T) throw Error(-1, "Gram-Schmidt supports k <= 96");
   const int vec2 = sizeof(R) == 4 && n % 2 == 0 && bstride % 2 == 0 && reinterpret_cast<uintptr_t>(basis) % 16 == 0 &&
                    reinterpret_cast<uintptr_t>(w) % 16 == 0;
@@ -296,8 +296,7 @@ void launch_project_norm(double* norm2, cplx<R>* w, const cplx<R>* basis, long l
   const int nb = (int)std::max(1LL, std::min(608LL, (n + per - 1) / per));
   k_project_norm<R><<<dim3(nb, nrhs), AN_T, 0, st>>>(w, basis, bstride, k, h, ld, n, partial, kdev, kadd, vec2);
   WCMG_LAUNCH_CHECK();
-  k_final<double><<<dim3(nrhs, 1), RED_T, 0, st>>>(norm2, partial, nb, nb, 0, 1);
-  WCMG_LAUNCH_CHECK();
+  return nb;
 }
 
 template <typename R>
@@ -529,16 +528,6 @@ void launch_copy_idx(cplx<R>* dst, const cplx<R>* src, long long n, const int* i
   k_copy_idx<R><<<nblk(n, 256), 256, 0, st>>>(dst, src, n, idx, dmul, smul);
   WCMG_LAUNCH_CHECK();
 }
-__global__ void k_fill_int(int* x, int v, int n) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) x[i] = v;
-}
-void launch_fill_int(int* x, int v, int n, cudaStream_t st) {
-  if (n <= 0) return;
-  k_fill_int<<<nblk(n, 256), 256, 0, st>>>(x, v, n);
-  WCMG_LAUNCH_CHECK();
-}
-
 template <typename R>
 __global__ void k_fill_zero(cplx<R>* x, long long n) {
   const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -564,59 +553,53 @@ __device__ void givens(double2 a, double2 b, double& c, double2& s, double2& rho
   rho = r * ph;
 }
 
+// init: the first cycle from x = 0, whose residual is b: also bnorm = beta and done = 0
 __global__ void k_gmres_start(GmresState S, const double* __restrict__ nrm2, double tol, int nrhs,
-                              double* __restrict__ inv_beta) {
+                              double* __restrict__ inv_beta, bool init) {
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= nrhs) return;
   const double beta = sqrt(nrm2[r]);
   const int m = S.m;
+  if (init) {
+    S.bnorm[r] = beta;
+    S.done[r] = 0;
+  }
   for (int i = 0; i <= m; ++i) S.g[(long long)r * (m + 1) + i] = make_double2(0, 0);
   S.g[(long long)r * (m + 1)] = make_double2(beta, 0);
   S.resid[r] = beta;
   S.jdone[r] = 0;
-  const bool go = !S.done[r] && beta > tol * S.bnorm[r] && beta > 0.0;
+  const bool go = (init || !S.done[r]) && beta > tol * S.bnorm[r] && beta > 0.0;
   S.active[r] = go ? 1 : 0;
   inv_beta[r] = go ? 1.0 / beta : 0.0;
 }
-
-// Column j of the Hessenberg matrix of rhs r: h_col[0..j] (both CGS passes summed)
-// and ||w||^2; the earlier rotations, a new complex Givens rotation and the
-// recurrence residual; returns 1 / ||w|| (0 if ||w|| = 0).
-__device__ double gmres_column(GmresState S, int r, int j, const double2* hcol, double hn2, double tol,
-                               int final_done) {
-  const int m = S.m;
-  double2* H = S.H + (long long)r * (m + 1) * m;
-  double* cs = S.cs + (long long)r * m;
-  double2* sn = S.sn + (long long)r * m;
-  double2* g = S.g + (long long)r * (m + 1);
-  for (int i = 0; i <= j; ++i) H[i * m + j] = hcol[i];
-  const double h = sqrt(hn2);
-  H[(j + 1) * m + j] = make_double2(h, 0);
-  for (int i = 0; i < j; ++i) {
-    const double2 a = H[i * m + j], b = H[(i + 1) * m + j];
-    H[i * m + j] = cs[i] * a + cmul(sn[i], b);
-    H[(i + 1) * m + j] = cs[i] * b - cmul(conjg(sn[i]), a);
-  }
-  double c; double2 s, rho;
-  givens(H[j * m + j], H[(j + 1) * m + j], c, s, rho);
-  cs[j] = c; sn[j] = s;
-  H[j * m + j] = rho;
-  H[(j + 1) * m + j] = make_double2(0, 0);
-  const double2 gj = g[j];
-  g[j + 1] = -cmul(conjg(s), gj);
-  g[j] = c * gj;
-  const double res = sqrt(cnorm2(g[j + 1]));
-  S.resid[r] = res;
-  S.jdone[r] = j + 1;
-  if (res <= tol * S.bnorm[r]) {
-    S.active[r] = 0;
-    if (final_done) S.done[r] = 1;
-  }
-  return h > 0.0 ? 1.0 / h : 0.0;
+// bnorm = sqrt(nrm2), done = 0 (before the restart loop)
+__global__ void k_gmres_init(GmresState S, const double* __restrict__ nrm2, int nrhs) {
+  const int r = blockIdx.x * blockDim.x + threadIdx.x;
+  if (r >= nrhs) return;
+  S.bnorm[r] = sqrt(nrm2[r]);
+  S.done[r] = 0;
 }
 
-// The same for one rhs (row 0 of the state) from shared copies: hcol [j + 1] is overwritten,
-// cs and sn hold the rotations of columns 0 .. j - 1.
+// the state of one rhs
+__device__ __forceinline__ GmresState gmres_of(GmresState S, int r) {
+  const long long m = S.m;
+  S.H += r * (m + 1) * m;
+  S.cs += r * m;
+  S.sn += r * m;
+  S.g += r * (m + 1);
+  S.y += r * m;
+  S.hnorm += r;
+  S.bnorm += r;
+  S.resid += r;
+  S.active += r;
+  S.jdone += r;
+  S.done += r;
+  return S;
+}
+
+// Column j of the Hessenberg matrix of one rhs: the earlier rotations on hcol (j + 1 entries,
+// overwritten; cs, sn: the rotations of columns 0 .. j - 1, all in shared memory), a new
+// complex Givens rotation that removes ||w|| = sqrt(hn2), and the recurrence residual.
 __device__ void gmres_rotate(GmresState S, int j, double2* hcol, const double* cs, const double2* sn, double hn2,
                              double tol, int final_done) {
   const int m = S.m;
@@ -642,14 +625,32 @@ __device__ void gmres_rotate(GmresState S, int j, double2* hcol, const double* c
   }
 }
 
-__global__ void k_gmres_step(GmresState S, int j, const double2* __restrict__ h, const double* __restrict__ hnorm2, double tol, int final_done, int nrhs,
-                             double* __restrict__ inv_h, const int* __restrict__ jdev) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= nrhs) return;
+// One CTA per rhs: ||w||^2 from the `count` partials of k_project_norm, then the rotation with
+// the column and the earlier rotations fetched in parallel (12 us; the rotation by one thread
+// from global memory took 12 us and the final sum another launch of 4 us).
+__global__ void __launch_bounds__(RED_T) k_gmres_step(GmresState S, int j, const double2* __restrict__ h,
+                                                      const double* __restrict__ partial, int count, double tol,
+                                                      int final_done, double* __restrict__ inv_h,
+                                                      const int* __restrict__ jdev) {
+  __shared__ double2 hcol[65], sn[65];
+  __shared__ double cs[65], scratch[RED_T / 32], red[1];
+  const int r = blockIdx.x;
   if (jdev) j = *jdev;
-  const int m = S.m;
-  if (!S.active[r]) { inv_h[r] = 0.0; return; }
-  inv_h[r] = gmres_column(S, r, j, h + (long long)r * (m + 1), hnorm2[r], tol, final_done);
+  S = gmres_of(S, r);
+  const bool act = S.active[0] != 0;
+  if (threadIdx.x <= j) hcol[threadIdx.x] = h[(long long)r * (S.m + 1) + threadIdx.x];
+  if (threadIdx.x < j) {
+    cs[threadIdx.x] = S.cs[threadIdx.x];
+    sn[threadIdx.x] = S.sn[threadIdx.x];
+  }
+  double acc = 0.0;
+  for (int b = threadIdx.x; b < count; b += RED_T) acc += partial[(long long)r * count + b];
+  block_sum_many<double>(&acc, 1, scratch, red);
+  if (threadIdx.x == 0) {
+    const double hn2 = red[0], nrm = sqrt(hn2);
+    inv_h[r] = act && nrm > 0.0 ? 1.0 / nrm : 0.0;
+    if (act) gmres_rotate(S, j, hcol, cs, sn, hn2, tol, final_done);
+  }
 }
 
 // ---- fused Arnoldi step for short vectors (one rhs) ----
@@ -908,21 +909,38 @@ template void launch_arnoldi_fused<float>(float2*, long long, float2*, long long
 template void launch_arnoldi_fused<double>(double2*, long long, double2*, long long, const GmresState&, double2*, int,
                                            const int*, double, int, cudaStream_t, double2*);
 
-__global__ void k_gmres_solve_y(GmresState S, int nrhs) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= nrhs) return;
-  const int m = S.m, jd = S.jdone[r];
-  const double2* H = S.H + (long long)r * (m + 1) * m;
-  const double2* g = S.g + (long long)r * (m + 1);
-  double2* y = S.y + (long long)r * m;
-  for (int i = m - 1; i >= jd; --i) y[i] = make_double2(0, 0);
-  for (int i = jd - 1; i >= 0; --i) {
-    double2 t = g[i];
-    for (int k = i + 1; k < jd; ++k) t -= cmul(H[i * m + k], y[k]);
-    const double2 d = H[i * m + i];
+// y = R^-1 g by columns, one warp per rhs: lane i holds the right-hand sides i and i + 32, R
+// (its columns from the diagonal up) lies in shared memory, and the diagonal's reciprocals
+// are formed at once (m = 20: 11 us with one thread walking through global memory, 8.6 us now).
+__global__ void __launch_bounds__(32) k_gmres_solve_y(GmresState S) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  double2* Rs = reinterpret_cast<double2*>(smem_raw);  // column k at k (k + 1) / 2
+  S = gmres_of(S, blockIdx.x);
+  const int m = S.m, jd = S.jdone[0], lane = threadIdx.x;
+  for (int k = 0; k < jd; ++k)
+    for (int i = lane; i <= k; i += 32) Rs[k * (k + 1) / 2 + i] = S.H[i * m + k];
+  double2 t[2];
+#pragma unroll
+  for (int u = 0; u < 2; ++u) t[u] = lane + 32 * u < jd ? S.g[lane + 32 * u] : make_double2(0, 0);
+  __syncwarp();
+  double2 inv[2];  // conj(d) / |d|^2, or 0
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const int k = lane + 32 * u;
+    const double2 d = k < jd ? Rs[k * (k + 1) / 2 + k] : make_double2(0, 0);
     const double dd = cnorm2(d);
-    y[i] = dd > 0.0 ? (1.0 / dd) * cjmul(d, t) : make_double2(0, 0);
+    inv[u] = dd > 0.0 ? (1.0 / dd) * conjg(d) : make_double2(0, 0);
   }
+  for (int k = jd - 1; k >= 0; --k) {
+    const double2* col = Rs + k * (k + 1) / 2;
+    double2 y = k < 32 ? cmul(inv[0], t[0]) : cmul(inv[1], t[1]);
+    y = make_double2(__shfl_sync(0xffffffffu, y.x, k & 31), __shfl_sync(0xffffffffu, y.y, k & 31));
+    if (lane == 0) S.y[k] = y;
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+      if (lane + 32 * u < k) cnmac(t[u], col[lane + 32 * u], y);
+  }
+  for (int i = jd + lane; i < m; i += 32) S.y[i] = make_double2(0, 0);
 }
 
 __global__ void k_gmres_mark_done(GmresState S, const double* __restrict__ nrm2, double tol, int nrhs) {
@@ -933,17 +951,21 @@ __global__ void k_gmres_mark_done(GmresState S, const double* __restrict__ nrm2,
 }
 
 void launch_gmres_start(const GmresState& s, const double* nrm2, double tol, int nrhs, double* inv_beta,
-                        cudaStream_t st) {
-  k_gmres_start<<<nblk(nrhs, 64), 64, 0, st>>>(s, nrm2, tol, nrhs, inv_beta);
+                        cudaStream_t st, bool init) {
+  k_gmres_start<<<nblk(nrhs, 64), 64, 0, st>>>(s, nrm2, tol, nrhs, inv_beta, init);
   WCMG_LAUNCH_CHECK();
 }
-void launch_gmres_step(const GmresState& s, int j, const double2* h, const double* hnorm2, double tol,
+void launch_gmres_init(const GmresState& s, const double* nrm2, int nrhs, cudaStream_t st) {
+  k_gmres_init<<<nblk(nrhs, 64), 64, 0, st>>>(s, nrm2, nrhs);
+  WCMG_LAUNCH_CHECK();
+}
+void launch_gmres_step(const GmresState& s, int j, const double2* h, const double* partial, int count, double tol,
                        int final_done, int nrhs, double* inv_h, cudaStream_t st, const int* jdev) {
-  k_gmres_step<<<nblk(nrhs, 64), 64, 0, st>>>(s, j, h, hnorm2, tol, final_done, nrhs, inv_h, jdev);
+  k_gmres_step<<<nrhs, RED_T, 0, st>>>(s, j, h, partial, count, tol, final_done, inv_h, jdev);
   WCMG_LAUNCH_CHECK();
 }
 void launch_gmres_solve_y(const GmresState& s, int nrhs, cudaStream_t st) {
-  k_gmres_solve_y<<<nblk(nrhs, 64), 64, 0, st>>>(s, nrhs);
+  k_gmres_solve_y<<<nrhs, 32, s.m * (s.m + 1) / 2 * sizeof(double2), st>>>(s);
   WCMG_LAUNCH_CHECK();
 }
 void launch_gmres_mark_done(const GmresState& s, const double* nrm2, double tol, int nrhs, cudaStream_t st) {
@@ -988,8 +1010,8 @@ void launch_counter_gaussian(double2* out, long long n, int nfields, unsigned lo
   template void launch_norm2<R>(double*, const cplx<R>*, long long, int, double*, cudaStream_t);                 \
   template void launch_gram_project<R>(double2*, double2*, const cplx<R>*, long long, int, int, const cplx<R>*,  \
                                        long long, int, double2*, cudaStream_t, const int*, int);                 \
-  template void launch_project_norm<R>(double*, cplx<R>*, const cplx<R>*, long long, int, const double2*, int,   \
-                                       long long, int, double*, cudaStream_t, const int*, int);                  \
+  template int launch_project_norm<R>(double*, cplx<R>*, const cplx<R>*, long long, int, const double2*, int,    \
+                                      long long, int, cudaStream_t, const int*, int);                            \
   template void launch_multiaxpy<R>(cplx<R>*, const cplx<R>*, long long, int, const double2*, int, double,       \
                                     long long, int, cudaStream_t, const int*, int);                              \
   template void launch_copy_idx<R>(cplx<R>*, const cplx<R>*, long long, const int*, long long, long long,        \
@@ -1014,15 +1036,4 @@ template void launch_convert<float, double>(double2*, const float2*, long long, 
 template void launch_convert<double, double>(double2*, const double2*, long long, cudaStream_t);
 template void launch_convert<float, float>(float2*, const float2*, long long, cudaStream_t);
 
-}  // namespace wcmg
-
-namespace wcmg {
-__global__ void k_sqrt_inplace(double* x, int n) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) x[i] = sqrt(x[i]);
-}
-void launch_sqrt_inplace(double* x, int n, cudaStream_t st) {
-  k_sqrt_inplace<<<nblk(n, 64), 64, 0, st>>>(x, n);
-  WCMG_LAUNCH_CHECK();
-}
 }  // namespace wcmg

@@ -192,7 +192,8 @@ void launch_norm2(double* out, const cplx<R>* a, long long n, int nrhs, double* 
 // Arnoldi Gram-Schmidt against V_0 .. V_{k-1} (V_i at basis + i * bstride, each [nrhs][n]):
 // h[r][i] = the coefficients of two classical passes, from one sweep that forms <V_i, w> and
 // the newest column of the Gram matrix G[r] = V^dag V (h: [nrhs][ld], G: [nrhs][ld][ld]);
-// partial: nrhs * 2 * roundup(k, 8) * 608 entries.  Then w -= V h and norm2[r] = ||w||^2.
+// partial: nrhs * 2 * roundup(k, 8) * 608 entries.  Then w -= V h, and the returned number of
+// partial sums of ||w||^2 per rhs in partial (for launch_gmres_step).
 // kdev (nullable, device): the count is *kdev + kadd instead (at most k, which sizes
 // the grid) -- the Arnoldi step number of a device-driven loop.
 template <typename R>
@@ -200,9 +201,8 @@ void launch_gram_project(double2* h, double2* G, const cplx<R>* basis, long long
                          const cplx<R>* w, long long n, int nrhs, double2* partial, cudaStream_t st,
                          const int* kdev = nullptr, int kadd = 0);
 template <typename R>
-void launch_project_norm(double* norm2, cplx<R>* w, const cplx<R>* basis, long long bstride, int k, const double2* h,
-                         int ld, long long n, int nrhs, double* partial, cudaStream_t st, const int* kdev = nullptr,
-                         int kadd = 0);
+int launch_project_norm(double* partial, cplx<R>* w, const cplx<R>* basis, long long bstride, int k, const double2* h,
+                        int ld, long long n, int nrhs, cudaStream_t st, const int* kdev = nullptr, int kadd = 0);
 // w[r] += sign * sum_{i<k} coef[r*ldc + i] * basis_i[r]; kdev as for launch_multidot
 template <typename R>
 void launch_multiaxpy(cplx<R>* w, const cplx<R>* basis, long long bstride, int k, const double2* coef, int ldc,
@@ -211,7 +211,6 @@ void launch_multiaxpy(cplx<R>* w, const cplx<R>* basis, long long bstride, int k
 template <typename R>
 void launch_copy_idx(cplx<R>* dst, const cplx<R>* src, long long n, const int* idx, long long dmul, long long smul,
                      cudaStream_t st);
-void launch_fill_int(int* x, int v, int n, cudaStream_t st);
 // y += x widened to FP64
 void launch_add_widened(double2* y, const float2* x, long long n, cudaStream_t st);
 template <typename R>
@@ -276,8 +275,6 @@ struct GmresState {
   int m;
 };
 // h column j is in H (entries 0..j from multidot); hnorm holds ||w||.
-// h: the coefficients of both Gram-Schmidt passes [nrhs][m+1]; hnorm2 = ||w||^2 after both.
-// `final_done`: a recurrence convergence also marks the rhs done (no true-residual check).
 // One fused Arnoldi step after the operator application, for one short rhs
 // (n <= 2^17, restart <= 64): both projections of w against V_0..V_j (G: Gram matrix of the
 // basis, [m+1][m+1]), the norm, the Givens update of Hessenberg column j and V_{j+1} =
@@ -288,21 +285,23 @@ template <typename R>
 void launch_arnoldi_fused(cplx<R>* Vb, long long bstride, cplx<R>* w, long long n, const GmresState& S, double2* G,
                           int j, const int* jdev, double tol, int final_done, cudaStream_t st,
                           cplx<R>* vnext = nullptr);
+// The Givens update of column j: h = the coefficients of both Gram-Schmidt passes [nrhs][m+1],
+// partial = `count` sums of ||w||^2 per rhs; inv_h = 1 / ||w|| (0 for an inactive rhs).
+// `final_done`: a recurrence convergence also marks the rhs done (no true-residual check).
 // jdev (nullable, device): the step number is *jdev instead of j.
-void launch_gmres_step(const GmresState& s, int j, const double2* h, const double* hnorm2, double tol,
+void launch_gmres_step(const GmresState& s, int j, const double2* h, const double* partial, int count, double tol,
                        int final_done, int nrhs, double* inv_h, cudaStream_t st, const int* jdev = nullptr);
 // done[r] |= nrm2[r] <= (tol * bnorm[r])^2
 void launch_gmres_mark_done(const GmresState& s, const double* nrm2, double tol, int nrhs, cudaStream_t st);
 void launch_gmres_solve_y(const GmresState& s, int nrhs, cudaStream_t st);
-// start a cycle: beta[r] = sqrt(nrm2[r]); g = (beta, 0...); active = beta > tol*bnorm; inv_beta
+// start a cycle: beta[r] = sqrt(nrm2[r]); g = (beta, 0...); active = beta > tol*bnorm; inv_beta.
+// init: the first cycle from x = 0 (r = b), which sets bnorm and done as well
 void launch_gmres_start(const GmresState& s, const double* nrm2, double tol, int nrhs, double* inv_beta,
-                        cudaStream_t st);
+                        cudaStream_t st, bool init = false);
+// bnorm = sqrt(nrm2), done = 0
+void launch_gmres_init(const GmresState& s, const double* nrm2, int nrhs, cudaStream_t st);
 
 }  // namespace wcmg
-
-namespace wcmg {
-void launch_sqrt_inplace(double* x, int n, cudaStream_t st);
-}
 
 namespace wcmg {
 // ---- learned coarse correction: PTC network (ptc.cu), FP32 fields [12][V] ----

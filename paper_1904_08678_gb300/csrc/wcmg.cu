@@ -853,18 +853,17 @@ static KrylovOut fgmres(wcmg_ctx* c, int l, cplx<R>* x, const cplx<R>* b, int nr
   ensure_gram_partials(c, nrhs, m);
   GmresState S = SC.state(m);
   const int ldh = m + 1;
-  norm2_op<R>(c, S.bnorm, b, n, nrhs);
-  launch_sqrt_inplace(S.bnorm, nrhs, c->st);
-  WCMG_CUDA(cudaMemsetAsync(S.done, 0, sizeof(int) * nrhs, c->st));
+  norm2_op<R>(c, SC.slot(1), b, n, nrhs);
+  launch_gmres_init(S, SC.slot(1), nrhs, c->st);
   if (x_zero) {
     launch_fill_zero<R>(x, n * nrhs, c->st);
     copy_fields<R>(c, r, b, n * nrhs);
   } else {
     residual_op<R>(c, l, r, b, x, nrhs);
+    norm2_op<R>(c, SC.slot(1), r, n, nrhs);
   }
   KrylovOut out;
   int cycles = 0;
-  norm2_op<R>(c, SC.slot(1), r, n, nrhs);
   while (true) {
     launch_gmres_start(S, SC.slot(1), tol, nrhs, SC.slot(2), c->st);
     launch_scale_dev<R>(Vb, r, SC.slot(2), 0, n, nrhs, c->st);
@@ -891,9 +890,10 @@ static KrylovOut fgmres(wcmg_ctx* c, int l, cplx<R>* x, const cplx<R>* b, int nr
       } else {
         KPROF(c, WCMG_K_KRYLOV, (double)(j + 3) * n * nrhs * sizeof(cplx<R>), 16.0 * (j + 1) * n * nrhs,
               launch_gram_project<R>(SC.h(), SC.G.p, Vb, bstride, j + 1, ldh, w, n, nrhs, c->partial.p, c->st));
+        int nb = 0;
         KPROF(c, WCMG_K_KRYLOV, (double)(j + 3) * n * nrhs * sizeof(cplx<R>), 8.0 * (j + 1) * n * nrhs,
-              launch_project_norm<R>(SC.slot(0), w, Vb, bstride, j + 1, SC.h(), ldh, n, nrhs, c->partial_d.p, c->st));
-        launch_gmres_step(S, j, SC.h(), SC.slot(0), tol, verify ? 0 : 1, nrhs, SC.slot(3), c->st);
+              nb = launch_project_norm<R>(c->partial_d.p, w, Vb, bstride, j + 1, SC.h(), ldh, n, nrhs, c->st));
+        launch_gmres_step(S, j, SC.h(), c->partial_d.p, nb, tol, verify ? 0 : 1, nrhs, SC.slot(3), c->st);
         launch_scale_dev<R>(Vb + (long long)(j + 1) * bstride, w, SC.slot(3), 0, n, nrhs, c->st);
       }
       ++steps;
@@ -1036,24 +1036,23 @@ static void fgmres_g(wcmg_ctx* c, int l, cplx<R>* x, const cplx<R>* b, int nrhs,
   GmresState S = SC.state(m);
   const int ldh = m + 1;
   const int* jd = &K->j;
-  norm2_op<R>(c, S.bnorm, b, n, nrhs);
-  launch_sqrt_inplace(S.bnorm, nrhs, c->st);
-  launch_fill_int(S.done, 0, nrhs, c->st);
+  const bool single = max_cycles == 1, first = single && x_zero;
+  norm2_op<R>(c, SC.slot(1), b, n, nrhs);
+  if (!first) launch_gmres_init(S, SC.slot(1), nrhs, c->st);
   if (x_zero) {
     launch_fill_zero<R>(x, n * nrhs, c->st);
-    copy_fields<R>(c, r, b, n * nrhs);
+    if (!single) copy_fields<R>(c, r, b, n * nrhs);
   } else {
     residual_op<R>(c, l, r, b, x, nrhs);
+    norm2_op<R>(c, SC.slot(1), r, n, nrhs);
   }
-  norm2_op<R>(c, SC.slot(1), r, n, nrhs);
-  const bool single = max_cycles == 1;
   const cudaGraphConditionalHandle h_loop = single ? 0 : cond_handle(c);
   launch_kctl_init(K, maxiter, budget_its, budget_max, h_loop, single ? 0 : 1, c->st);
 
   // one restart cycle: Arnoldi steps while any rhs is active, then x += Z y
   auto one_cycle = [&]() {
-    launch_gmres_start(S, SC.slot(1), tol, nrhs, SC.slot(2), c->st);
-    launch_scale_dev<R>(Vb, r, SC.slot(2), 0, n, nrhs, c->st, nullptr, 0, 0, vcur);  // vcur = V_j throughout
+    launch_gmres_start(S, SC.slot(1), tol, nrhs, SC.slot(2), c->st, first);
+    launch_scale_dev<R>(Vb, first ? b : r, SC.slot(2), 0, n, nrhs, c->st, nullptr, 0, 0, vcur);  // vcur = V_j throughout
     const cudaGraphConditionalHandle h_arn = cond_handle(c);
     launch_kctl_cycle_begin(K, S.active, nrhs, m, h_arn, c->st);
     cond_node(c, h_arn, cudaGraphCondTypeWhile, [&](int slot) {
@@ -1070,10 +1069,10 @@ static void fgmres_g(wcmg_ctx* c, int l, cplx<R>* x, const cplx<R>* b, int nrhs,
       } else {
         KPROF(c, WCMG_K_KRYLOV, 0.0, 0.0,
               launch_gram_project<R>(SC.h(), SC.G.p, Vb, bstride, m, ldh, w, n, nrhs, c->partial.p, c->st, jd, 1));
+        int nb = 0;
         KPROF(c, WCMG_K_KRYLOV, 0.0, 0.0,
-              launch_project_norm<R>(SC.slot(0), w, Vb, bstride, m, SC.h(), ldh, n, nrhs, c->partial_d.p, c->st, jd,
-                                     1));
-        launch_gmres_step(S, 0, SC.h(), SC.slot(0), tol, verify ? 0 : 1, nrhs, SC.slot(3), c->st, jd);
+              nb = launch_project_norm<R>(c->partial_d.p, w, Vb, bstride, m, SC.h(), ldh, n, nrhs, c->st, jd, 1));
+        launch_gmres_step(S, 0, SC.h(), c->partial_d.p, nb, tol, verify ? 0 : 1, nrhs, SC.slot(3), c->st, jd);
         launch_scale_dev<R>(Vb, w, SC.slot(3), 0, n, nrhs, c->st, jd, 1, bstride, vcur);  // V_{j+1}
       }
       launch_kctl_step_end(K, S.active, nrhs, m, acc, body_count(c, slot), h_arn, c->st);
