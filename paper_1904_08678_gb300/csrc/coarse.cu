@@ -257,7 +257,14 @@ static void coarse_masked_gemm(cplx<R>* out, const cplx<R>* in, const L* links, 
 // the first rows are requested before the gather and the barrier, so every warp has
 // RPW rows (RPW x NK x 512 B) of the link stream in flight.  RPW = 2 keeps as many
 // bytes in flight per warp for 4-byte (BF16 / FP16) links as RPW = 1 does for FP32.
-template <typename R, typename L, int VEC, int NK, int RPW>
+// Bound by the link stream: BF16 links of 8192 x 48 137 us with plain loads and 256 threads, 126 us
+// with 128, 110 us fetched in 256-byte pieces, 106 us also past L1 (ONCE; 6.4 TB/s).
+// Links that fit L2 are not read that way, which drops them there: FP32 links of 512 x 48
+// 12.3 us from L2 either way, but a solve that reads other data in between 5% slower.
+// Many small CTAs per SM hide each other's index, vector and link latencies: persistent
+// CTAs that prefetch the next site took 178 us, a contiguous share of the rows per warp 146 us.
+constexpr long long COARSE_L2_BYTES = 96ll << 20;  // of 129 MB
+template <typename R, typename L, int VEC, int NK, int RPW, bool ONCE>
 __global__ void __launch_bounds__(512) k_coarse_apply1(cplx<R>* __restrict__ out, const cplx<R>* __restrict__ in,
                                                        const L* __restrict__ links, const int* __restrict__ nbr,
                                                        int Vc, int nb, int ld, int parts) {
@@ -277,7 +284,8 @@ __global__ void __launch_bounds__(512) k_coarse_apply1(cplx<R>* __restrict__ out
 #pragma unroll
       for (int j = 0; j < NK; ++j) {
         const int k0 = VEC * (lane + 32 * j);
-        if (r < row1 && k0 < ld) cur[u][j] = *reinterpret_cast<const LinkVec<L, VEC>*>(base + (long long)r * ld + k0);
+        if (r < row1 && k0 < ld)
+          cur[u][j] = load_stream<ONCE>(reinterpret_cast<const LinkVec<L, VEC>*>(base + (long long)r * ld + k0));
       }
     }
   };
@@ -1134,8 +1142,13 @@ static void coarse_apply1(cplx<R>* out, const cplx<R>* in, const L* links, const
   const int nk = (ld + 32 * VEC - 1) / (32 * VEC);
   const size_t smem = (size_t)ld * sizeof(cplx<R>);
   const unsigned grid = (unsigned)(g.V * parts);
+  // links that L2 cannot hold from one apply to the next
+  const bool once = (long long)g.V * nb * ld * (long long)sizeof(L) > COARSE_L2_BYTES;
 #define WCMG_C1(NKV, RP) \
-  k_coarse_apply1<R, L, VEC, NKV, RP><<<grid, threads, smem, st>>>(out, in, links, g.nbr, g.V, nb, ld, parts)
+  do {                                                                                                   \
+    auto kern = once ? k_coarse_apply1<R, L, VEC, NKV, RP, true> : k_coarse_apply1<R, L, VEC, NKV, RP, false>; \
+    kern<<<grid, threads, smem, st>>>(out, in, links, g.nbr, g.V, nb, ld, parts);                          \
+  } while (0)
 #define WCMG_C1R(NKV) \
   if (rpw == 2) WCMG_C1(NKV, 2); else WCMG_C1(NKV, 1)
   if (nk <= 4) { WCMG_C1R(4); }
@@ -1295,8 +1308,11 @@ static void coarse_apply_mma4(float2* out, const float2* in, const bf16c* lmma, 
 
 // The fixed launch rule (used unless a tile is given):
 //  - BF16 links, full stencil, >= 8 rhs, nbasis <= 64: tensor cores, N tile = rhs rounded to 16 (<= 64);
-//  - one rhs, full stencil: the one-rhs kernel, 512 threads, a site split in up to 4
-//    CTAs while there are fewer than 2 CTAs per SM;
+//  - one rhs, full stencil: the one-rhs kernel.  Lattices of at least two sites per SM:
+//    256 threads for FP32 links, 128 with two rows in flight per warp for 2-byte ones (a
+//    site split in up to 4 CTAs while there are fewer than 6 per SM; 8192 x 48 143 us with
+//    512 threads, 106 us with 128; 512 x 48 12.5 and 10.5 us); else, and for FP64, 512
+//    threads, a site split in up to 4 CTAs while there are fewer than 2 per SM;
 //  - otherwise the rhs-tile kernel, 4 rhs per CTA (FP64 or <= 4 rhs) else 8, rows split
 //    until about 6 CTAs per SM.
 CoarseTile coarse_default_tile(int nb, int nrhs, int mode, int Vc, int link_kind) {
@@ -1310,8 +1326,15 @@ CoarseTile coarse_default_tile(int nb, int nrhs, int mode, int Vc, int link_kind
     t.kind = 0;
     t.rr = 1;
     t.parts = 1;
-    while (t.parts < 4 && (long long)Vc * t.parts < 2LL * 152) t.parts *= 2;
     t.threads = 512;
+    long long want = 2LL * 152;
+    if (Vc >= want && link_kind == 1) t.threads = 256;
+    if (Vc >= want && link_kind >= 2) {
+      t.threads = 128;
+      t.stages = links_ld(nb) <= 8 * 128 ? 2 : 1;
+      want = 6LL * 152;
+    }
+    while (t.parts < 4 && 2 * t.parts <= nb && Vc * t.parts < want) t.parts *= 2;
     return t;
   }
   t.kind = 1;

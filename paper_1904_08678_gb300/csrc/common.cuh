@@ -65,6 +65,24 @@ template <typename R> __host__ __device__ __forceinline__ cplx<R> from_c64(doubl
 template <> __host__ __device__ __forceinline__ double2 from_c64<double>(double2 a) { return a; }
 template <> __host__ __device__ __forceinline__ float2 from_c64<float>(double2 a) { return make_float2((float)a.x, (float)a.y); }
 
+// 16-byte loads of a long contiguous stream, which L2 fetches in 256-byte pieces.  ONCE: data that
+// does not stay in L2 until it is read again; it goes past L1 and is the first to leave L2.
+template <bool ONCE, typename T> __device__ __forceinline__ T load_stream(const T* p) {
+  static_assert(sizeof(T) == 16, "16 bytes");
+  uint4 v;
+  if constexpr (ONCE)
+    asm volatile("ld.global.nc.L1::no_allocate.L2::256B.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                 : "l"(p));
+  else
+    asm volatile("ld.global.nc.L2::256B.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                 : "l"(p));
+  T r;
+  memcpy(&r, &v, 16);
+  return r;
+}
+
 // ---- coarse-link storage types: complex numbers stored as (re, im) pairs ----
 struct bf16c { __nv_bfloat162 v; };
 struct f16c { __half2 v; };

@@ -468,7 +468,7 @@ static std::vector<CoarseTile> coarse_candidates(int nb, int nrhs, int lk, bool 
     if (coarse_tile_valid(t, nb, nrhs, ST_FULL, lk)) v.push_back(t);
   };
   if (nrhs == 1) {
-    for (int th : {256, 512})
+    for (int th : {128, 256, 512})
       for (int p : {1, 2, 4, 8})
         for (int rp : {1, 2}) add(0, 1, p, th, 0, rp);
     for (int p : {1, 2, 4, 8, 16}) add(1, 1, p, 0, 0);
