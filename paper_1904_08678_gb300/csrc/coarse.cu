@@ -263,7 +263,6 @@ static void coarse_masked_gemm(cplx<R>* out, const cplx<R>* in, const L* links, 
 // 12.3 us from L2 either way, but a solve that reads other data in between 5% slower.
 // Many small CTAs per SM hide each other's index, vector and link latencies: persistent
 // CTAs that prefetch the next site took 178 us, a contiguous share of the rows per warp 146 us.
-constexpr long long COARSE_L2_BYTES = 96ll << 20;  // of 129 MB
 template <typename R, typename L, int VEC, int NK, int RPW, bool ONCE>
 __global__ void __launch_bounds__(512) k_coarse_apply1(cplx<R>* __restrict__ out, const cplx<R>* __restrict__ in,
                                                        const L* __restrict__ links, const int* __restrict__ nbr,
@@ -1143,7 +1142,7 @@ static void coarse_apply1(cplx<R>* out, const cplx<R>* in, const L* links, const
   const size_t smem = (size_t)ld * sizeof(cplx<R>);
   const unsigned grid = (unsigned)(g.V * parts);
   // links that L2 cannot hold from one apply to the next
-  const bool once = (long long)g.V * nb * ld * (long long)sizeof(L) > COARSE_L2_BYTES;
+  const bool once = (long long)g.V * nb * ld * (long long)sizeof(L) > L2_KEEP_BYTES;
 #define WCMG_C1(NKV, RP) \
   do {                                                                                                   \
     auto kern = once ? k_coarse_apply1<R, L, VEC, NKV, RP, true> : k_coarse_apply1<R, L, VEC, NKV, RP, false>; \

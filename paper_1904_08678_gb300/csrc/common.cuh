@@ -65,6 +65,8 @@ template <typename R> __host__ __device__ __forceinline__ cplx<R> from_c64(doubl
 template <> __host__ __device__ __forceinline__ double2 from_c64<double>(double2 a) { return a; }
 template <> __host__ __device__ __forceinline__ float2 from_c64<float>(double2 a) { return make_float2((float)a.x, (float)a.y); }
 
+// what a stream may hold to be still in L2 (129 MB) when it is read again
+constexpr long long L2_KEEP_BYTES = 96ll << 20;
 // 16-byte loads of a long contiguous stream, which L2 fetches in 256-byte pieces.  ONCE: data that
 // does not stay in L2 until it is read again; it goes past L1 and is the first to leave L2.
 template <bool ONCE, typename T> __device__ __forceinline__ T load_stream(const T* p) {

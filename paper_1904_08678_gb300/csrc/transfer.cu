@@ -159,6 +159,106 @@ __global__ void __launch_bounds__(256) k_prolong(cplx<R>* __restrict__ out, cons
   }
 }
 
+// One right-hand side on the fine layout, bound by the vector stream: 16 bytes (two FP32 sites or
+// one FP64 site) of 4 vectors in flight per thread; ONCE as in load_stream.  With 24 FP32
+// vectors and the change of layout, 16^3x32 (302 MB) 84 us with 8-byte loads, 65 us now (8 vectors in
+// flight 76 us, through L1 83 us); 24^3x48 305 and 278 us; 32^3x64 828 and 829 us.
+template <typename T> struct alignas(16) Wide { T v[16 / sizeof(T)]; };
+template <typename R, bool ONCE>
+__global__ void __launch_bounds__(256) k_prolong1(cplx<R>* __restrict__ out, const cplx<R>* __restrict__ cin,
+                                                  const cplx<R>* __restrict__ vecs, int Vf, int nc, int bvol,
+                                                  int nvec) {
+  using T = cplx<R>;
+  using W = Wide<T>;
+  constexpr int VEC = 16 / sizeof(T), UN = 4;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  T* phi = reinterpret_cast<T*>(smem_raw);  // [2 nvec]
+  const int blk = blockIdx.x, per = bvol / VEC;
+  const long long fstride = (long long)Vf * nc;
+  for (int k = threadIdx.x; k < 2 * nvec; k += blockDim.x) phi[k] = cin[(long long)blk * 2 * nvec + k];
+  __syncthreads();
+  for (int e = threadIdx.x; e < per * nc; e += blockDim.x) {
+    const int c = e / per;
+    const long long a = (long long)c * Vf + (long long)blk * bvol + VEC * (e - c * per);
+    const T* ph = phi + (c >= nc / 2 ? nvec : 0);
+    W acc;
+#pragma unroll
+    for (int w = 0; w < VEC; ++w) acc.v[w] = czero<R>();
+    for (int i0 = 0; i0 < nvec; i0 += UN) {
+      W v[UN];
+#pragma unroll
+      for (int u = 0; u < UN; ++u)
+        if (i0 + u < nvec) v[u] = load_stream<ONCE>(reinterpret_cast<const W*>(vecs + (i0 + u) * fstride + a));
+#pragma unroll
+      for (int u = 0; u < UN; ++u)
+        if (i0 + u < nvec) {
+#pragma unroll
+          for (int w = 0; w < VEC; ++w) cmac(acc.v[w], v[u].v[w], ph[i0 + u]);
+        }
+    }
+    *reinterpret_cast<W*>(out + a) = acc;
+  }
+}
+
+// The restriction of one right-hand side in the same way: one warp per (aggregate, chirality,
+// vector), four 16-byte pieces of the vector in flight per lane; the CTA's 8 vectors share the
+// field's entries in L1.  The same sizes 71, 272 and 798 us before, 62, 272 and 792 us now (two
+// components at once 64, 281 and 826 us).
+template <typename R, bool ONCE>
+__global__ void __launch_bounds__(256) k_restrict1(cplx<R>* __restrict__ out, const cplx<R>* __restrict__ in,
+                                                   const cplx<R>* __restrict__ vecs, int Vf, int nc, int bvol,
+                                                   int nvec) {
+  using T = cplx<R>;
+  using W = Wide<T>;
+  constexpr int VEC = 16 / sizeof(T), UN = 4;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int vgroups = (nvec + 7) / 8;
+  const int s = (blockIdx.x / vgroups) & 1, blk = blockIdx.x / (2 * vgroups);
+  const int i = (blockIdx.x % vgroups) * 8 + warp;
+  if (i >= nvec) return;
+  const int half = nc >> 1, per = bvol / VEC;
+  const long long base = (long long)(s * half) * Vf + (long long)blk * bvol;
+  const T* v = vecs + i * (long long)Vf * nc + base;
+  const T* p = in + base;
+  T acc[VEC];
+#pragma unroll
+  for (int w = 0; w < VEC; ++w) acc[w] = czero<R>();
+  for (int c = 0; c < half; ++c)
+    for (int q0 = lane; q0 < per; q0 += 32 * UN) {
+      W vv[UN], pp[UN];
+#pragma unroll
+      for (int u = 0; u < UN; ++u)
+        if (q0 + 32 * u < per) {
+          const long long a = (long long)c * Vf + VEC * (q0 + 32 * u);
+          vv[u] = load_stream<ONCE>(reinterpret_cast<const W*>(v + a));
+          pp[u] = *reinterpret_cast<const W*>(p + a);
+        }
+#pragma unroll
+      for (int u = 0; u < UN; ++u)
+        if (q0 + 32 * u < per) {
+#pragma unroll
+          for (int w = 0; w < VEC; ++w) cjmac(acc[w], vv[u].v[w], pp[u].v[w]);
+        }
+    }
+  T t = acc[0];
+#pragma unroll
+  for (int w = 1; w < VEC; ++w) t = t + acc[w];
+  t = warp_sum(t);
+  if (lane == 0) out[(long long)blk * 2 * nvec + s * nvec + i] = t;
+}
+
+// One rhs on the fine layout in 16-byte pieces: whole pieces per aggregate and component,
+// 16-byte aligned (an aggregate's sites start at a multiple of bvol).
+template <typename R>
+static bool wide_pieces(const void* a, const void* b, int bvol, int nrhs, bool fine) {
+  return nrhs == 1 && fine && bvol % (16 / sizeof(cplx<R>)) == 0 &&
+         (reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(b)) % 16 == 0;
+}
+template <typename R>
+static bool vectors_once(int Vf, int nc, int nvec) {
+  return (long long)Vf * nc * nvec * (long long)sizeof(cplx<R>) > L2_KEEP_BYTES;
+}
+
 // Few right-hand sides: one warp per (aggregate, chirality, vector) dot
 // product.  A CTA holds 8 warps = 8 vectors of one (aggregate, chirality), so
 // the fine-field entries they all read come from L1; each lane streams its
@@ -236,6 +336,13 @@ static void restrict_few(cplx<R>* coarse, const cplx<R>* in, const cplx<R>* vecs
                          int nrhs, bool fine, const FaceSel& fs, cudaStream_t st) {
   const int vgroups = (nvec + 7) / 8;
   const unsigned grid = (unsigned)((Vf / bvol) * 2 * vgroups);
+  // a warp's lanes all have a piece (smaller aggregates leave too many of them idle)
+  if (fs.fd < 0 && wide_pieces<R>(in, vecs, bvol, nrhs, fine) && bvol >= 32 * (int)(16 / sizeof(cplx<R>))) {
+    auto kern = vectors_once<R>(Vf, nc, nvec) ? k_restrict1<R, true> : k_restrict1<R, false>;
+    kern<<<grid, 256, 0, st>>>(coarse, in, vecs, Vf, nc, bvol, nvec);
+    WCMG_LAUNCH_CHECK();
+    return;
+  }
   k_restrict_few<R, 8><<<grid, 256, 0, st>>>(coarse, in, vecs, Vf, nc, bvol, nvec, nrhs, fine, fs);
   WCMG_LAUNCH_CHECK();
 }
@@ -594,6 +701,11 @@ void launch_prolong(cplx<R>* out, const cplx<R>* coarse, const cplx<R>* vecs, in
   if (nrhs >= 4) {
     k_prolong<R, 4><<<dim3(Vc * ((nrhs + 3) / 4)), 256, 4 * nb * sizeof(cplx<R>), st>>>(out, coarse, vecs, Vf, nc,
                                                                                        bvol, nvec, nrhs, fine);
+  } else if (wide_pieces<R>(out, vecs, bvol, nrhs, fine)) {
+    auto kern = vectors_once<R>(Vf, nc, nvec) ? k_prolong1<R, true> : k_prolong1<R, false>;
+    const int pieces = bvol / (int)(16 / sizeof(cplx<R>)) * nc;
+    kern<<<Vc, std::min(256, (pieces + 31) / 32 * 32), nb * sizeof(cplx<R>), st>>>(out, coarse, vecs, Vf, nc, bvol,
+                                                                                   nvec);
   } else {
     k_prolong<R, 1><<<dim3(Vc * nrhs), 256, nb * sizeof(cplx<R>), st>>>(out, coarse, vecs, Vf, nc, bvol, nvec,
                                                                            nrhs, fine);
