@@ -260,7 +260,8 @@ static void coarse_masked_gemm(cplx<R>* out, const cplx<R>* in, const L* links, 
 // Bound by the link stream: BF16 links of 8192 x 48 137 us with plain loads and 256 threads, 126 us
 // with 128, 110 us fetched in 256-byte pieces, 106 us also past L1 (ONCE; 6.4 TB/s).
 // Links that fit L2 are not read that way, which drops them there: FP32 links of 512 x 48
-// 12.3 us from L2 either way, but a solve that reads other data in between 5% slower.
+// 12.3 us from L2 either way, but a solve that reads other data in between 5% slower.  FP64
+// links keep plain loads: the FP64 units bound them (8192 x 48 1400 against 1490 us).
 // Many small CTAs per SM hide each other's index, vector and link latencies: persistent
 // CTAs that prefetch the next site took 178 us, a contiguous share of the rows per warp 146 us.
 template <typename R, typename L, int VEC, int NK, int RPW, bool ONCE>
@@ -283,8 +284,11 @@ __global__ void __launch_bounds__(512) k_coarse_apply1(cplx<R>* __restrict__ out
 #pragma unroll
       for (int j = 0; j < NK; ++j) {
         const int k0 = VEC * (lane + 32 * j);
-        if (r < row1 && k0 < ld)
-          cur[u][j] = load_stream<ONCE>(reinterpret_cast<const LinkVec<L, VEC>*>(base + (long long)r * ld + k0));
+        if (r < row1 && k0 < ld) {
+          const auto* q = reinterpret_cast<const LinkVec<L, VEC>*>(base + (long long)r * ld + k0);
+          if constexpr (sizeof(L) == 16) cur[u][j] = *q;
+          else cur[u][j] = load_stream<ONCE>(q);
+        }
       }
     }
   };
