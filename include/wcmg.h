@@ -126,8 +126,10 @@ typedef struct wcmg_params {
   int ortho_df;                         /* arithmetic of the block orthonormalisation (Sec. 2.2 Q factor
                                            per aggregate and chirality): 0 FP64; 1 double-float on
                                            the FP32 pipe (each value the unevaluated sum of two
-                                           floats, 48-bit significands, compensated dot products),
-                                           FP64 input and output.  Same algorithm and stopping rule. */
+                                           floats, 48-bit significands, compensated dot products;
+                                           FP64 input and output): Cholesky QR, and Gram-Schmidt
+                                           as for 0 where a column of a panel keeps less than 1/16
+                                           of its squared norm. */
   int coarse_eo;                        /* 1: even-odd (red-black) preconditioned coarsest solve (Sec. 4
                                            lists red-black preconditioning among the missing features):
                                            with coarse sites even / odd by the parity of x + y + z + t,
