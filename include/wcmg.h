@@ -128,8 +128,8 @@ typedef struct wcmg_params {
                                            the FP32 pipe (each value the unevaluated sum of two
                                            floats, 48-bit significands, compensated dot products;
                                            FP64 input and output): Cholesky QR, and Gram-Schmidt
-                                           as for 0 where a column of a panel keeps less than 1/16
-                                           of its squared norm. */
+                                           as for 0 for a panel whose triangular factor R would
+                                           amplify rounding: max_i sum_j |(R^-1)_ji|^2 |a_j|^2 > 8. */
   int coarse_eo;                        /* 1: even-odd (red-black) preconditioned coarsest solve (Sec. 4
                                            lists red-black preconditioning among the missing features):
                                            with coarse sites even / odd by the parity of x + y + z + t,

@@ -10,11 +10,16 @@
 // multiply-add).  G is summed in double-float and, across the threads, in FP64; the k x k
 // factorisation and inverse run in FP64.
 //
-// Accuracy.  Forming G squares the condition number, so a panel is taken here only if no
-// column lost more than 15/16 of its squared norm to the earlier ones (pivot >= |a_j|^2 / 16:
-// near-null candidates keep 0.3 and more); the others are flagged and the Gram-Schmidt
-// kernel does them.  Error against 64 bits on mixed Gaussian panels: 8e-15 (Gram-Schmidt
-// 1.7e-14).
+// Accuracy.  With W = L^-1, Q^H Q - 1 = W dG W^H for the error dG of the sums, whose entries
+// are of the order u |a_i| |a_j|: column i of Q is off by u e_i, e_i = sum_j |W_ij|^2 |a_j|^2.
+// Measured on 24 and 32 columns of 1536 rows with e from 4 to 1e10: max |Q^H Q - 1| is 1.3e-15
+// to 6.3e-15 times max e_i (1e-14 below e = 4).  A panel is therefore taken here only if no
+// e_i exceeds CQ_AMP = 8, where 24 and 32 columns are orthonormal to 1.8e-14 and 2.3e-14 (by
+// Gram-Schmidt 1.6e-14 and 1.1e-14); the others are flagged and the Gram-Schmidt kernel does
+// them.  The pivots alone do not bound e: 24 columns that each keep
+// 0.36 of their squared norm can have e = 3e6.  Near-null candidates have e below 4 after the
+// initial sweeps and below 8 after two refinement sweeps on 32^3x64 (2823 of 16384 panels above
+// 4).  Error against 64 bits on mixed Gaussian panels (e = 2): 8e-15 (Gram-Schmidt 1.7e-14).
 //
 // 1024 panels of 1536 x 24 (16^3x32): 3.35 ms by Gram-Schmidt; now 1.10 + 0.10 + 1.23 ms from
 // FP64 and 0.83 + 0.10 + 0.94 ms from FP32 input (Gram, factor, product).  The arithmetic
@@ -29,7 +34,8 @@ namespace wcmg {
 constexpr int CQ_T = 256;     // Gram kernel: threads
 constexpr int CQ_ROWS = 32;   // panel rows per staged tile
 constexpr int CQ_FLUSH = 2;   // tiles between additions of the running double-float sums
-constexpr double CQ_PIVOT = 1.0 / 16.0;
+constexpr float CQ_AMP = 8.f;       // greatest e
+constexpr double CQ_LEAST = 1e-28;  // least |a_j|^2: the error terms of smaller columns' products underflow in FP32
 
 // offset of panel row e (element of chirality s of aggregate blk) within a field
 __device__ __forceinline__ long long cq_addr(bool fine, int blk, int e, int s, int Vf, int nc, int bvol) {
@@ -131,7 +137,7 @@ __global__ void __launch_bounds__(CQ_T, 2) k_cholqr_gram(double2* __restrict__ W
   }
   int gj = pr - (gi * ng - gi * (gi - 1) / 2) + gi;
   float4* tile = reinterpret_cast<float4*>(smem_raw);  // [2][CQ_ROWS][pitch]
-  // staging role: row lane of the tile, columns warp, warp + 9, ...
+  // staging role: row lane of the tile, columns warp, warp + NW, ...
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   constexpr int NW = CQ_T / 32, NL = (33 + NW - 1) / NW;
   TIN pre[NL];
@@ -240,7 +246,8 @@ __global__ void __launch_bounds__(32 * CQ_CW) k_cholqr_factor(double2* __restric
   for (int k = 0; k < nvec; ++k) {
     const double piv = M[k * nvec + k].x;
     const double ref = __shfl_sync(0xffffffffu, d0, k);
-    if (!(piv > CQ_PIVOT * ref) || !isfinite(piv)) {  // also for a NaN; uniform over the warp
+    // e_k >= |a_k|^2 / pivot; also for a NaN; uniform over the warp
+    if (!(CQ_AMP * piv > ref) || !(ref > CQ_LEAST) || !isfinite(piv)) {
       ok = false;
       break;
     }
@@ -255,15 +262,20 @@ __global__ void __launch_bounds__(32 * CQ_CW) k_cholqr_factor(double2* __restric
     }
     __syncwarp();
   }
+  if (ok) {
+    const double scale = 1.0 / sqrt(piv_own), norm = sqrt(d0);
+    for (int i = 0; i < nvec; ++i) {
+      const double si = __shfl_sync(0xffffffffu, scale, i);
+      const double2 v = !col || lane > i ? make_double2(0, 0) : si * (lane == i ? make_double2(1, 0) : M[i * nvec + lane]);
+      if (col) w[i * nvec + lane] = v;
+      const float2 t = make_float2((float)(norm * v.x), (float)(norm * v.y));
+      const float e = warp_sum(cnorm2(t));  // needs no more than FP32; the same in every lane
+      ok = ok && e <= CQ_AMP;               // false for a NaN
+    }
+  }
   if (lane == 0) {
     flag[panel] = ok ? 0 : 1;
     if (!ok) atomicAdd(nflag, 1);
-  }
-  if (!ok) return;
-  const double scale = 1.0 / sqrt(piv_own);
-  for (int i = 0; i < nvec; ++i) {
-    const double si = __shfl_sync(0xffffffffu, scale, i);
-    if (col) w[i * nvec + lane] = lane > i ? make_double2(0, 0) : si * (lane == i ? make_double2(1, 0) : M[i * nvec + lane]);
   }
 }
 

@@ -71,3 +71,30 @@ def test_rank_deficient_aggregate_is_refused():
     with pytest.raises(wcmg.WcmgError) as e:
         ctx.set_nullvecs(0, dev(v))
     assert e.value.code == wcmg.ERR_NAN
+
+
+def chained_panels(nvec, keep):
+    """One 4^4 aggregate, 1536 rows per chirality: unit columns a_j = keep q_j + sqrt(1 - keep^2) q_{j-1}
+    with orthonormal q.  Every pivot is about keep^2 or more; the condition number grows
+    geometrically with the columns."""
+    R = np.diag(np.full(nvec, keep)) + np.diag(np.full(nvec - 1, np.sqrt(1 - keep**2)), 1)
+    R[0, 0] = 1
+    out = np.empty((nvec, 256, 2, 6), complex)
+    for s in (0, 1):
+        q, _ = np.linalg.qr(inputs.complex_gaussian(35 + s, nvec, (1536, nvec)))
+        out[:, :, s] = (q @ R).T.reshape(nvec, 256, 6)
+    return out.reshape(nvec, 256, 4, 3), np.linalg.cond(R)
+
+
+# The double-float unit here is 1e-14 (the factor of a well-conditioned panel): twice that times
+# the condition number, on panels that Cholesky QR takes (0.95 to 0.8) and on such as it
+# must leave (0.6 and less; its own error there is the square of the condition number).
+@pytest.mark.parametrize("nvec,keep", [(24, 0.95), (32, 0.9), (24, 0.8), (32, 0.8), (24, 0.6), (32, 0.6), (24, 0.53),
+                                       (8, 0.283), (10, 0.283), (4, 0.28)])
+def test_chained_columns_stay_orthonormal(nvec, keep):
+    v, cond = chained_panels(nvec, keep)
+    a, b = q_factor((4, 4, 4, 4), (4, 4, 4, 4), nvec, v, 1), q_factor((4, 4, 4, 4), (4, 4, 4, 4), nvec, v, 0)
+    for s in (0, 1):
+        q = a.reshape(nvec, 256, 2, 6)[:, :, s].reshape(nvec, -1)
+        assert np.abs(q.conj() @ q.T - np.eye(nvec)).max() < 2e-14 * cond
+    assert rel(a, b) < 2e-14 * cond
