@@ -104,136 +104,82 @@ void launch_norm2(double* out, const cplx<R>* a, long long n, int nrhs, double* 
   WCMG_LAUNCH_CHECK();
 }
 
-// ---- Gram-Schmidt of an Arnoldi step: two sweeps over the basis ----
-// Classical Gram-Schmidt twice is h1 = V^dag w, w1 = w - V h1, h2 = V^dag w1, w1 - V h2.
-// Since h2 = h1 - G h1 with the Gram matrix G = V^dag V of the basis, the second projection
-// needs no sweep of its own once G is known: the sweep that forms <V_i, w> also forms the
-// newest column <V_i, V_j> of G (V_j and w are read once per chunk of 8 basis vectors and
-// stay in L2 between the chunks), and one update subtracts V (h1 + h2).  G is as accurate
-// as the sums are (FP32 products, FP64 across warps), so what is left of V in the result
-// is of the order |1 - G|^2, as after two explicit passes.  Bound by HBM: k + 2 + k + 2
-// fields instead of 4 k + 9 (norm included): the 12-rhs solve on 24^3x48 went from 621 to 538 ms.
+// ---- Gram-Schmidt of an Arnoldi step: classical, twice ----
+// h1 = V^dag w, w1 = w - V h1, h2 = V^dag w1, w2 = w1 - V h2 and ||w2||^2: four sweeps over the
+// basis, bound by HBM.  The second projection has to be formed from w1 itself: what the first
+// pass leaves of V in w1 is mostly the rounding of h1 and of the update, u |w| of |w1|, which
+// h1 - (V^dag V) h1 (two sweeps fewer) does not contain.  With |w1| / |w| = 0.03 in FP32 that
+// form left 7e-6 to 1e-4 of V in the new basis vector, two explicit passes 1e-7.
 constexpr int MD_K = 8;
+constexpr int GS_MAXK = 80;  // basis vectors (restart <= 64)
+// <V_i, w> in chunks of 8 basis vectors
 template <typename R>
-__global__ void __launch_bounds__(RED_T) k_gram_partial(double2* __restrict__ partial, const cplx<R>* __restrict__ basis,
-                                                        long long bstride, int k, const cplx<R>* __restrict__ w,
-                                                        long long n, int nchunk, const int* __restrict__ kdev, int kadd,
-                                                        int vec2) {
-  __shared__ double2 scratch[2][(RED_T / 32) * MD_K];
-  // chunks of basis vectors fastest in the grid: CTAs running together read the same w, V_j
+__global__ void __launch_bounds__(RED_T) k_multidot_partial(double2* __restrict__ partial,
+                                                            const cplx<R>* __restrict__ basis, long long bstride,
+                                                            int k, const cplx<R>* __restrict__ w, long long n,
+                                                            int nchunk, const int* __restrict__ kdev, int kadd,
+                                                            int vec2) {
+  __shared__ double2 scratch[(RED_T / 32) * MD_K];
+  // chunks of basis vectors fastest in the grid: CTAs running together read the same w
   const int i0 = (blockIdx.x % nchunk) * MD_K, blk = blockIdx.x / nchunk, nblk_ = gridDim.x / nchunk;
   const int r = blockIdx.y, kpad = nchunk * MD_K;
   if (kdev) k = *kdev + kadd;
   if (i0 >= k) return;  // uniform per block
   const long long off = (long long)r * n;
-  const cplx<R>* vj = basis + (k - 1) * bstride + off;
-  cplx<R> aw[MD_K], av[MD_K];
+  cplx<R> acc[MD_K];
 #pragma unroll
-  for (int q = 0; q < MD_K; ++q) aw[q] = av[q] = czero<R>();
+  for (int q = 0; q < MD_K; ++q) acc[q] = czero<R>();
   if constexpr (sizeof(R) == 4) {
     if (vec2) {  // two complex entries per 16-byte load (n, bstride even; 16-byte aligned fields)
       const float4* w4 = reinterpret_cast<const float4*>(w + off);
-      const float4* v4 = reinterpret_cast<const float4*>(vj);
       const long long n2 = n >> 1;
       for (long long e = blk * (long long)RED_T + threadIdx.x; e < n2; e += (long long)nblk_ * RED_T) {
-        const float4 x = w4[e], y = v4[e];
+        const float4 x = w4[e];
 #pragma unroll
         for (int q = 0; q < MD_K; ++q)
           if (i0 + q < k) {
             const float4 v = reinterpret_cast<const float4*>(basis + (i0 + q) * bstride + off)[e];
-            cjmac(aw[q], make_float2(v.x, v.y), make_float2(x.x, x.y));
-            cjmac(aw[q], make_float2(v.z, v.w), make_float2(x.z, x.w));
-            cjmac(av[q], make_float2(v.x, v.y), make_float2(y.x, y.y));
-            cjmac(av[q], make_float2(v.z, v.w), make_float2(y.z, y.w));
+            cjmac(acc[q], make_float2(v.x, v.y), make_float2(x.x, x.y));
+            cjmac(acc[q], make_float2(v.z, v.w), make_float2(x.z, x.w));
           }
       }
     }
   }
   if (sizeof(R) == 8 || !vec2)
     for (long long e = blk * (long long)RED_T + threadIdx.x; e < n; e += (long long)nblk_ * RED_T) {
-      const cplx<R> x = w[off + e], y = vj[e];
+      const cplx<R> x = w[off + e];
 #pragma unroll
       for (int q = 0; q < MD_K; ++q)
-        if (i0 + q < k) {
-          const cplx<R> v = basis[(i0 + q) * bstride + off + e];
-          cjmac(aw[q], v, x);
-          cjmac(av[q], v, y);
-        }
+        if (i0 + q < k) cjmac(acc[q], basis[(i0 + q) * bstride + off + e], x);
     }
-  // warp sums in the working precision (one transposing butterfly for 8 values), then
-  // FP64 across the warps of the CTA and across CTAs
+  // warp sums in the working precision (one transposing butterfly for the 8 values),
+  // then FP64 across the warps of the CTA and across CTAs
   static_assert(MD_K == 8, "transposing warp reduction of 8 values");
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  warp_sum8_transposed(aw, lane);
-  warp_sum8_transposed(av, lane);
-  if ((lane & 3) == 0) {
-    scratch[0][warp * MD_K + warp_sum8_index(lane)] = to_c64(aw[0]);
-    scratch[1][warp * MD_K + warp_sum8_index(lane)] = to_c64(av[0]);
-  }
+  warp_sum8_transposed(acc, lane);
+  if ((lane & 3) == 0) scratch[warp * MD_K + warp_sum8_index(lane)] = to_c64(acc[0]);
   __syncthreads();
-  const int q = threadIdx.x % MD_K, z = threadIdx.x / MD_K;
-  if (z < 2 && i0 + q < k) {
-    double2 t = scratch[z][q];
-    for (int u = 1; u < RED_T / 32; ++u) t += scratch[z][u * MD_K + q];
-    partial[(((long long)r * 2 + z) * kpad + i0 + q) * nblk_ + blk] = t;
+  if (threadIdx.x < MD_K && i0 + threadIdx.x < k) {
+    double2 t = scratch[threadIdx.x];
+    for (int u = 1; u < RED_T / 32; ++u) t += scratch[u * MD_K + threadIdx.x];
+    partial[((long long)r * kpad + i0 + threadIdx.x) * nblk_ + blk] = t;
   }
 }
-// Row i, z = 0: <V_i, w> -> h[r][i]; z = 1: <V_i, V_j> -> column j = k - 1 and row j of G[r]
-__global__ void __launch_bounds__(RED_T) k_gram_final(double2* __restrict__ h, double2* __restrict__ G,
-                                                      const double2* __restrict__ partial, int count, int kpad, int ld,
-                                                      int k, const int* __restrict__ kdev, int kadd) {
-  __shared__ double2 scratch[RED_T / 32];
-  __shared__ double2 red[1];
-  const int r = blockIdx.x, i = blockIdx.y, z = blockIdx.z;
-  if (kdev) k = *kdev + kadd;
-  if (i >= k) return;  // uniform per block
-  const double2* p = partial + (((long long)r * 2 + z) * kpad + i) * count;
-  double2 acc = make_double2(0, 0);
-  for (int b = threadIdx.x; b < count; b += RED_T) acc += p[b];
-  block_sum_many<double2>(&acc, 1, scratch, red);
-  if (threadIdx.x == 0) {
-    if (z == 0) {
-      h[(long long)r * ld + i] = red[0];
-    } else {
-      double2* g = G + (long long)r * ld * ld;
-      g[(long long)(k - 1) * ld + i] = conjg(red[0]);
-      g[(long long)i * ld + k - 1] = red[0];
-    }
-  }
-}
-// h <- h + (h - G h): the coefficients of both projections (one CTA per rhs, k <= 65)
-constexpr int GC_T = 96;
-__global__ void __launch_bounds__(GC_T) k_gram_coef(double2* __restrict__ h, const double2* __restrict__ G, int ld,
-                                                    int k, const int* __restrict__ kdev, int kadd) {
-  __shared__ double2 hs[GC_T];
-  const int r = blockIdx.x, i = threadIdx.x;
-  if (kdev) k = *kdev + kadd;
-  double2* hr = h + (long long)r * ld;
-  if (i < k) hs[i] = hr[i];
-  __syncthreads();
-  if (i >= k) return;
-  const double2* g = G + (long long)r * ld * ld;
-  double2 t = hs[i];
-  for (int l = 0; l < k; ++l) t -= cjmul(g[(long long)l * ld + i], hs[l]);  // G_il = conj(G_li)
-  hr[i] = hs[i] + t;
-}
-// k basis vectors, the newest one V_{k-1}; with kdev the count is *kdev + kadd (<= k) read on
-// the device.  h: [nrhs][ld] coefficients of both projections, G: [nrhs][ld][ld].
+// 16-byte accesses to the basis and w
 template <typename R>
-void launch_gram_project(double2* h, double2* G, const cplx<R>* basis, long long bstride, int k, int ld,
-                         const cplx<R>* w, long long n, int nrhs, double2* partial, cudaStream_t st, const int* kdev,
-                         int kadd) {
+static int basis_vec2(const cplx<R>* basis, long long bstride, const cplx<R>* w, long long n) {
+  return sizeof(R) == 4 && n % 2 == 0 && bstride % 2 == 0 && reinterpret_cast<uintptr_t>(basis) % 16 == 0 &&
+         reinterpret_cast<uintptr_t>(w) % 16 == 0;
+}
+template <typename R>
+static void multidot(double2* out, const cplx<R>* basis, long long bstride, int k, int ldo, const cplx<R>* w,
+                     long long n, int nrhs, double2* partial, cudaStream_t st, const int* kdev, int kadd) {
   const int nchunk = (k + MD_K - 1) / MD_K, kpad = nchunk * MD_K;
-  if (k > GC_T) throw Error(-1, "Gram-Schmidt supports k <= 96");
   const int nb = red_blocks(n, nrhs);  // independent of k: a captured graph sums in the same order
-  const int vec2 = sizeof(R) == 4 && n % 2 == 0 && bstride % 2 == 0 && reinterpret_cast<uintptr_t>(basis) % 16 == 0 &&
-                   reinterpret_cast<uintptr_t>(w) % 16 == 0;
-  k_gram_partial<R><<<dim3(nb * nchunk, nrhs), RED_T, 0, st>>>(partial, basis, bstride, k, w, n, nchunk, kdev, kadd,
-                                                               vec2);
+  k_multidot_partial<R><<<dim3(nb * nchunk, nrhs), RED_T, 0, st>>>(partial, basis, bstride, k, w, n, nchunk, kdev,
+                                                                   kadd, basis_vec2<R>(basis, bstride, w, n));
   WCMG_LAUNCH_CHECK();
-  k_gram_final<<<dim3(nrhs, k, 2), RED_T, 0, st>>>(h, G, partial, nb, kpad, ld, k, kdev, kadd);
-  WCMG_LAUNCH_CHECK();
-  k_gram_coef<<<nrhs, GC_T, 0, st>>>(h, G, ld, k, kdev, kadd);
+  k_final<double2><<<dim3(nrhs, k), RED_T, 0, st>>>(out, partial, nb, (long long)kpad * nb, nb, ldo, kdev, kadd);
   WCMG_LAUNCH_CHECK();
 }
 
@@ -245,7 +191,7 @@ __global__ void __launch_bounds__(AN_T) k_project_norm(cplx<R>* __restrict__ w, 
                                                        long long bstride, int k, const double2* __restrict__ h, int ld,
                                                        long long n, double* __restrict__ partial,
                                                        const int* __restrict__ kdev, int kadd, int vec2) {
-  __shared__ cplx<R> cf[GC_T];
+  __shared__ cplx<R> cf[GS_MAXK];
   __shared__ double scratch[AN_T / 32];
   __shared__ double red[1];
   const int r = blockIdx.y;
@@ -287,11 +233,9 @@ __global__ void __launch_bounds__(AN_T) k_project_norm(cplx<R>* __restrict__ w, 
   if (threadIdx.x == 0) partial[(long long)r * gridDim.x + blockIdx.x] = red[0];
 }
 template <typename R>
-int launch_project_norm(double* partial, cplx<R>* w, const cplx<R>* basis, long long bstride, int k, const double2* h,
+static int project_norm(double* partial, cplx<R>* w, const cplx<R>* basis, long long bstride, int k, const double2* h,
                         int ld, long long n, int nrhs, cudaStream_t st, const int* kdev, int kadd) {
-  if (k > GC_T) throw Error(-1, "Gram-Schmidt supports k <= 96");
-  const int vec2 = sizeof(R) == 4 && n % 2 == 0 && bstride % 2 == 0 && reinterpret_cast<uintptr_t>(basis) % 16 == 0 &&
-                   reinterpret_cast<uintptr_t>(w) % 16 == 0;
+  const int vec2 = basis_vec2<R>(basis, bstride, w, n);
   const long long per = (long long)AN_T * (vec2 ? 2 : 1);
   const int nb = (int)std::max(1LL, std::min(608LL, (n + per - 1) / per));
   k_project_norm<R><<<dim3(nb, nrhs), AN_T, 0, st>>>(w, basis, bstride, k, h, ld, n, partial, kdev, kadd, vec2);
@@ -303,7 +247,7 @@ template <typename R>
 __global__ void k_multiaxpy(cplx<R>* __restrict__ w, const cplx<R>* __restrict__ basis, long long bstride, int k,
                            const double2* __restrict__ coef, int ldc, double sign, long long n,
                            const int* __restrict__ kdev, int kadd) {
-  __shared__ cplx<R> cf[80];  // k <= 65 (restart <= 64)
+  __shared__ cplx<R> cf[GS_MAXK];
   const int r = blockIdx.y;
   if (kdev) k = min(*kdev + kadd, k);
   for (int i = threadIdx.x; i < k; i += blockDim.x) {
@@ -322,9 +266,20 @@ template <typename R>
 void launch_multiaxpy(cplx<R>* w, const cplx<R>* basis, long long bstride, int k, const double2* coef, int ldc,
                       double sign, long long n, int nrhs, cudaStream_t st, const int* kdev, int kadd) {
   if (k <= 0) return;
-  if (k > 80) throw Error(-1, "multiaxpy supports k <= 80");
+  if (k > GS_MAXK) throw Error(-1, "multiaxpy supports k <= 80");
   k_multiaxpy<R><<<dim3(nblk(n, 256), nrhs), 256, 0, st>>>(w, basis, bstride, k, coef, ldc, sign, n, kdev, kadd);
   WCMG_LAUNCH_CHECK();
+}
+
+template <typename R>
+int launch_gram_schmidt(double2* h1, double2* h2, double* norm_partial, cplx<R>* w, const cplx<R>* basis,
+                        long long bstride, int k, int ld, long long n, int nrhs, double2* partial, cudaStream_t st,
+                        const int* kdev, int kadd) {
+  if (k > GS_MAXK) throw Error(-1, "Gram-Schmidt supports k <= 80");
+  multidot<R>(h1, basis, bstride, k, ld, w, n, nrhs, partial, st, kdev, kadd);
+  launch_multiaxpy<R>(w, basis, bstride, k, h1, ld, -1.0, n, nrhs, st, kdev, kadd);
+  multidot<R>(h2, basis, bstride, k, ld, w, n, nrhs, partial, st, kdev, kadd);
+  return project_norm<R>(norm_partial, w, basis, bstride, k, h2, ld, n, nrhs, st, kdev, kadd);
 }
 
 template <typename R>
@@ -626,9 +581,10 @@ __device__ void gmres_rotate(GmresState S, int j, double2* hcol, const double* c
 }
 
 // One CTA per rhs: ||w||^2 from the `count` partials of k_project_norm, then the rotation with
-// the column and the earlier rotations fetched in parallel (12 us; the rotation by one thread
-// from global memory took 12 us and the final sum another launch of 4 us).
-__global__ void __launch_bounds__(RED_T) k_gmres_step(GmresState S, int j, const double2* __restrict__ h,
+// the column and the earlier rotations fetched in parallel (12 us, a launch of 4 us for the final
+// sum less than the rotation by one thread from global memory, which took 12 us as well).
+__global__ void __launch_bounds__(RED_T) k_gmres_step(GmresState S, int j, const double2* __restrict__ h1,
+                                                      const double2* __restrict__ h2,
                                                       const double* __restrict__ partial, int count, double tol,
                                                       int final_done, double* __restrict__ inv_h,
                                                       const int* __restrict__ jdev) {
@@ -638,7 +594,10 @@ __global__ void __launch_bounds__(RED_T) k_gmres_step(GmresState S, int j, const
   if (jdev) j = *jdev;
   S = gmres_of(S, r);
   const bool act = S.active[0] != 0;
-  if (threadIdx.x <= j) hcol[threadIdx.x] = h[(long long)r * (S.m + 1) + threadIdx.x];
+  if (threadIdx.x <= j) {
+    const long long i = (long long)r * (S.m + 1) + threadIdx.x;
+    hcol[threadIdx.x] = h1[i] + h2[i];
+  }
   if (threadIdx.x < j) {
     cs[threadIdx.x] = S.cs[threadIdx.x];
     sn[threadIdx.x] = S.sn[threadIdx.x];
@@ -656,19 +615,19 @@ __global__ void __launch_bounds__(RED_T) k_gmres_step(GmresState S, int j, const
 // ---- fused Arnoldi step for short vectors (one rhs) ----
 // Everything of one (F)GMRES Arnoldi step after the operator application, for
 // vectors short enough that a single thread-block cluster streams them from L2:
-// the sweep of <V_i, w> and <V_i, V_j> (the newest column of the Gram matrix), the
-// coefficients h + (h - G h) of both Gram-Schmidt passes, w - V h, its norm, the Givens
-// update of Hessenberg column j and V_{j+1} = w / ||w||.  CTA c of the C-CTA cluster owns
-// a contiguous range of the vector.  Bound by latency, so: the warps share the basis vectors
-// of the sweep evenly (warp sums only, no block barrier per chunk of vectors), the updated
-// elements stay in registers until the norm is known, everything the coefficients and the
-// rotation need (G, cs, sn) is requested before the sweep, remote sums are read all at once,
-// FP64 work is left to as few warps as it has values (a warp's FP64 instruction takes 16
-// cycles of the SM's unit), and the rotation runs from shared memory while the cluster writes
-// V_{j+1}.  Partial sums are exchanged through distributed
-// shared memory and every CTA adds the C partials in the same order, so all CTAs hold
-// identical coefficients.  24.6k entries, 16 CTAs, in a solve under ncu: 36 us with one warp
-// per basis vector and every thread adding the remote norms in FP64, 22 us now.
+// both classical Gram-Schmidt passes h1 = V^dag w, w -= V h1, h2 = V^dag w,
+// w -= V h2, the norm ||w||^2, the Givens update of Hessenberg column j and
+// V_{j+1} = w / ||w||.  CTA c of the C-CTA cluster owns a contiguous range of the
+// vector.  Bound by latency, so: the warps share the basis vectors of a sweep evenly (warp
+// sums only, no block barrier per chunk of vectors), the updated elements stay in registers
+// until the norm is known (and in w for the second sweep), the rotations are requested before
+// the first sweep, remote sums are read all at once, FP64 work is left to as few warps as it
+// has values (a warp's FP64 instruction takes 16 cycles of the SM's unit), and the new
+// rotation runs from shared memory while the cluster writes V_{j+1}.  Partial sums are
+// exchanged through distributed shared memory and every CTA adds the C partials in the same
+// order, so all CTAs hold identical coefficients.  24.6k entries, 16 CTAs, in a solve under ncu:
+// 36 us with one warp per basis vector and every thread adding the remote norms in FP64, 20 us
+// now (registers for one CTA per SM: under the default 64 the elements spilled).
 constexpr int AC_T = 512, AC_MAXK = 65, AC_W = AC_T / 32;
 constexpr int AC_EL = 16;  // most elements per thread
 
@@ -684,119 +643,44 @@ __device__ __forceinline__ double2 ac_cluster_sum(cooperative_groups::cluster_gr
   return v[0];
 }
 
-// NE: elements per thread (power of two; the vector has at most C x AC_T x NE entries)
-template <typename R, int NE>
-__global__ void __launch_bounds__(AC_T) k_arnoldi_cluster(cplx<R>* __restrict__ Vb, long long bstride,
-                                                          const cplx<R>* __restrict__ w, long long n, GmresState S,
-                                                          double2* __restrict__ G, int j, const int* __restrict__ jdev,
-                                                          double tol, int final_done, cplx<R>* __restrict__ vnext) {
-  namespace cg = cooperative_groups;
-  cg::cluster_group cl = cg::this_cluster();
-  const int C = (int)cl.num_blocks(), crank = (int)cl.block_rank();
+// out[i] = this CTA's part of <V_i, w>, i < k: the 16 warps split into one group of P per basis
+// vector (P = 16, 8, .. 1: as many as there are vectors for), each warp a P-th of the range.
+// pw: scratch, one sum per warp.  Complete after the next barrier of the cluster.
+template <typename R>
+__device__ __forceinline__ void ac_sweep(double2* out, cplx<R>* pw, const cplx<R>* V, long long bstride,
+                                         const cplx<R>* w, int cnt, int k) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  __shared__ double2 pA[2 * AC_MAXK];  // this CTA's sums <V_i, w>, then <V_i, V_j> (read by the whole cluster)
-  __shared__ cplx<R> pw[AC_W][2];      // per warp, when several warps share a basis vector
-  __shared__ double2 pN;
-  __shared__ double2 hs[2 * AC_MAXK], hcol[AC_MAXK];
-  __shared__ cplx<R> cf[AC_MAXK];
-  __shared__ double csn[AC_MAXK];
-  __shared__ double2 snn[AC_MAXK];
-  __shared__ R wsum[AC_W];
-  __shared__ double hn_s;
-  __shared__ R inv_s;
-  if (jdev) j = *jdev;
-  const int k = j + 1, m = S.m, ld = m + 1;
-  const bool act = S.active[0] != 0;  // before this step (CTA 0 may change it below)
-  const int per = (int)((n + C - 1) / C);
-  const int e0 = crank * per, cnt = max(0, min(per, (int)n - e0));
-  // row gi of G without its newest entry: 8 lanes per row
-  const int gi = threadIdx.x >> 3, gl = threadIdx.x & 7;
-  double2 gr[8];
-#pragma unroll
-  for (int t = 0; t < 8; ++t) {
-    const int l = gl + 8 * t;
-    gr[t] = gi < k && l < k && l != j && gi != j ? G[(long long)l * ld + gi] : make_double2(0, 0);
-  }
-  if (crank == 0)
-    for (int i = threadIdx.x; i < j; i += AC_T) {
-      csn[i] = S.cs[i];
-      snn[i] = S.sn[i];
-    }
-  // sweep: <V_i, w> and <V_i, V_j>; the 16 warps split into one group of P per basis vector
-  // (P = 16, 8, .. 1: as many as there are vectors for), each warp a P-th of the range
-  const cplx<R>* wv = w + e0;
-  const cplx<R>* vj = Vb + (long long)j * bstride + e0;
   const int P = k == 1 ? 16 : k == 2 ? 8 : k <= 4 ? 4 : k <= 8 ? 2 : 1;
   for (int i = warp / P; i < k; i += AC_W / P) {
-    const cplx<R>* vi = Vb + (long long)i * bstride + e0;
-    cplx<R> aw = czero<R>(), av = czero<R>();
+    const cplx<R>* vi = V + (long long)i * bstride;
+    cplx<R> acc = czero<R>();
 #pragma unroll 8
-    for (int e = lane + 32 * (warp % P); e < cnt; e += 32 * P) {
-      const cplx<R> v = vi[e];
-      cjmac(aw, v, wv[e]);
-      cjmac(av, v, vj[e]);
-    }
-    const cplx<R> tw = warp_sum(aw), tv = warp_sum(av);
+    for (int e = lane + 32 * (warp % P); e < cnt; e += 32 * P) cjmac(acc, vi[e], w[e]);
+    const cplx<R> t = warp_sum(acc);
     if (lane == 0) {
-      if (P == 1) {
-        pA[i] = to_c64(tw);
-        pA[k + i] = to_c64(tv);
-      } else {
-        pw[warp][0] = tw;
-        pw[warp][1] = tv;
-      }
+      if (P == 1) out[i] = to_c64(t);
+      else pw[warp] = t;
     }
   }
   if (P > 1) {
     __syncthreads();
-    if (threadIdx.x < 2 * k) {
-      const int i = threadIdx.x % k, z = threadIdx.x / k;
-      double2 t = to_c64(pw[i * P][z]);
-      for (int u = 1; u < P; ++u) t += to_c64(pw[i * P + u][z]);
-      pA[threadIdx.x] = t;
+    if (threadIdx.x < k) {
+      double2 t = to_c64(pw[threadIdx.x * P]);
+      for (int u = 1; u < P; ++u) t += to_c64(pw[threadIdx.x * P + u]);
+      out[threadIdx.x] = t;
     }
   }
-  cl.sync();
-  if (threadIdx.x < 2 * k) hs[threadIdx.x] = ac_cluster_sum(cl, pA + threadIdx.x, C);
-  __syncthreads();
-  const double2* gs = hs + k;
-  // h + (h - G h), G's newest column gs: G_{l j} = gs_l, G_{j l} = conj(gs_l)
-  if (gi < (k + 3) / 4 * 4) {  // whole warps
-    double2 t = make_double2(0, 0);
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const int l = gl + 8 * q;
-      if (gi < k && l < k) {
-        // gr holds G_{l gi}; the sum needs G_{gi l} = conj(G_{l gi})
-        const double2 g = l == j ? conjg(gs[gi]) : gi == j ? gs[l] : gr[q];
-        t += cjmul(g, hs[l]);
-      }
-    }
-#pragma unroll
-    for (int o = 4; o > 0; o >>= 1) t += shfl_xor2(t, o);
-    if (gi < k && gl == 0) {
-      const double2 h = hs[gi] + (hs[gi] - t);
-      hcol[gi] = h;
-      cf[gi] = cmk(R(h.x), R(h.y));
-      if (crank == 0) {
-        G[(long long)j * ld + gi] = conjg(gs[gi]);
-        G[(long long)gi * ld + j] = gs[gi];
-      }
-    }
-  }
-  __syncthreads();
-  // w - V h in registers (all of a thread's elements per basis vector: loads in flight),
-  // and its norm: warp sums in R, the warps' in FP64
-  cplx<R> x[NE];
-#pragma unroll
-  for (int u = 0; u < NE; ++u) {
-    const int e = threadIdx.x + u * AC_T;
-    x[u] = e < cnt ? wv[e] : czero<R>();
-  }
+}
+
+// x -= V c over the CTA's range, a thread's elements in registers: its loads of all elements
+// per basis vector are in flight together
+template <typename R, int NE>
+__device__ __forceinline__ void ac_update(cplx<R> (&x)[NE], const cplx<R>* V, long long bstride, const cplx<R>* cf,
+                                          int cnt, int k) {
   constexpr int UI = NE >= 8 ? 1 : 8 / NE;
 #pragma unroll UI
   for (int i = 0; i < k; ++i) {
-    const cplx<R>* v = Vb + (long long)i * bstride + e0;
+    const cplx<R>* v = V + (long long)i * bstride;
     const cplx<R> c = cf[i];
 #pragma unroll
     for (int u = 0; u < NE; ++u) {
@@ -804,6 +688,63 @@ __global__ void __launch_bounds__(AC_T) k_arnoldi_cluster(cplx<R>* __restrict__ 
       if (e < cnt) cnmac(x[u], c, v[e]);
     }
   }
+}
+
+// NE: elements per thread (power of two; the vector has at most C x AC_T x NE entries)
+template <typename R, int NE>
+__global__ void __launch_bounds__(AC_T, 1) k_arnoldi_cluster(cplx<R>* Vb, long long bstride, cplx<R>* w, long long n,
+                                                          GmresState S, int j, const int* __restrict__ jdev,
+                                                          double tol, int final_done, cplx<R>* __restrict__ vnext) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  const int C = (int)cl.num_blocks(), crank = (int)cl.block_rank();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  __shared__ double2 pA[2][AC_MAXK];  // this CTA's sums of the two passes (read by the whole cluster)
+  __shared__ double2 pN;
+  __shared__ cplx<R> pw[AC_W], cf[AC_MAXK];
+  __shared__ double2 hcol[AC_MAXK], snn[AC_MAXK];
+  __shared__ double csn[AC_MAXK];
+  __shared__ R wsum[AC_W];
+  __shared__ double hn_s;
+  __shared__ R inv_s;
+  if (jdev) j = *jdev;
+  const int k = j + 1;
+  const bool act = S.active[0] != 0;  // before this step (CTA 0 may change it below)
+  const int per = (int)((n + C - 1) / C);
+  const int e0 = crank * per, cnt = max(0, min(per, (int)n - e0));
+  if (crank == 0)
+    for (int i = threadIdx.x; i < j; i += AC_T) {
+      csn[i] = S.cs[i];
+      snn[i] = S.sn[i];
+    }
+  const cplx<R>* V = Vb + e0;
+  cplx<R>* wv = w + e0;
+  cplx<R> x[NE];
+#pragma unroll
+  for (int u = 0; u < NE; ++u) {
+    const int e = threadIdx.x + u * AC_T;
+    x[u] = e < cnt ? wv[e] : czero<R>();
+  }
+  for (int pass = 0; pass < 2; ++pass) {
+    ac_sweep<R>(pA[pass], pw, V, bstride, wv, cnt, k);
+    cl.sync();
+    if (threadIdx.x < k) {
+      const double2 h = ac_cluster_sum(cl, pA[pass] + threadIdx.x, C);
+      cf[threadIdx.x] = cmk(R(h.x), R(h.y));
+      hcol[threadIdx.x] = pass == 0 ? h : hcol[threadIdx.x] + h;
+    }
+    __syncthreads();
+    ac_update<R, NE>(x, V, bstride, cf, cnt, k);
+    if (pass == 0) {
+#pragma unroll
+      for (int u = 0; u < NE; ++u) {
+        const int e = threadIdx.x + u * AC_T;
+        if (e < cnt) wv[e] = x[u];
+      }
+      __syncthreads();  // w is complete for every warp, and cf and pw are free
+    }
+  }
+  // the norm: warp sums in R, the warps' in FP64
   R nn = 0;
 #pragma unroll
   for (int u = 0; u < NE; ++u) nn += cnorm2(x[u]);
@@ -879,8 +820,8 @@ bool arnoldi_fused_ok(long long n, int nrhs, int m) {
 }
 
 template <typename R>
-void launch_arnoldi_fused(cplx<R>* Vb, long long bstride, cplx<R>* w, long long n, const GmresState& S, double2* G,
-                          int j, const int* jdev, double tol, int final_done, cudaStream_t st, cplx<R>* vnext) {
+void launch_arnoldi_fused(cplx<R>* Vb, long long bstride, cplx<R>* w, long long n, const GmresState& S, int j,
+                          const int* jdev, double tol, int final_done, cudaStream_t st, cplx<R>* vnext) {
   const int C = arnoldi_cluster_size();
   if (C <= 0) throw Error(-1, "no thread-block cluster available for the fused Arnoldi step");
   const long long per = ((n + C - 1) / C + AC_T - 1) / AC_T;  // elements per thread
@@ -901,12 +842,12 @@ void launch_arnoldi_fused(cplx<R>* Vb, long long bstride, cplx<R>* w, long long 
   at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  WCMG_CUDA(cudaLaunchKernelEx(&cfg, kern, Vb, bstride, (const cplx<R>*)w, n, S, G, j, jdev, tol, final_done, vnext));
+  WCMG_CUDA(cudaLaunchKernelEx(&cfg, kern, Vb, bstride, w, n, S, j, jdev, tol, final_done, vnext));
   WCMG_LAUNCH_CHECK();
 }
-template void launch_arnoldi_fused<float>(float2*, long long, float2*, long long, const GmresState&, double2*, int,
-                                          const int*, double, int, cudaStream_t, float2*);
-template void launch_arnoldi_fused<double>(double2*, long long, double2*, long long, const GmresState&, double2*, int,
+template void launch_arnoldi_fused<float>(float2*, long long, float2*, long long, const GmresState&, int, const int*,
+                                          double, int, cudaStream_t, float2*);
+template void launch_arnoldi_fused<double>(double2*, long long, double2*, long long, const GmresState&, int,
                                            const int*, double, int, cudaStream_t, double2*);
 
 // y = R^-1 g by columns, one warp per rhs: lane i holds the right-hand sides i and i + 32, R
@@ -959,9 +900,10 @@ void launch_gmres_init(const GmresState& s, const double* nrm2, int nrhs, cudaSt
   k_gmres_init<<<nblk(nrhs, 64), 64, 0, st>>>(s, nrm2, nrhs);
   WCMG_LAUNCH_CHECK();
 }
-void launch_gmres_step(const GmresState& s, int j, const double2* h, const double* partial, int count, double tol,
-                       int final_done, int nrhs, double* inv_h, cudaStream_t st, const int* jdev) {
-  k_gmres_step<<<nrhs, RED_T, 0, st>>>(s, j, h, partial, count, tol, final_done, inv_h, jdev);
+void launch_gmres_step(const GmresState& s, int j, const double2* h1, const double2* h2, const double* partial,
+                       int count, double tol, int final_done, int nrhs, double* inv_h, cudaStream_t st,
+                       const int* jdev) {
+  k_gmres_step<<<nrhs, RED_T, 0, st>>>(s, j, h1, h2, partial, count, tol, final_done, inv_h, jdev);
   WCMG_LAUNCH_CHECK();
 }
 void launch_gmres_solve_y(const GmresState& s, int nrhs, cudaStream_t st) {
@@ -1008,10 +950,8 @@ void launch_counter_gaussian(double2* out, long long n, int nfields, unsigned lo
 #define WCMG_INST(R)                                                                                             \
   template void launch_dot<R>(double2*, const cplx<R>*, const cplx<R>*, long long, int, double2*, cudaStream_t); \
   template void launch_norm2<R>(double*, const cplx<R>*, long long, int, double*, cudaStream_t);                 \
-  template void launch_gram_project<R>(double2*, double2*, const cplx<R>*, long long, int, int, const cplx<R>*,  \
-                                       long long, int, double2*, cudaStream_t, const int*, int);                 \
-  template int launch_project_norm<R>(double*, cplx<R>*, const cplx<R>*, long long, int, const double2*, int,    \
-                                      long long, int, cudaStream_t, const int*, int);                            \
+  template int launch_gram_schmidt<R>(double2*, double2*, double*, cplx<R>*, const cplx<R>*, long long, int, int, \
+                                      long long, int, double2*, cudaStream_t, const int*, int);                  \
   template void launch_multiaxpy<R>(cplx<R>*, const cplx<R>*, long long, int, const double2*, int, double,       \
                                     long long, int, cudaStream_t, const int*, int);                              \
   template void launch_copy_idx<R>(cplx<R>*, const cplx<R>*, long long, const int*, long long, long long,        \

@@ -189,21 +189,17 @@ void launch_dot(double2* out, const cplx<R>* a, const cplx<R>* b, long long n, i
                 cudaStream_t st);
 template <typename R>
 void launch_norm2(double* out, const cplx<R>* a, long long n, int nrhs, double* partial, cudaStream_t st);
-// Arnoldi Gram-Schmidt against V_0 .. V_{k-1} (V_i at basis + i * bstride, each [nrhs][n]):
-// h[r][i] = the coefficients of two classical passes, from one sweep that forms <V_i, w> and
-// the newest column of the Gram matrix G[r] = V^dag V (h: [nrhs][ld], G: [nrhs][ld][ld]);
-// partial: nrhs * 2 * roundup(k, 8) * 608 entries.  Then w -= V h, and the returned number of
-// partial sums of ||w||^2 per rhs in partial (for launch_gmres_step).
+// Arnoldi Gram-Schmidt, two classical passes against V_0 .. V_{k-1} (V_i at basis + i * bstride,
+// each [nrhs][n]): h1 = V^dag w, w -= V h1, h2 = V^dag w, w -= V h2 (h1, h2: [nrhs][ld]), and the
+// returned number of partial sums of ||w||^2 per rhs in norm_partial (for launch_gmres_step;
+// nrhs * 608 entries).  partial: nrhs * roundup(k, 8) * 608 entries.
 // kdev (nullable, device): the count is *kdev + kadd instead (at most k, which sizes
 // the grid) -- the Arnoldi step number of a device-driven loop.
 template <typename R>
-void launch_gram_project(double2* h, double2* G, const cplx<R>* basis, long long bstride, int k, int ld,
-                         const cplx<R>* w, long long n, int nrhs, double2* partial, cudaStream_t st,
-                         const int* kdev = nullptr, int kadd = 0);
-template <typename R>
-int launch_project_norm(double* partial, cplx<R>* w, const cplx<R>* basis, long long bstride, int k, const double2* h,
-                        int ld, long long n, int nrhs, cudaStream_t st, const int* kdev = nullptr, int kadd = 0);
-// w[r] += sign * sum_{i<k} coef[r*ldc + i] * basis_i[r]; kdev as for launch_multidot
+int launch_gram_schmidt(double2* h1, double2* h2, double* norm_partial, cplx<R>* w, const cplx<R>* basis,
+                        long long bstride, int k, int ld, long long n, int nrhs, double2* partial, cudaStream_t st,
+                        const int* kdev = nullptr, int kadd = 0);
+// w[r] += sign * sum_{i<k} coef[r*ldc + i] * basis_i[r]; kdev as for launch_gram_schmidt
 template <typename R>
 void launch_multiaxpy(cplx<R>* w, const cplx<R>* basis, long long bstride, int k, const double2* coef, int ldc,
                       double sign, long long n, int nrhs, cudaStream_t st, const int* kdev = nullptr, int kadd = 0);
@@ -274,23 +270,22 @@ struct GmresState {
   int* done;       // [nrhs]  finished for good (frozen in later cycles)
   int m;
 };
-// h column j is in H (entries 0..j from multidot); hnorm holds ||w||.
 // One fused Arnoldi step after the operator application, for one short rhs
-// (n <= 2^17, restart <= 64): both projections of w against V_0..V_j (G: Gram matrix of the
-// basis, [m+1][m+1]), the norm, the Givens update of Hessenberg column j and V_{j+1} =
-// w / ||w||, in one launch of a thread-block cluster (16 CTAs, else 8).  jdev (nullable):
-// step on the device.  vnext (nullable): a second copy of V_{j+1}.
+// (n <= 2^17, restart <= 64): both Gram-Schmidt passes of w (overwritten) against V_0..V_j, the
+// norm, the Givens update of Hessenberg column j and V_{j+1} = w / ||w||, in one launch of a
+// thread-block cluster (16 CTAs, else 8).  jdev (nullable): step on the device.  vnext
+// (nullable): a second copy of V_{j+1}.
 bool arnoldi_fused_ok(long long n, int nrhs, int m);
 template <typename R>
-void launch_arnoldi_fused(cplx<R>* Vb, long long bstride, cplx<R>* w, long long n, const GmresState& S, double2* G,
-                          int j, const int* jdev, double tol, int final_done, cudaStream_t st,
-                          cplx<R>* vnext = nullptr);
-// The Givens update of column j: h = the coefficients of both Gram-Schmidt passes [nrhs][m+1],
+void launch_arnoldi_fused(cplx<R>* Vb, long long bstride, cplx<R>* w, long long n, const GmresState& S, int j,
+                          const int* jdev, double tol, int final_done, cudaStream_t st, cplx<R>* vnext = nullptr);
+// The Givens update of column j: h1, h2 = the coefficients of the Gram-Schmidt passes [nrhs][m+1],
 // partial = `count` sums of ||w||^2 per rhs; inv_h = 1 / ||w|| (0 for an inactive rhs).
 // `final_done`: a recurrence convergence also marks the rhs done (no true-residual check).
 // jdev (nullable, device): the step number is *jdev instead of j.
-void launch_gmres_step(const GmresState& s, int j, const double2* h, const double* partial, int count, double tol,
-                       int final_done, int nrhs, double* inv_h, cudaStream_t st, const int* jdev = nullptr);
+void launch_gmres_step(const GmresState& s, int j, const double2* h1, const double2* h2, const double* partial,
+                       int count, double tol, int final_done, int nrhs, double* inv_h, cudaStream_t st,
+                       const int* jdev = nullptr);
 // done[r] |= nrm2[r] <= (tol * bnorm[r])^2
 void launch_gmres_mark_done(const GmresState& s, const double* nrm2, double tol, int nrhs, cudaStream_t st);
 void launch_gmres_solve_y(const GmresState& s, int nrhs, cudaStream_t st);

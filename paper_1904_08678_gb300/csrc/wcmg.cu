@@ -91,8 +91,7 @@ static inline void coords(int s, const int* d, int* x) {
 // Scalars of one level's Krylov loops (device) and its (F)GMRES state.
 struct LevelScalars {
   int cap_rhs = 0, cap_m = 0;
-  DevBuf<double2> c2;  // h [rhs][m+1]; pr [2][rhs] (steps of a pair)
-  DevBuf<double2> G;   // Gram matrix of the Krylov basis [rhs][m+1][m+1]
+  DevBuf<double2> c2;  // h1, h2 [2][rhs][m+1]; pr [2][rhs] (steps of a pair)
   DevBuf<double> d;    // hn2, nrm2, inv_beta, inv_h, pp, bnorm, resid, cs... [slots][rhs]
   DevBuf<double2> H, sn, g, y;
   DevBuf<double> cs;
@@ -101,8 +100,7 @@ struct LevelScalars {
     if (rhs <= cap_rhs && m <= cap_m) return;
     rhs = std::max(rhs, cap_rhs);
     m = std::max(m, cap_m);
-    c2.ensure((size_t)rhs * ((m + 1) + 2));
-    G.ensure((size_t)rhs * (m + 1) * (m + 1));
+    c2.ensure((size_t)rhs * (2 * (m + 1) + 2));
     d.ensure((size_t)rhs * 9);
     H.ensure((size_t)rhs * (m + 1) * m);
     sn.ensure((size_t)rhs * m);
@@ -117,8 +115,9 @@ struct LevelScalars {
   void need() const {
     if (!c2.p || !d.p || !H.p || !ints.p) throw Error(WCMG_ERR_STATE, "Krylov scalars used before allocation");
   }
-  double2* h() { need(); return c2.p; }
-  double2* pr(int k = 0) { need(); return c2.p + (size_t)cap_rhs * (cap_m + 1) + (size_t)(k & 1) * cap_rhs; }
+  double2* h1() { need(); return c2.p; }
+  double2* h2() { need(); return c2.p + (size_t)cap_rhs * (cap_m + 1); }
+  double2* pr(int k = 0) { need(); return c2.p + (size_t)2 * cap_rhs * (cap_m + 1) + (size_t)(k & 1) * cap_rhs; }
   double* pp(int k = 0) { return slot(k & 1 ? 8 : 4); }
   double* slot(int k) { need(); return d.p + (size_t)k * cap_rhs; }
   GmresState state(int m) {
@@ -367,8 +366,9 @@ static void ensure_partials(wcmg_ctx* c) {
   c->partial_d.ensure((size_t)r * 608);
 }
 
-static void ensure_gram_partials(wcmg_ctx* c, int nrhs, int m) {
-  c->partial.ensure((size_t)nrhs * 2 * ((m + 7) / 8 * 8) * 608);
+// the projections on m basis vectors (restarts and K-cycles may be longer than outer_restart)
+static void ensure_basis_partials(wcmg_ctx* c, int nrhs, int m) {
+  c->partial.ensure((size_t)nrhs * ((m + 7) / 8 * 8) * 608);
 }
 
 // ---------------- accessors at a precision ----------------
@@ -850,7 +850,7 @@ static KrylovOut fgmres(wcmg_ctx* c, int l, cplx<R>* x, const cplx<R>* b, int nr
   cplx<R>* w = ws<R>(L, precond ? "fg_w" : "gm_w", nrhs);
   cplx<R>* r = ws<R>(L, precond ? "fg_r" : "gm_r", nrhs);
   const long long bstride = n * nrhs;
-  ensure_gram_partials(c, nrhs, m);
+  ensure_basis_partials(c, nrhs, m);
   GmresState S = SC.state(m);
   const int ldh = m + 1;
   norm2_op<R>(c, SC.slot(1), b, n, nrhs);
@@ -886,14 +886,13 @@ static KrylovOut fgmres(wcmg_ctx* c, int l, cplx<R>* x, const cplx<R>* b, int nr
       apply_op<R>(c, l, w, z, nrhs);
       if (arnoldi_fused_ok(n, nrhs, m)) {
         KPROF(c, WCMG_K_KRYLOV, (4.0 * (j + 1) + 6.0) * n * sizeof(cplx<R>), 32.0 * (j + 1) * n,
-              launch_arnoldi_fused<R>(Vb, bstride, w, n, S, SC.G.p, j, nullptr, tol, verify ? 0 : 1, c->st));
+              launch_arnoldi_fused<R>(Vb, bstride, w, n, S, j, nullptr, tol, verify ? 0 : 1, c->st));
       } else {
-        KPROF(c, WCMG_K_KRYLOV, (double)(j + 3) * n * nrhs * sizeof(cplx<R>), 16.0 * (j + 1) * n * nrhs,
-              launch_gram_project<R>(SC.h(), SC.G.p, Vb, bstride, j + 1, ldh, w, n, nrhs, c->partial.p, c->st));
         int nb = 0;
-        KPROF(c, WCMG_K_KRYLOV, (double)(j + 3) * n * nrhs * sizeof(cplx<R>), 8.0 * (j + 1) * n * nrhs,
-              nb = launch_project_norm<R>(c->partial_d.p, w, Vb, bstride, j + 1, SC.h(), ldh, n, nrhs, c->st));
-        launch_gmres_step(S, j, SC.h(), c->partial_d.p, nb, tol, verify ? 0 : 1, nrhs, SC.slot(3), c->st);
+        KPROF(c, WCMG_K_KRYLOV, (4.0 * (j + 1) + 6.0) * n * nrhs * sizeof(cplx<R>), 32.0 * (j + 1) * n * nrhs,
+              nb = launch_gram_schmidt<R>(SC.h1(), SC.h2(), c->partial_d.p, w, Vb, bstride, j + 1, ldh, n, nrhs,
+                                          c->partial.p, c->st));
+        launch_gmres_step(S, j, SC.h1(), SC.h2(), c->partial_d.p, nb, tol, verify ? 0 : 1, nrhs, SC.slot(3), c->st);
         launch_scale_dev<R>(Vb + (long long)(j + 1) * bstride, w, SC.slot(3), 0, n, nrhs, c->st);
       }
       ++steps;
@@ -1032,7 +1031,7 @@ static void fgmres_g(wcmg_ctx* c, int l, cplx<R>* x, const cplx<R>* b, int nrhs,
   cplx<R>* vcur = ws<R>(L, precond ? "fg_vc" : "gm_vc", nrhs);
   cplx<R>* zcur = precond ? ws<R>(L, "fg_zc", nrhs) : nullptr;
   const long long bstride = n * nrhs;
-  ensure_gram_partials(c, nrhs, m);
+  ensure_basis_partials(c, nrhs, m);
   GmresState S = SC.state(m);
   const int ldh = m + 1;
   const int* jd = &K->j;
@@ -1065,14 +1064,14 @@ static void fgmres_g(wcmg_ctx* c, int l, cplx<R>* x, const cplx<R>* b, int nrhs,
       apply_op<R>(c, l, w, z, nrhs);
       if (arnoldi_fused_ok(n, nrhs, m)) {
         KPROF(c, WCMG_K_KRYLOV, 0.0, 0.0,
-              launch_arnoldi_fused<R>(Vb, bstride, w, n, S, SC.G.p, 0, jd, tol, verify ? 0 : 1, c->st, vcur));
+              launch_arnoldi_fused<R>(Vb, bstride, w, n, S, 0, jd, tol, verify ? 0 : 1, c->st, vcur));
       } else {
-        KPROF(c, WCMG_K_KRYLOV, 0.0, 0.0,
-              launch_gram_project<R>(SC.h(), SC.G.p, Vb, bstride, m, ldh, w, n, nrhs, c->partial.p, c->st, jd, 1));
         int nb = 0;
         KPROF(c, WCMG_K_KRYLOV, 0.0, 0.0,
-              nb = launch_project_norm<R>(c->partial_d.p, w, Vb, bstride, m, SC.h(), ldh, n, nrhs, c->st, jd, 1));
-        launch_gmres_step(S, 0, SC.h(), c->partial_d.p, nb, tol, verify ? 0 : 1, nrhs, SC.slot(3), c->st, jd);
+              nb = launch_gram_schmidt<R>(SC.h1(), SC.h2(), c->partial_d.p, w, Vb, bstride, m, ldh, n, nrhs,
+                                          c->partial.p, c->st, jd, 1));
+        launch_gmres_step(S, 0, SC.h1(), SC.h2(), c->partial_d.p, nb, tol, verify ? 0 : 1, nrhs, SC.slot(3), c->st,
+                          jd);
         launch_scale_dev<R>(Vb, w, SC.slot(3), 0, n, nrhs, c->st, jd, 1, bstride, vcur);  // V_{j+1}
       }
       launch_kctl_step_end(K, S.active, nrhs, m, acc, body_count(c, slot), h_arn, c->st);
