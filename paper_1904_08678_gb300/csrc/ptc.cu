@@ -16,8 +16,8 @@
 // for the mixing, where transporting every field's 9 hops costs 3888 more.  The backward
 // passes are the same two kernels with the hops reversed and the weights conjugate-transposed
 // (T_h^dag = T_{opp h}).  Bound by the FP32 pipe (22 k multiply-adds per site and layer).
-// Forward and backward of four fields on 16^3x32, seven layer passes: 8.7 ms before, 5.7 ms
-// now (per pass: expanding 0.69 ms, contracting 0.77, weight gradients 0.84 + 0.06; before:
+// Forward and backward of four fields on 16^3x32, seven layer passes: 8.7 ms before, 5.8 ms
+// now (per pass: expanding 0.69 ms, contracting 0.78, weight gradients 0.91 + 0.06; before:
 // forward 0.68 and 0.85, backward 1.2, gradients 1.65 + 0.23).
 #include "kernels.h"
 
@@ -69,16 +69,25 @@ __device__ __forceinline__ void ptc_load_weights(float2* Ws, const float2* __res
   }
   __syncthreads();
 }
-// acc += W t, a 4 x 4 spin matrix from shared memory
+// acc += W t, a 4 x 4 spin matrix from shared memory.  The four products are summed before they
+// join acc: one chain over all hops and fields (5.79 instead of 5.84 ms for the seven passes
+// above) was half as much further from the FP64 result (2.8e-7, now 1.9e-7).
 __device__ __forceinline__ void spin_mix(float2 (&acc)[12], const float2* __restrict__ w, const float2 (&t)[12]) {
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
+  for (int a = 0; a < 4; ++a) {
+    float2 s[3];
 #pragma unroll
     for (int b = 0; b < 4; ++b) {
       const float2 wab = w[4 * a + b];
 #pragma unroll
-      for (int c = 0; c < 3; ++c) cmac(acc[3 * a + c], wab, t[3 * b + c]);
+      for (int c = 0; c < 3; ++c) {
+        if (b == 0) s[c] = cmul(wab, t[c]);
+        else cmac(s[c], wab, t[3 * b + c]);
+      }
     }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) acc[3 * a + c] += s[c];
+  }
 }
 
 // Expanding layer (1 -> nf fields): out_i(x) = sum_h W_ih (T_h in)(x); each thread forms OG
@@ -184,11 +193,14 @@ __global__ void __launch_bounds__(128) k_ptc_contract(float2* __restrict__ out, 
 // sum_x g[a] conj((T_h in_j)[b]) = sum_y (T_h^dag g)[a] conj(in_j[b]), is P^dag with m = its
 // inputs and t = T_h^dag g.  A CTA stages WG_S sites at a time in shared memory ([row][c, site]),
 // and thread (c, ti, tj) sums a 4 x 6 tile (rows ti + TI q, columns tj + 6 p) over the sites of
-// colour c: 10 shared reads per 24 complex multiply-adds, against one warp reduction of 16
-// values per 48 before.  Three CTAs per SM: one stages while the others multiply.  The
-// colours are added in a fixed order and written as one partial per CTA (WG_TILES tiles, so
-// that the FP32 chains stay short); k_ptc_wgrad_sum and _final add the partials in FP64.
+// colour c, three columns at a time (14 shared reads per 24 complex multiply-adds, against one
+// warp reduction of 16 values per 48 before).  The sums are in two levels, WG_CH sites and then
+// the CTA's WG_TILES tiles: one chain over all of its 128 sites was twice as far from the FP64
+// result (3.4e-7, now 1.75e-7; 0.84 instead of 0.91 ms on the sizes above).
+// Three CTAs per SM: one stages while the others multiply.  The colours are added in a fixed
+// order and written as one partial per CTA; k_ptc_wgrad_sum and _final add the partials in FP64.
 constexpr int WG_S = 32, WG_TILES = 4, WG_P = 3 * WG_S + 1;
+constexpr int WG_CH = 16;    // sites per first-level sum
 constexpr int WG_COLS = 36;  // 9 hops x 4 spins
 constexpr int WG_T = 224;    // 3 colours x 12 x 6 threads multiply, all stage
 __global__ void __maxnreg__(96) k_ptc_wgrad_partial(float2* __restrict__ partial, const float2* __restrict__ mf,
@@ -204,11 +216,11 @@ __global__ void __maxnreg__(96) k_ptc_wgrad_partial(float2* __restrict__ partial
   const int rows = 4 * nf, TI = nf;  // nf <= 12
   const int colour = threadIdx.x / 72, t = threadIdx.x % 72;
   const int ti = t / 6, tj = t % 6;
-  float2 acc[4][6];
+  float2 tot[4][6];
 #pragma unroll
   for (int q = 0; q < 4; ++q)
 #pragma unroll
-    for (int p = 0; p < 6; ++p) acc[q][p] = make_float2(0.f, 0.f);
+    for (int p = 0; p < 6; ++p) tot[q][p] = make_float2(0.f, 0.f);
   for (int u = 0; u < WG_TILES; ++u) {
     const long long tile = (long long)blockIdx.x * WG_TILES + u;
     if (tile >= (long long)tps * nrhs) break;  // uniform
@@ -229,17 +241,32 @@ __global__ void __maxnreg__(96) k_ptc_wgrad_partial(float2* __restrict__ partial
       for (int c = 0; c < 12; ++c) Ts[(4 * h + c / 3) * WG_P + (c % 3) * WG_S + (threadIdx.x & 31)] = v[c];
     }
     __syncthreads();
+    if (ti < TI && colour < 3) {
+#pragma unroll
+      for (int half = 0; half < 6; half += 3)
+        for (int k0 = colour * WG_S; k0 < (colour + 1) * WG_S; k0 += WG_CH) {
+          float2 acc[4][3];
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+#pragma unroll
+            for (int p = 0; p < 3; ++p) acc[q][p] = make_float2(0.f, 0.f);
 #pragma unroll 2
-    for (int k = colour * WG_S; k < (colour + 1) * WG_S && ti < TI && colour < 3; ++k) {
-      float2 a[4], b[6];
+          for (int k = k0; k < k0 + WG_CH; ++k) {
+            float2 a[4], b[3];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) a[q] = Ms[(ti + TI * q) * WG_P + k];
+            for (int q = 0; q < 4; ++q) a[q] = Ms[(ti + TI * q) * WG_P + k];
 #pragma unroll
-      for (int p = 0; p < 6; ++p) b[p] = Ts[(tj + 6 * p) * WG_P + k];
+            for (int p = 0; p < 3; ++p) b[p] = Ts[(tj + 6 * (half + p)) * WG_P + k];
 #pragma unroll
-      for (int q = 0; q < 4; ++q)
+            for (int q = 0; q < 4; ++q)
 #pragma unroll
-        for (int p = 0; p < 6; ++p) cjmac(acc[q][p], b[p], a[q]);  // m conj(t)
+              for (int p = 0; p < 3; ++p) cjmac(acc[q][p], b[p], a[q]);  // m conj(t)
+          }
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+#pragma unroll
+            for (int p = 0; p < 3; ++p) tot[q][half + p] += acc[q][p];
+        }
     }
     __syncthreads();
   }
@@ -252,8 +279,8 @@ __global__ void __maxnreg__(96) k_ptc_wgrad_partial(float2* __restrict__ partial
 #pragma unroll
         for (int p = 0; p < 6; ++p) {
           float2* o = red + (ti + TI * q) * WG_COLS + tj + 6 * p;
-          if (k == 0) *o = acc[q][p];
-          else *o += acc[q][p];
+          if (k == 0) *o = tot[q][p];
+          else *o += tot[q][p];
         }
     }
     __syncthreads();
