@@ -34,14 +34,27 @@ __global__ void k_pack_fine(cplx<R>* __restrict__ out, const double2* __restrict
   for (int c = 0; c < 12; ++c) o[(long long)c * V + s] = from_c64<R>(e[c]);
 }
 
-// The transpose goes through shared memory: a thread per site storing its own 12 entries
-// writes 16 bytes every 192 (half sectors, 2.7 TB/s); with consecutive lanes on
-// consecutive entries of a site the stores are whole lines (runs of the aggregate's x
-// extent in the external order).  Bound by HBM.  12 FP32 rhs on 24^3x48 (2.29 GB): 858 us
-// before, 372 us now; FP64, 24 fields on 16^3x32 (1.21 GB): 474 us before, 200 us now.
+// Two kernels.  A thread per site that stores its own 12 entries writes 16 bytes every 192
+// (half sectors, 2.7 TB/s), but has no barrier between its loads and its stores: the
+// better one while all CTAs run at once, one per SM (8192 to 19,456 sites x rhs 2.3 us, through
+// shared memory 2.8; from 22,000 on 3.3 and 3.2).  With the transpose through shared memory,
+// consecutive lanes on consecutive entries of a site, the stores are whole lines (runs of the
+// aggregate's x extent in the external order).  Bound by HBM.  12 FP32 rhs on 24^3x48 (2.29 GB):
+// 858 us before, 372 us now; FP64, 24 fields on 16^3x32 (1.21 GB): 474 us before, 200 us now.
 // (Packing reads the same strided pattern, but its lines stay in L1: 6.7 TB/s as it is.)
-constexpr int UNPACK_T = 128;        // sites per CTA
-constexpr int UNPACK_P = UNPACK_T + 5;  // row stride: 5 mod 16, so that 16 consecutive (site, component) hit distinct banks
+constexpr int UNPACK_T = 128;           // sites per CTA
+constexpr int UNPACK_P = UNPACK_T + 5;  // row stride: at most two of 16 consecutive (site, component) share a bank
+template <typename R>
+__global__ void __launch_bounds__(UNPACK_T) k_unpack_fine_direct(double2* __restrict__ ext,
+                                                                 const cplx<R>* __restrict__ in,
+                                                                 const int* __restrict__ perm, int V) {
+  const int s = blockIdx.x * UNPACK_T + threadIdx.x, r = blockIdx.y;
+  if (s >= V) return;
+  double2* e = ext + ((long long)r * V + perm[s]) * 12;
+  const cplx<R>* i = in + (long long)r * 12 * V;
+#pragma unroll
+  for (int c = 0; c < 12; ++c) e[c] = to_c64(i[(long long)c * V + s]);
+}
 template <typename R>
 __global__ void __launch_bounds__(UNPACK_T) k_unpack_fine(double2* __restrict__ ext, const cplx<R>* __restrict__ in,
                                                           const int* __restrict__ perm, int V, int nrhs) {
@@ -82,7 +95,9 @@ void launch_pack_fine(cplx<R>* out, const double2* ext, const int* perm, int V, 
 }
 template <typename R>
 void launch_unpack_fine(double2* ext, const cplx<R>* in, const int* perm, int V, int nrhs, cudaStream_t st) {
-  k_unpack_fine<R><<<dim3(nblk(V, UNPACK_T), nrhs), UNPACK_T, 0, st>>>(ext, in, perm, V, nrhs);
+  const dim3 grid(nblk(V, UNPACK_T), nrhs);
+  if ((long long)grid.x * nrhs <= 152) k_unpack_fine_direct<R><<<grid, UNPACK_T, 0, st>>>(ext, in, perm, V);
+  else k_unpack_fine<R><<<grid, UNPACK_T, 0, st>>>(ext, in, perm, V, nrhs);
   WCMG_LAUNCH_CHECK();
 }
 template <typename R>
