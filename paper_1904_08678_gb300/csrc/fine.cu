@@ -490,9 +490,9 @@ __device__ __forceinline__ bool on_face(const BlockInfo& bi, int s, int d) {
 // MR epilogue (DOTS): the CTA also sums <out, in> = sum conj(out) in and <out, out>
 // over its sites (FP32/FP64 per thread, FP64 across the CTA) into one partial per
 // (rhs, CTA): the minimal-residual step p = D r, alpha = <p, r>/<p, p> then needs
-// no extra pass over p and r.  A null `out` keeps the sums only (the last step of a
+// no extra pass over p and r.  Without STORE only the sums are kept (the last step of a
 // fixed-step MR, whose new residual nobody reads).
-template <typename R, int MODE, bool DOTS, int NR, bool RSD = false>
+template <typename R, int MODE, bool DOTS, int NR, bool RSD = false, bool STORE = true>
 __global__ void __launch_bounds__(128, (sizeof(R) == 4 && NR == 1) ? 6 : (sizeof(R) == 4 ? 4 : 1))
     k_dslash(cplx<R>* __restrict__ out, const cplx<R>* __restrict__ in, const cplx<R>* __restrict__ U,
              const cplx<R>* __restrict__ clov, const int* __restrict__ nbr, int V, BlockInfo bi, int hopdir, int nrhs,
@@ -569,7 +569,7 @@ __global__ void __launch_bounds__(128, (sizeof(R) == 4 && NR == 1) ? 6 : (sizeof
       }
 #pragma unroll
       for (int q = 0; q < NR; ++q)
-        if (q < nq && !(DOTS && !out)) {
+        if (STORE && q < nq) {
           cplx<R>* oq = out + off + q * rstride;
           const cplx<R>* bq = RSD ? rsd + off + q * rstride : nullptr;
 #pragma unroll
@@ -1346,17 +1346,22 @@ void launch_dslash_mr(cplx<R>* out, const cplx<R>* in, const cplx<R>* gauge, con
   const int nsb = (int)nblk(g.V, 128);
   const int nr = dslash_nr<R>(nrhs);
   const unsigned grid = (unsigned)((long long)nsb * ((nrhs + nr - 1) / nr));
+#define WCMG_DSM(NR, STORE)                                                                                        \
+  k_dslash<R, ST_FULL, true, NR, false, STORE><<<grid, 128, 0, st>>>(out, in, gauge, clov, g.nbr, g.V, bi, 0, nrhs, \
+                                                                     pr_part, pp_part, nullptr, 0, nullptr)
   bool done = false;
   if constexpr (sizeof(R) == 4) {
     if (nr == 2) {
-      k_dslash<R, ST_FULL, true, 2><<<grid, 128, 0, st>>>(out, in, gauge, clov, g.nbr, g.V, bi, 0, nrhs, pr_part,
-                                                           pp_part, nullptr, 0, nullptr);
+      if (out) WCMG_DSM(2, true);
+      else WCMG_DSM(2, false);
       done = true;
     }
   }
-  if (!done)
-    k_dslash<R, ST_FULL, true, 1><<<grid, 128, 0, st>>>(out, in, gauge, clov, g.nbr, g.V, bi, 0, nrhs, pr_part,
-                                                         pp_part, nullptr, 0, nullptr);
+  if (!done) {
+    if (out) WCMG_DSM(1, true);
+    else WCMG_DSM(1, false);
+  }
+#undef WCMG_DSM
   WCMG_LAUNCH_CHECK();
   k_mr_final<<<nrhs, 256, 0, st>>>(pr, pp, pr_part, pp_part, nsb);
   WCMG_LAUNCH_CHECK();
