@@ -17,6 +17,8 @@
 //   spinor : [12][V] complex   (component c = 3 * spin + colour)
 //   gauge  : [4][9][V] complex (entry (mu, 3 a + b) = U_mu(x)[a][b])
 //   clover : [36][V] complex   (chirality s uses entries 18 s .. 18 s + 17)
+#include <algorithm>
+
 #include "kernels.h"
 
 namespace wcmg {
@@ -1324,7 +1326,10 @@ __global__ void __launch_bounds__(256) k_mr_final(double2* __restrict__ pr, doub
   }
 }
 
-int dslash_partials(int V) { return (int)nblk(V, 32); }  // the most: 32 sites each
+// one per 128 sites and rhs, or per 32 where k_dslash_split may run
+long long dslash_partials(int V, int nrhs) {
+  return std::max((long long)nrhs * nblk(V, 128), std::min<long long>(nrhs, DS64_SITES / V) * nblk(V, 32));
+}
 
 template <typename R>
 void launch_dslash_mr(cplx<R>* out, const cplx<R>* in, const cplx<R>* gauge, const cplx<R>* clov, const LevelGeom& g,

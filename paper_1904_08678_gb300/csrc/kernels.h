@@ -63,9 +63,9 @@ void launch_sap_fine_eo(cplx<R>* x, const cplx<R>* b, const cplx<R>* Dx, const c
                         int nblocks, int steps, int nrhs, cudaStream_t st);
 // out = D in (full stencil) and, per rhs r, pr[r] = <out_r, in_r> = sum conj(out) in,
 // pp[r] = <out_r, out_r> (the minimal-residual step's two reductions, fused into the
-// stencil); out may be null: the sums only.  pr_part / pp_part: scratch of nrhs *
-// dslash_partials(V) entries.
-int dslash_partials(int V);
+// stencil); out may be null: the sums only.  pr_part / pp_part: scratch of
+// dslash_partials(V, n) entries for any nrhs up to n.
+long long dslash_partials(int V, int nrhs);
 // Masked stencil (ST_BLOCK_INTERIOR or ST_FACE_HOP) of both chirality projections of
 // nv vectors: out[i] = D_mode(Pi_+ v_i), out[nv + i] = D_mode(Pi_- v_i) (CoarsenOperator).
 template <typename R>

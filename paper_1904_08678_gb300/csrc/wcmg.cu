@@ -774,7 +774,7 @@ static void mr(wcmg_ctx* c, int l, cplx<R>* x, const cplx<R>* b, int nrhs, int s
   auto stencil = [&](int k, cplx<R>* p, const cplx<R>* r) {
     if (l == 0) {
       if (!c->have_gauge) throw Error(WCMG_ERR_STATE, "gauge field not set");
-      const long long np = (long long)max_rhs_all(c) * dslash_partials(L.g.V);
+      const long long np = dslash_partials(L.g.V, max_rhs_all(c));
       c->mr_pr.ensure(np);
       c->mr_pp.ensure(np);
       const double V = L.g.V, s = sizeof(cplx<R>);
