@@ -460,7 +460,7 @@ static const Lt* links5_of(wcmg_ctx* c, int l) {
 
 // ---------------- coarse-apply autotuner ----------------
 // Candidate launch shapes of the full nine-point coarse apply (K4 / K4m).
-static std::vector<CoarseTile> coarse_candidates(int nb, int nrhs, int lk, bool have5) {
+static std::vector<CoarseTile> coarse_candidates(int nb, int nrhs, int Vc, int lk, bool have5) {
   std::vector<CoarseTile> v;
   auto add = [&](int kind, int rr, int parts, int threads, int ntile, int stages = 0) {
     CoarseTile t;
@@ -468,7 +468,10 @@ static std::vector<CoarseTile> coarse_candidates(int nb, int nrhs, int lk, bool 
     if (coarse_tile_valid(t, nb, nrhs, ST_FULL, lk)) v.push_back(t);
   };
   if (nrhs == 1) {
-    for (int th : {128, 256, 512})
+    // the two widths around the fixed rule's: each further one costs every context's first apply
+    // 8 shapes x 12 applies (FP32 links of 512 x 48: 8.6 ms in all, 10.4 ms with three widths)
+    const bool narrow = coarse_default_tile(nb, 1, ST_FULL, Vc, lk).threads == 128;
+    for (int th : {narrow ? 128 : 256, narrow ? 256 : 512})
       for (int p : {1, 2, 4, 8})
         for (int rp : {1, 2}) add(0, 1, p, th, 0, rp);
     for (int p : {1, 2, 4, 8, 16}) add(1, 1, p, 0, 0);
@@ -553,7 +556,7 @@ static Level::TileInfo tune_coarse(wcmg_ctx* c, int l, const Lt* links, int nrhs
   ti.t = coarse_default_tile(nb, nrhs, ST_FULL, L.g.V, lk);
   try {
     ti.us_default = ti.us = time_one(nullptr);
-    const auto cands = coarse_candidates(nb, nrhs, lk, l5 != nullptr);
+    const auto cands = coarse_candidates(nb, nrhs, L.g.V, lk, l5 != nullptr);
     for (const auto& cand : cands) {
       const double us = time_one(&cand);
       if (us < ti.us) {

@@ -31,3 +31,18 @@ def test_default_rule_is_exact(lib, dims, nvec, links):
     out = dev(np.zeros_like(phi))
     ctx.apply_coarse(1, dev(phi), out, prec=prec)
     assert np.array_equal(host(out)[0], op(fields(phi, cd, nb)[0]).reshape(Vc, nb))
+
+
+# Every shape in the list is 12 applies on a context's first: two thread counts x four splits x two
+# depths, the five rhs-tile shapes, the streaming ones that hold (FP32 7, BF16 12) and the fixed rule.
+@pytest.mark.parametrize("dims", [(8, 8, 8, 8), (8, 8, 8, 16)])
+@pytest.mark.parametrize("links,count", [("F32", 29), ("BF16", 34)])
+def test_one_rhs_tuning_list_stays_short(lib, dims, links, count):
+    nvec, block = 24, (2, 2, 2, 2)
+    Vc = int(np.prod(coarse_dims(dims, block)))
+    ctx = lib.Context(lib.default_params(dims=dims, blocks=[block], nvec=[nvec], inner_prec=lib.F32,
+                                         coarse_link_prec=getattr(lib, links)))
+    ctx.set_coarse_links(1, dev(np.ones((9, Vc, 2 * nvec, 2 * nvec), dtype=complex)))
+    t = ctx.tune_coarse(1, 1, lib.F32)
+    assert t["candidates"] <= count
+    assert t["us"] <= t["us_default"]
