@@ -79,15 +79,14 @@ __global__ void __launch_bounds__(UNPACK_T) k_unpack_fine(double2* __restrict__ 
   }
 }
 
-template <typename R>
-__global__ void k_pack_gauge(cplx<R>* __restrict__ out, const double2* __restrict__ ext, const int* __restrict__ perm,
+__global__ void k_pack_gauge(double2* __restrict__ out, const double2* __restrict__ ext, const int* __restrict__ perm,
                              int V) {
   int s = blockIdx.x * blockDim.x + threadIdx.x;
   int mu = blockIdx.y;
   if (s >= V) return;
   const double2* e = ext + ((long long)mu * V + perm[s]) * 9;
 #pragma unroll
-  for (int k = 0; k < 9; ++k) out[((long long)mu * 9 + k) * V + s] = from_c64<R>(e[k]);
+  for (int k = 0; k < 9; ++k) out[((long long)mu * 9 + k) * V + s] = e[k];
 }
 
 template <typename R>
@@ -102,9 +101,8 @@ void launch_unpack_fine(double2* ext, const cplx<R>* in, const int* perm, int V,
   else k_unpack_fine<R><<<grid, UNPACK_T, 0, st>>>(ext, in, perm, V, nrhs);
   WCMG_LAUNCH_CHECK();
 }
-template <typename R>
-void launch_pack_gauge(cplx<R>* out, const double2* ext, const int* perm, int V, cudaStream_t st) {
-  k_pack_gauge<R><<<dim3(nblk(V, 128), 4), 128, 0, st>>>(out, ext, perm, V);
+void launch_pack_gauge(double2* out, const double2* ext, const int* perm, int V, cudaStream_t st) {
+  k_pack_gauge<<<dim3(nblk(V, 128), 4), 128, 0, st>>>(out, ext, perm, V);
   WCMG_LAUNCH_CHECK();
 }
 
@@ -160,17 +158,18 @@ __device__ __forceinline__ void mm_add(Su3& acc, const Su3& a, const Su3& b) {
 // separate leaves.  The chiral blocks of sigma_{mu nu} are signed Pauli matrices, so the
 // site blocks are sums of the i Fhat (no products).  FP64 units: 2 DFMA per cycle and SM.
 // 24^3x48: 10.4 ms before, 4.4 ms now (2.8 + 1.6).
-// T: [6][9][V], planes in the order (0,1) (0,2) (0,3) (1,2) (1,3) (2,3).
-__global__ void __launch_bounds__(128) k_clover_staple(double2* __restrict__ T, const double2* __restrict__ g,
-                                                       const int* __restrict__ nbr, int V) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x, plane = blockIdx.y;
+// Planes in the order (0,1) (0,2) (0,3) (1,2) (1,3) (2,3); T[plane]: [9][V].
+struct CloverPlanes { double2* T[6]; };
+__global__ void __launch_bounds__(128) k_clover_staple(CloverPlanes cp, const double2* __restrict__ g,
+                                                       const int* __restrict__ nbr, int V, int p0, int dp) {
+  const int s = blockIdx.x * blockDim.x + threadIdx.x, plane = p0 + dp * (int)blockIdx.y;
   if (s >= V) return;
   const int mu = plane < 3 ? 0 : plane < 5 ? 1 : 2, nu = plane < 3 ? plane + 1 : plane < 5 ? plane - 1 : 3;
   const int xpm = nbr[(2 * mu) * V + s], xpn = nbr[(2 * nu) * V + s], xmn = nbr[(2 * nu + 1) * V + s];
   const int xpm_mn = nbr[(2 * nu + 1) * V + xpm];  // x + mu - nu
   Su3 r = mm(load_u(g, V, nu, xpm), dag(mm(load_u(g, V, nu, s), load_u(g, V, mu, xpn))));
   mm_add<-1>(r, dag(mm(load_u(g, V, mu, xmn), load_u(g, V, nu, xpm_mn))), load_u(g, V, nu, xmn));
-  double2* t = T + (long long)plane * 9 * V + s;
+  double2* t = cp.T[plane] + s;
 #pragma unroll
   for (int k = 0; k < 9; ++k) t[(long long)k * V] = r.m[k];
 }
@@ -183,7 +182,7 @@ struct CloverSign { double s[6][2]; };  // [plane][chirality]: sigma_{mu nu} = s
 struct Herm3 { double d[3]; double2 o[3]; };
 __device__ __forceinline__ void clover_plane(Herm3 (&h)[2], const double2* __restrict__ T,
                                              const double2* __restrict__ g, const int* __restrict__ nbr, int V, int s,
-                                             int mu, int plane, double s0, double s1) {
+                                             int mu, double s0, double s1) {
   const int xmm = nbr[(2 * mu + 1) * V + s];
   double2 off[6];  // X01, X02, X12, X10, X20, X21
   double im[3] = {0, 0, 0};
@@ -191,7 +190,7 @@ __device__ __forceinline__ void clover_plane(Herm3 (&h)[2], const double2* __res
   for (int k = 0; k < 6; ++k) off[k] = make_double2(0, 0);
 #pragma unroll
   for (int half = 0; half < 2; ++half) {
-    const Su3 u = load_u(g, V, mu, half ? xmm : s), t = load_u(T, V, plane, half ? xmm : s);
+    const Su3 u = load_u(g, V, mu, half ? xmm : s), t = load_u(T, V, 0, half ? xmm : s);
     const Su3& a = half ? t : u;
     const Su3& b = half ? u : t;
 #pragma unroll
@@ -216,17 +215,19 @@ __device__ __forceinline__ void clover_plane(Herm3 (&h)[2], const double2* __res
   }
 }
 
-// C = diag + sum_k sigma_k (x) H_k per chirality: [[d + H_z, H_x - i H_y], [.., d - H_z]]
-__global__ void __launch_bounds__(128) k_clover_build(double2* __restrict__ clov, const double2* __restrict__ T,
+// C = diag + sum_k sigma_k (x) H_k per chirality: [[d + H_z, H_x - i H_y], [.., d - H_z]].
+// Z: the diagonal blocks (H_z); XY: the off-diagonal one.
+template <bool Z, bool XY>
+__global__ void __launch_bounds__(128) k_clover_build(double2* __restrict__ clov, CloverPlanes cp,
                                                       const double2* __restrict__ g, const int* __restrict__ nbr,
                                                       int V, double diag, CloverSign sg) {
   const int s = blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= V) return;
   const Herm3 zero = {{0, 0, 0}, {make_double2(0, 0), make_double2(0, 0), make_double2(0, 0)}};
-  {
+  if constexpr (Z) {
     Herm3 z[2] = {zero, zero};  // sigma_z: planes (0,1), (2,3)
-    clover_plane(z, T, g, nbr, V, s, 0, 0, sg.s[0][0], sg.s[0][1]);
-    clover_plane(z, T, g, nbr, V, s, 2, 5, sg.s[5][0], sg.s[5][1]);
+    clover_plane(z, cp.T[0], g, nbr, V, s, 0, sg.s[0][0], sg.s[0][1]);
+    clover_plane(z, cp.T[5], g, nbr, V, s, 2, sg.s[5][0], sg.s[5][1]);
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       double2* c = clov + (long long)(18 * h) * V + s;
@@ -243,11 +244,12 @@ __global__ void __launch_bounds__(128) k_clover_build(double2* __restrict__ clov
       c[17LL * V] = -z[h].o[2];
     }
   }
+  if constexpr (!XY) return;
   Herm3 x[2] = {zero, zero}, y[2] = {zero, zero};  // sigma_x: (0,3), (1,2); sigma_y: (0,2), (1,3)
-  clover_plane(x, T, g, nbr, V, s, 0, 2, sg.s[2][0], sg.s[2][1]);
-  clover_plane(x, T, g, nbr, V, s, 1, 3, sg.s[3][0], sg.s[3][1]);
-  clover_plane(y, T, g, nbr, V, s, 0, 1, sg.s[1][0], sg.s[1][1]);
-  clover_plane(y, T, g, nbr, V, s, 1, 4, sg.s[4][0], sg.s[4][1]);
+  clover_plane(x, cp.T[2], g, nbr, V, s, 0, sg.s[2][0], sg.s[2][1]);
+  clover_plane(x, cp.T[3], g, nbr, V, s, 1, sg.s[3][0], sg.s[3][1]);
+  clover_plane(y, cp.T[1], g, nbr, V, s, 0, sg.s[1][0], sg.s[1][1]);
+  clover_plane(y, cp.T[4], g, nbr, V, s, 1, sg.s[4][0], sg.s[4][1]);
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     double2* c = clov + (long long)(18 * h) * V + s;
@@ -335,13 +337,33 @@ static CloverSign clover_sign(double f) {
   return c;
 }
 
-// scratch: 54 V entries (the staples of the six planes)
+// Small lattices hold the staples of all planes at once (54 V entries, at most 57 MB): two launches.
+// Above, the diagonal blocks' two planes go first, so that 36 V entries are enough, which the
+// caller has at hand (set_gauge and D on 8^3x16 155 us in two launches, 165 in four; on 24^3x48
+// 6203 and 6229 us).
+long long clover_scratch(int V) { return V <= 1 << 16 ? 54LL * V : 0; }
 void launch_clover_build(double2* clov, const double2* gauge64, const int* nbr, int V, double m0, double csw,
-                         double2* scratch, cudaStream_t st) {
-  k_clover_staple<<<dim3(nblk(V, 128), 6), 128, 0, st>>>(scratch, gauge64, nbr, V);
-  WCMG_LAUNCH_CHECK();
+                         double2* a, double2* b, double2* scratch, cudaStream_t st) {
+  const long long n = 9LL * V;
+  const CloverPlanes all = {{scratch, scratch + n, scratch + 2 * n, scratch + 3 * n, scratch + 4 * n, scratch + 5 * n}};
+  const CloverPlanes two = {{a, b, a, a + n, b + n, a + n}};
   // C = 4 + m0 + (c_sw / 2) sum sigma (x) i Fhat, i Fhat = i (Q - Q^dag) / 8
-  k_clover_build<<<nblk(V, 128), 128, 0, st>>>(clov, scratch, gauge64, nbr, V, 4.0 + m0, clover_sign(csw / 16.0));
+  const CloverSign sg = clover_sign(csw / 16.0);
+  const unsigned grid = nblk(V, 128);
+  if (scratch) {
+    k_clover_staple<<<dim3(grid, 6), 128, 0, st>>>(all, gauge64, nbr, V, 0, 1);
+    WCMG_LAUNCH_CHECK();
+    k_clover_build<true, true><<<grid, 128, 0, st>>>(clov, all, gauge64, nbr, V, 4.0 + m0, sg);
+    WCMG_LAUNCH_CHECK();
+    return;
+  }
+  k_clover_staple<<<dim3(grid, 2), 128, 0, st>>>(two, gauge64, nbr, V, 0, 5);  // planes 0, 5
+  WCMG_LAUNCH_CHECK();
+  k_clover_build<true, false><<<grid, 128, 0, st>>>(clov, two, gauge64, nbr, V, 4.0 + m0, sg);
+  WCMG_LAUNCH_CHECK();
+  k_clover_staple<<<dim3(grid, 4), 128, 0, st>>>(two, gauge64, nbr, V, 1, 1);  // planes 1 to 4
+  WCMG_LAUNCH_CHECK();
+  k_clover_build<false, true><<<grid, 128, 0, st>>>(clov, two, gauge64, nbr, V, 4.0 + m0, sg);
   WCMG_LAUNCH_CHECK();
 }
 void launch_clover_expand(double2* ext, const double2* clov, const int* perm, int V, cudaStream_t st) {
@@ -1375,7 +1397,6 @@ void launch_dslash_mr(cplx<R>* out, const cplx<R>* in, const cplx<R>* gauge, con
 #define WCMG_INST(R)                                                                                          \
   template void launch_pack_fine<R>(cplx<R>*, const double2*, const int*, int, int, cudaStream_t);            \
   template void launch_unpack_fine<R>(double2*, const cplx<R>*, const int*, int, int, cudaStream_t);          \
-  template void launch_pack_gauge<R>(cplx<R>*, const double2*, const int*, int, cudaStream_t);                \
   template void launch_dslash<R>(cplx<R>*, const cplx<R>*, const cplx<R>*, const cplx<R>*, const LevelGeom&, \
                                  int, int, int, cudaStream_t, const unsigned char*, int, const cplx<R>*);    \
   template void launch_sap_fine<R>(cplx<R>*, const cplx<R>*, const cplx<R>*, const cplx<R>*, const cplx<R>*,  \

@@ -27,10 +27,11 @@ template <typename R>
 void launch_pack_fine(cplx<R>* out, const double2* ext, const int* perm, int V, int nrhs, cudaStream_t st);
 template <typename R>
 void launch_unpack_fine(double2* ext, const cplx<R>* in, const int* perm, int V, int nrhs, cudaStream_t st);
-template <typename R>
-void launch_pack_gauge(cplx<R>* out, const double2* ext, const int* perm, int V, cudaStream_t st);
+void launch_pack_gauge(double2* out, const double2* ext, const int* perm, int V, cudaStream_t st);
+// a, b: 18 V entries each that may be overwritten; scratch: clover_scratch(V) entries (null for 0)
+long long clover_scratch(int V);
 void launch_clover_build(double2* clov, const double2* gauge64, const int* nbr, int V, double m0, double csw,
-                         double2* scratch, cudaStream_t st);
+                         double2* a, double2* b, double2* scratch, cudaStream_t st);
 void launch_clover_expand(double2* ext, const double2* clov, const int* perm, int V, cudaStream_t st);
 // External [V][12][12] site blocks -> packed clover layout; *bad (zeroed by the
 // caller) becomes nonzero at a site whose block is not Hermitian and block diagonal

@@ -2274,14 +2274,20 @@ void wcmg_destroy(wcmg_ctx* ctx) { delete ctx; }
 const char* wcmg_last_error(const wcmg_ctx* ctx) { return ctx ? ctx->err.c_str() : "null context"; }
 
 extern "C++" {
+// The clover term of gauge64, then gauge32: on large lattices the staples take the FP32 copies'
+// place (288 bytes per site each) before those are written, so a context holds nothing for
+// them; on small ones the coarsening's column workspace, which no set-up uses meanwhile.
 static void clover_build(wcmg_ctx* c) {
   Level& L = c->L[0];
   const int V = L.g.V;
-  // the staples (864 bytes per site) live in the coarsening's column workspace, which no
-  // set-up runs concurrently with
-  double2* t = inner64(c) ? ws<double>(L, "co_T", 5) : reinterpret_cast<double2*>(ws<float>(L, "co_T", 9));
+  const long long fields = (clover_scratch(V) + L.n() - 1) / L.n();  // of double2
+  double2* t = nullptr;
+  if (fields) t = inner64(c) ? ws<double>(L, "co_T", fields) : reinterpret_cast<double2*>(ws<float>(L, "co_T", 2 * fields));
   KPROF(c, WCMG_K_CLOVER, 36.0 * V * 16 * 5, 0,
-        launch_clover_build(c->clover64.p, c->gauge64.p, L.g.d_nbr.p, V, c->p.m0, c->p.csw, t, c->st));
+        launch_clover_build(c->clover64.p, c->gauge64.p, L.g.d_nbr.p, V, c->p.m0, c->p.csw,
+                            reinterpret_cast<double2*>(c->gauge32.p), reinterpret_cast<double2*>(c->clover32.p), t,
+                            c->st));
+  launch_convert<double, float>(c->gauge32.p, c->gauge64.p, (long long)36 * V, c->st);
 }
 }  // extern "C++"
 
@@ -2295,8 +2301,7 @@ int wcmg_set_gauge(wcmg_ctx* c, const void* U, int where, void* stream) {
   c->gauge32.ensure((size_t)36 * V);
   c->clover64.ensure((size_t)36 * V);
   c->clover32.ensure((size_t)36 * V);
-  KPROF(c, WCMG_K_PACK, 36.0 * V * 32, 0, launch_pack_gauge<double>(c->gauge64.p, u, L.g.d_perm.p, V, c->st));
-  launch_pack_gauge<float>(c->gauge32.p, u, L.g.d_perm.p, V, c->st);
+  KPROF(c, WCMG_K_PACK, 36.0 * V * 32, 0, launch_pack_gauge(c->gauge64.p, u, L.g.d_perm.p, V, c->st));
   clover_build(c);
   clover_derived(c);
   c->have_gauge = true;

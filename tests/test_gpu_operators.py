@@ -310,3 +310,39 @@ def test_block_orthonormalisation_ill_conditioned_panels(lib, ortho_df, dims, bl
     cd = coarse_dims(dims, block)
     phi = to_grid(inputs.complex_gaussian(92, 0, (int(np.prod(cd)), 2 * nvec)), cd)
     assert rel(agg_g.restrict(agg_g.prolong(phi)), phi) < 1e-13  # P^dag P = 1
+
+
+def test_gauge_field_holds_only_links_and_clover(lib):
+    """36 + 36 complex entries per site in each precision (1728 bytes), and no working memory beside
+    them (lattices of more than 2^16 sites); each of the four buffers in whole pages of 2 MiB."""
+    import torch
+    dims = (16, 16, 16, 20)
+    V = int(np.prod(dims))
+    for prec in (lib.F64, lib.F32):
+        ctx = make(lib, dims, (4, 4, 4, 4), 4, prec=prec)
+        U = dev(inputs.random_gauge(dims, 0.3, 2002))
+        torch.cuda.synchronize()
+        before = torch.cuda.mem_get_info()[0]
+        ctx.set_gauge(U)
+        ctx.set_clover(1.3)
+        torch.cuda.synchronize()
+        pages = sum(-(-36 * size * V // (2 << 20)) for size in (16, 8, 16, 8))
+        assert before - torch.cuda.mem_get_info()[0] <= pages * (2 << 20)
+        del ctx
+
+
+@pytest.mark.parametrize("prec,tol", [("F64", 1e-12), ("F32", 1e-5)])
+@pytest.mark.parametrize("dims", [(6, 4, 8, 10), (16, 16, 16, 16), (16, 16, 16, 17)])
+def test_operator_after_a_new_clover_coefficient(lib, dims, prec, tol):
+    """Both precisions' links are still there after set_clover, which on more than 2^16 sites builds
+    the term in their place."""
+    block, nvec = [2 if d % 2 == 0 else 1 for d in dims], 4
+    U = inputs.random_gauge(dims, 0.35, 2003)
+    ctx = make(lib, dims, block, nvec)
+    ctx.set_gauge(dev(U))
+    ctx.set_clover(0.6)
+    b = inputs.complex_gaussian(2003, 1, (2, int(np.prod(dims)), 12))
+    x = dev(np.zeros_like(b))
+    ctx.apply_D(dev(b), x, 2, getattr(lib, prec))
+    D = WilsonClover(U, dims, -0.17, 0.6)
+    assert rel(host(x), ext([D(f) for f in fields(b, dims, 12)])) < tol
