@@ -79,13 +79,13 @@ void launch_dslash_mr(cplx<R>* out, const cplx<R>* in, const cplx<R>* gauge, con
 // ---- transfers (transfer.cu) ----
 // `fine` selects the component-major fine layout [ncomp][V]; otherwise fields are
 // site-major [V][ncomp].  Vectors and fields of one level share the layout.
-// face >= 0 restricts only the sites on that face of every aggregate (2 mu: +mu
-// face, 2 mu + 1: -mu face; `block` = aggregate extents); other sites are not read.
 template <typename R>
 void launch_restrict(cplx<R>* coarse, const cplx<R>* in, const cplx<R>* vecs, int Vf, int nc, int bvol, int nvec,
-                     int nrhs, bool fine, cudaStream_t st, int face = -1, const int* block = nullptr);
+                     int nrhs, bool fine, cudaStream_t st);
 // Restriction of nrhs operator columns straight into block d of the link rows: rhs r is
-// column first + r (r < nfirst) or second + r.
+// column first + r (r < nfirst) or second + r.  face >= 0 restricts only the sites on that face
+// of every aggregate (2 mu: +mu face, 2 mu + 1: -mu face; `block` = aggregate extents); other
+// sites are not read.
 struct LinkCols {
   int ld = 0, d = 0;
   int first = 0, nfirst = 0, second = 0;

@@ -31,8 +31,8 @@ __device__ __forceinline__ long long elem_addr(bool fine, int blk, int e, int s,
 // Face restriction (coarsening): only the sites of an aggregate whose neighbour
 // across face `fd` (2 mu for +mu, 2 mu + 1 for -mu) lies in the next aggregate.
 struct FaceSel {
-  int fd;     // -1: whole aggregate
-  int b[4];   // aggregate extents
+  int fd = -1;              // -1: whole aggregate
+  int b[4] = {1, 1, 1, 1};  // aggregate extents
 };
 
 // local site of the aggregate for index f over the selected sites
@@ -58,7 +58,7 @@ __device__ __forceinline__ int face_site(const FaceSel& fs, int f) {
 template <typename R, int RR, int VPW>
 __global__ void __launch_bounds__(256) k_restrict(cplx<R>* __restrict__ out, const cplx<R>* __restrict__ in,
                                                   const cplx<R>* __restrict__ vecs, int Vf, int nc, int bvol,
-                                                  int nvec, int nrhs, bool fine, FaceSel fs) {
+                                                  int nvec, int nrhs, bool fine) {
   using T = cplx<R>;
   constexpr int CH = 256;
   __shared__ T ps[RR][CH];
@@ -68,8 +68,7 @@ __global__ void __launch_bounds__(256) k_restrict(cplx<R>* __restrict__ out, con
   const int blk = blockIdx.x / ntile, r0 = (blockIdx.x % ntile) * RR, s = blockIdx.y;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int half = nc >> 1, nb = 2 * nvec;
-  const int nsite = fs.fd < 0 ? bvol : bvol / fs.b[fs.fd >> 1];
-  const int nelem = nsite * half;
+  const int nelem = bvol * half;
   const int Vc = Vf / bvol;
   const long long fstride = (long long)Vf * nc;
   const T* vb[VPW];
@@ -87,11 +86,7 @@ __global__ void __launch_bounds__(256) k_restrict(cplx<R>* __restrict__ out, con
     // stage: element -> offset (fast index of the layout first), and the rhs values
     const int e = c0 + threadIdx.x;
     if (e < nelem) {
-      int c, f;
-      if (fine) { c = s * half + e / nsite; f = e % nsite; }
-      else { f = e / half; c = s * half + e % half; }
-      const int site = blk * bvol + face_site(fs, f);
-      const int a = fine ? c * Vf + site : site * nc + c;
+      const int a = (int)elem_addr(fine, blk, e, s, Vf, nc, bvol);
       off_s[threadIdx.x] = a;
 #pragma unroll
       for (int r = 0; r < RR; ++r) ps[r][threadIdx.x] = (r0 + r < nrhs) ? in[(r0 + r) * fstride + a] : czero<R>();
@@ -268,7 +263,7 @@ static bool vectors_once(int Vf, int nc, int nvec) {
 template <typename R, int UNR>
 __global__ void __launch_bounds__(256) k_restrict_few(cplx<R>* __restrict__ out, const cplx<R>* __restrict__ in,
                                                       const cplx<R>* __restrict__ vecs, int Vf, int nc, int bvol,
-                                                      int nvec, int nrhs, bool fine, FaceSel fs) {
+                                                      int nvec, int nrhs, bool fine) {
   using T = cplx<R>;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int vgroups = (nvec + 7) / 8;
@@ -281,13 +276,11 @@ __global__ void __launch_bounds__(256) k_restrict_few(cplx<R>* __restrict__ out,
   const int Vc = Vf / bvol;
   const long long fstride = (long long)Vf * nc;
   const T* v = vecs + i * fstride;
-  const bool plain = fine && fs.fd < 0;
-  const int nsite = fs.fd < 0 ? bvol : bvol / fs.b[fs.fd >> 1];
-  const int nelem = nsite * half;
+  const int nelem = bvol * half;
   for (int r = 0; r < nrhs; ++r) {
     const T* p = in + r * fstride;
     T acc = czero<R>();
-    if (plain) {
+    if (fine) {
       // element (c, site): offset (s half + c) Vf + blk bvol + site
       const long long base = (long long)(s * half) * Vf + (long long)blk * bvol;
       for (int c = 0; c < half; ++c) {
@@ -313,11 +306,7 @@ __global__ void __launch_bounds__(256) k_restrict_few(cplx<R>* __restrict__ out,
           vv[u] = czero<R>();
           pp[u] = czero<R>();
           if (e < nelem) {
-            int c, f;
-            if (fine) { c = s * half + e / nsite; f = e % nsite; }
-            else { f = e / half; c = s * half + e % half; }
-            const int site = blk * bvol + face_site(fs, f);
-            const long long a = fine ? (long long)c * Vf + site : (long long)site * nc + c;
+            const long long a = elem_addr(false, blk, e, s, Vf, nc, bvol);
             vv[u] = v[a];
             pp[u] = p[a];
           }
@@ -333,17 +322,17 @@ __global__ void __launch_bounds__(256) k_restrict_few(cplx<R>* __restrict__ out,
 
 template <typename R>
 static void restrict_few(cplx<R>* coarse, const cplx<R>* in, const cplx<R>* vecs, int Vf, int nc, int bvol, int nvec,
-                         int nrhs, bool fine, const FaceSel& fs, cudaStream_t st) {
+                         int nrhs, bool fine, cudaStream_t st) {
   const int vgroups = (nvec + 7) / 8;
   const unsigned grid = (unsigned)((Vf / bvol) * 2 * vgroups);
   // a warp's lanes all have a piece (smaller aggregates leave too many of them idle)
-  if (fs.fd < 0 && wide_pieces<R>(in, vecs, bvol, nrhs, fine) && bvol >= 32 * (int)(16 / sizeof(cplx<R>))) {
+  if (wide_pieces<R>(in, vecs, bvol, nrhs, fine) && bvol >= 32 * (int)(16 / sizeof(cplx<R>))) {
     auto kern = vectors_once<R>(Vf, nc, nvec) ? k_restrict1<R, true> : k_restrict1<R, false>;
     kern<<<grid, 256, 0, st>>>(coarse, in, vecs, Vf, nc, bvol, nvec);
     WCMG_LAUNCH_CHECK();
     return;
   }
-  k_restrict_few<R, 8><<<grid, 256, 0, st>>>(coarse, in, vecs, Vf, nc, bvol, nvec, nrhs, fine, fs);
+  k_restrict_few<R, 8><<<grid, 256, 0, st>>>(coarse, in, vecs, Vf, nc, bvol, nvec, nrhs, fine);
   WCMG_LAUNCH_CHECK();
 }
 
@@ -451,8 +440,8 @@ __global__ void __launch_bounds__(8 * TR) k_restrict_gemm(cplx<R>* __restrict__ 
     }
 }
 
-// 4 to 15 FP32 rhs: bound by HBM (the vectors are read once for all rhs) as long as the
-// loads run ahead of the arithmetic.  The CTA's four warps split the aggregate's elements
+// 4 to 15 FP32 rhs.  The vectors are read once for all rhs; bound by the FP32 lanes' register reads
+// and the L2 latency that three chunks per warp leave (0.49 of the copy rate).  The CTA's four warps split the aggregate's elements
 // (warp w takes the chunks w, w + 4, ... of RT_KT elements) and each forms the whole M x N
 // tile (M = LX VI vectors, N = LT NT rhs) of its share: lane (ti, tr) of the LX x LT lane
 // grid owns vectors ti + LX q and rhs tr + LT p.  Each warp stages its own chunks with
@@ -460,9 +449,9 @@ __global__ void __launch_bounds__(8 * TR) k_restrict_gemm(cplx<R>* __restrict__ 
 // the sum over the warps at the end; rows of RT_RS entries (80 bytes) put the 16-byte
 // reads of 8 rows on distinct banks, and one such read serves two elements.  12 rhs,
 // Nvec 24, 24^3x48 (2.3 GB): 0.7 ms, against 2.75 ms with one shared read per complex
-// MAC and two block barriers per 256 elements (a 12-rhs solve there: 755 -> 667 ms).  48 columns stay with k_restrict_gemm: there
-// the FMA pipe's register reads bound both (354 us on 16^3x32; this layout 506 us, its
-// 3 CTAs per SM leaving 2.2 waves of 1024).
+// MAC and two block barriers per 256 elements (a 12-rhs solve there: 755 -> 667 ms).  48 columns
+// stay with k_restrict_gemm: there the FMA pipe's register reads bound both (354 us on 16^3x32;
+// this layout 506 us, its 3 CTAs per SM leaving 2.2 waves of 1024).
 constexpr int RT_KT = 8, RT_RS = RT_KT + 2, RT_ST = 3, RT_W = 4;
 
 template <int LX, int VI, int NT>
@@ -478,17 +467,16 @@ __device__ __forceinline__ void cp_async8(uint32_t dst, const void* src, int byt
 }
 
 template <int LX, int VI, int NT>
-__global__ void __launch_bounds__(32 * RT_W)
+__global__ void __launch_bounds__(32 * RT_W, VI * NT <= 9 ? 4 : 3)  // four fit by shared memory
     k_restrict_tile(float2* __restrict__ out, const float2* __restrict__ in, const float2* __restrict__ vecs, int Vf,
-                    int nc, int bvol, int nvec, int nrhs, bool fine, FaceSel fs) {
+                    int nc, int bvol, int nvec, int nrhs, bool fine) {
   constexpr int LT = 32 / LX, M = LX * VI, N = LT * NT, ROWS = M + N;
   static_assert(ROWS % 4 == 0, "four rows per copy pass");
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int blk = blockIdx.x, s = blockIdx.y, r0 = blockIdx.z * N;
   const int half = nc >> 1, nb = 2 * nvec;
-  const int nsite = fs.fd < 0 ? bvol : bvol / fs.b[fs.fd >> 1];
-  const int nelem = nsite * half, nchunk = (nelem + RT_KT - 1) / RT_KT;
+  const int nelem = bvol * half, nchunk = (nelem + RT_KT - 1) / RT_KT;
   const int Vc = Vf / bvol;
   const long long fstride = (long long)Vf * nc;
   float2* st = reinterpret_cast<float2*>(smem_raw) + (long long)warp * RT_ST * ROWS * RT_RS;
@@ -497,14 +485,7 @@ __global__ void __launch_bounds__(32 * RT_W)
     if (chunk < nchunk) {
       const int e = chunk * RT_KT + kl;
       const bool ok = e < nelem;
-      long long a = 0;
-      if (ok) {
-        int c, f;
-        if (fine) { c = s * half + e / nsite; f = e % nsite; }
-        else { f = e / half; c = s * half + e % half; }
-        const int site = blk * bvol + face_site(fs, f);
-        a = fine ? (long long)c * Vf + site : (long long)site * nc + c;
-      }
+      const long long a = ok ? elem_addr(fine, blk, e, s, Vf, nc, bvol) : 0;
       uint32_t dst = smem_u32(st + (slot * ROWS + fl) * RT_RS + kl);
 #pragma unroll
       for (int j = 0; j < ROWS / 4; ++j) {
@@ -580,21 +561,21 @@ __global__ void __launch_bounds__(32 * RT_W)
 
 template <int LX, int VI, int NT>
 static void restrict_tile_v(float2* coarse, const float2* in, const float2* vecs, int Vf, int nc, int bvol, int nvec,
-                            int nrhs, bool fine, const FaceSel& fs, cudaStream_t st) {
+                            int nrhs, bool fine, cudaStream_t st) {
   constexpr int N = 32 / LX * NT, smem = restrict_tile_smem<LX, VI, NT>();
   auto kern = k_restrict_tile<LX, VI, NT>;
   if (smem > 48 * 1024) WCMG_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
   kern<<<dim3(Vf / bvol, 2, (nrhs + N - 1) / N), 32 * RT_W, smem, st>>>(coarse, in, vecs, Vf, nc, bvol, nvec, nrhs,
-                                                                        fine, fs);
+                                                                        fine);
   WCMG_LAUNCH_CHECK();
 }
 
 // N = 4, 8, 12 or 16 rhs per CTA, M = 8, 16, 24 or 32 vectors: at most three rhs and seven
 // vectors of a tile are padding.
 static void restrict_tile(float2* coarse, const float2* in, const float2* vecs, int Vf, int nc, int bvol, int nvec,
-                          int nrhs, bool fine, const FaceSel& fs, cudaStream_t st) {
+                          int nrhs, bool fine, cudaStream_t st) {
 #define WCMG_RT(VI, NT) \
-  restrict_tile_v<8, VI, NT>(coarse, in, vecs, Vf, nc, bvol, nvec, nrhs, fine, fs, st)
+  restrict_tile_v<8, VI, NT>(coarse, in, vecs, Vf, nc, bvol, nvec, nrhs, fine, st)
 #define WCMG_RTN(VI)                      \
   do {                                    \
     if (nrhs <= 4) WCMG_RT(VI, 1);        \
@@ -623,49 +604,45 @@ static void restrict_gemm_v(cplx<R>* coarse, const cplx<R>* in, const cplx<R>* v
 
 template <typename R, int VI>
 static void restrict_gemm_vi(cplx<R>* coarse, const cplx<R>* in, const cplx<R>* vecs, int Vf, int nc, int bvol,
-                             int nvec, int nrhs, bool fine, const FaceSel& fs, cudaStream_t st) {
+                             int nvec, int nrhs, bool fine, cudaStream_t st) {
   // rhs per CTA 16 x RT: 32 (<= 32 rhs), 48 (more; the 48 column fields of nbasis 48)
-  if (nrhs <= 32) restrict_gemm_v<R, VI, 2>(coarse, in, vecs, Vf, nc, bvol, nvec, nrhs, fine, fs, st);
-  else restrict_gemm_v<R, VI, 3>(coarse, in, vecs, Vf, nc, bvol, nvec, nrhs, fine, fs, st);
+  if (nrhs <= 32) restrict_gemm_v<R, VI, 2>(coarse, in, vecs, Vf, nc, bvol, nvec, nrhs, fine, FaceSel(), st);
+  else restrict_gemm_v<R, VI, 3>(coarse, in, vecs, Vf, nc, bvol, nvec, nrhs, fine, FaceSel(), st);
 }
 
 template <typename R>
 static void restrict_gemm(cplx<R>* coarse, const cplx<R>* in, const cplx<R>* vecs, int Vf, int nc, int bvol, int nvec,
-                          int nrhs, bool fine, const FaceSel& fs, cudaStream_t st) {
+                          int nrhs, bool fine, cudaStream_t st) {
   const int vi = (nvec + 7) / 8;
-  if (vi <= 2) restrict_gemm_vi<R, 2>(coarse, in, vecs, Vf, nc, bvol, nvec, nrhs, fine, fs, st);
-  else if (vi == 3) restrict_gemm_vi<R, 3>(coarse, in, vecs, Vf, nc, bvol, nvec, nrhs, fine, fs, st);
-  else restrict_gemm_vi<R, 4>(coarse, in, vecs, Vf, nc, bvol, nvec, nrhs, fine, fs, st);
+  if (vi <= 2) restrict_gemm_vi<R, 2>(coarse, in, vecs, Vf, nc, bvol, nvec, nrhs, fine, st);
+  else if (vi == 3) restrict_gemm_vi<R, 3>(coarse, in, vecs, Vf, nc, bvol, nvec, nrhs, fine, st);
+  else restrict_gemm_vi<R, 4>(coarse, in, vecs, Vf, nc, bvol, nvec, nrhs, fine, st);
 }
 
 // 4 to 15 rhs in FP64
 template <typename R, int RR>
 static void restrict_rr(cplx<R>* coarse, const cplx<R>* in, const cplx<R>* vecs, int Vf, int nc, int bvol, int nvec,
-                        int nrhs, bool fine, const FaceSel& fs, cudaStream_t st) {
+                        int nrhs, bool fine, cudaStream_t st) {
   const dim3 grid((Vf / bvol) * ((nrhs + RR - 1) / RR), 2);
   const int vpw = (nvec + 7) / 8;
-  if (vpw == 1) k_restrict<R, RR, 1><<<grid, 256, 0, st>>>(coarse, in, vecs, Vf, nc, bvol, nvec, nrhs, fine, fs);
-  else if (vpw == 2) k_restrict<R, RR, 2><<<grid, 256, 0, st>>>(coarse, in, vecs, Vf, nc, bvol, nvec, nrhs, fine, fs);
-  else if (vpw == 3) k_restrict<R, RR, 3><<<grid, 256, 0, st>>>(coarse, in, vecs, Vf, nc, bvol, nvec, nrhs, fine, fs);
-  else k_restrict<R, RR, 4><<<grid, 256, 0, st>>>(coarse, in, vecs, Vf, nc, bvol, nvec, nrhs, fine, fs);
+  if (vpw == 1) k_restrict<R, RR, 1><<<grid, 256, 0, st>>>(coarse, in, vecs, Vf, nc, bvol, nvec, nrhs, fine);
+  else if (vpw == 2) k_restrict<R, RR, 2><<<grid, 256, 0, st>>>(coarse, in, vecs, Vf, nc, bvol, nvec, nrhs, fine);
+  else if (vpw == 3) k_restrict<R, RR, 3><<<grid, 256, 0, st>>>(coarse, in, vecs, Vf, nc, bvol, nvec, nrhs, fine);
+  else k_restrict<R, RR, 4><<<grid, 256, 0, st>>>(coarse, in, vecs, Vf, nc, bvol, nvec, nrhs, fine);
   WCMG_LAUNCH_CHECK();
 }
 
 template <typename R>
 void launch_restrict(cplx<R>* coarse, const cplx<R>* in, const cplx<R>* vecs, int Vf, int nc, int bvol, int nvec,
-                     int nrhs, bool fine, cudaStream_t st, int face, const int* block) {
+                     int nrhs, bool fine, cudaStream_t st) {
   if (nvec > 32) throw Error(-1, "restrict supports nvec <= 32");
-  FaceSel fs;
-  fs.fd = face;
-  for (int k = 0; k < 4; ++k) fs.b[k] = block ? block[k] : 1;
-  if (face >= 0 && !block) throw Error(-1, "face restriction needs the aggregate extents");
   if (nrhs >= 16) {
-    restrict_gemm<R>(coarse, in, vecs, Vf, nc, bvol, nvec, nrhs, fine, fs, st);
+    restrict_gemm<R>(coarse, in, vecs, Vf, nc, bvol, nvec, nrhs, fine, st);
   } else if (nrhs >= 4) {
-    if constexpr (sizeof(R) == 4) restrict_tile(coarse, in, vecs, Vf, nc, bvol, nvec, nrhs, fine, fs, st);
-    else restrict_rr<R, 4>(coarse, in, vecs, Vf, nc, bvol, nvec, nrhs, fine, fs, st);
+    if constexpr (sizeof(R) == 4) restrict_tile(coarse, in, vecs, Vf, nc, bvol, nvec, nrhs, fine, st);
+    else restrict_rr<R, 4>(coarse, in, vecs, Vf, nc, bvol, nvec, nrhs, fine, st);
   } else {
-    restrict_few<R>(coarse, in, vecs, Vf, nc, bvol, nvec, nrhs, fine, fs, st);
+    restrict_few<R>(coarse, in, vecs, Vf, nc, bvol, nvec, nrhs, fine, st);
   }
 }
 
@@ -1219,7 +1196,7 @@ void launch_make_columns(cplx<R>* cols, const cplx<R>* vecs, int Vf, int nc, int
 
 #define WCMG_INST(R)                                                                                            \
   template void launch_restrict<R>(cplx<R>*, const cplx<R>*, const cplx<R>*, int, int, int, int, int, bool,     \
-                                   cudaStream_t, int, const int*);                                              \
+                                   cudaStream_t);                                                               \
   template void launch_restrict_links<R>(cplx<R>*, const cplx<R>*, const cplx<R>*, int, int, int, int, int,     \
                                          bool, cudaStream_t, int, const int*, const LinkCols&);                 \
   template void launch_prolong<R>(cplx<R>*, const cplx<R>*, const cplx<R>*, int, int, int, int, int, bool,      \

@@ -697,17 +697,15 @@ static void apply_op(wcmg_ctx* c, int l, cplx<R>* out, const cplx<R>* in, int nr
 }
 
 template <typename R>
-static void restrict_op(wcmg_ctx* c, int l, cplx<R>* coarse, const cplx<R>* fine, int nrhs, int face = -1) {
+static void restrict_op(wcmg_ctx* c, int l, cplx<R>* coarse, const cplx<R>* fine, int nrhs) {
   Level& L = c->L[l];
   if (!L.have_P) throw Error(WCMG_ERR_STATE, "prolongator of level not built");
   if (!c->in_coarsen && !c->capturing) c->opc[WCMG_OPC_RESTRICT][l] += nrhs;
   const double s = sizeof(cplx<R>);
-  const double frac = face < 0 ? 1.0 : 1.0 / L.g.b[face >> 1];  // share of the sites read
   KPROF(c, WCMG_K_RESTRICT,
-        frac * (double)L.n() * s * (L.nvec + nrhs) + (double)L.g.V / L.g.bvol * 2 * L.nvec * s * nrhs,
-        frac * (double)L.n() * 8.0 * L.nvec * nrhs,
-        launch_restrict<R>(coarse, fine, Prec<R>::vecs(c, L), L.g.V, L.nc, L.g.bvol, L.nvec, nrhs, L.fine, c->st,
-                           face, L.g.b));
+        (double)L.n() * s * (L.nvec + nrhs) + (double)L.g.V / L.g.bvol * 2 * L.nvec * s * nrhs,
+        (double)L.n() * 8.0 * L.nvec * nrhs,
+        launch_restrict<R>(coarse, fine, Prec<R>::vecs(c, L), L.g.V, L.nc, L.g.bvol, L.nvec, nrhs, L.fine, c->st));
 }
 template <typename R>
 static void prolong_op(wcmg_ctx* c, int l, cplx<R>* fine, const cplx<R>* coarse, int nrhs) {
