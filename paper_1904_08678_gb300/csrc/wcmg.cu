@@ -3217,12 +3217,6 @@ int wcmg_load_setup(wcmg_ctx* c, const char* path) {
     L.v64.ensure(nv);
     if (L.fine) launch_pack_fine<double>(L.v64.p, d, L.g.d_perm.p, L.g.V, L.nvec, c->st);
     else launch_pack_coarse<double>(L.v64.p, d, L.g.d_perm.p, L.g.V, L.nc, L.nvec, c->st);
-    L.raw64.ensure(nv);
-    copy_fields<double>(c, L.raw64.p, L.v64.p, (long long)nv);
-    if (!inner64(c)) {
-      L.raw32.ensure(nv);
-      launch_convert<double, float>(L.raw32.p, L.v64.p, (long long)nv, c->st);
-    }
     L.v32_valid = false;
     L.have_P = true;
     WCMG_CUDA(cudaStreamSynchronize(c->st));

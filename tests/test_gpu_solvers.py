@@ -340,3 +340,23 @@ def test_even_odd_coarsest_solve_three_levels_and_graph_replay(lib):
         assert st.converged and st.true_residual <= 1e-10
         assert st.outer_iterations == runs[0][0].outer_iterations
         assert rel(x, runs[0][1]) < 1e-13
+
+
+def test_loaded_setup_holds_no_raw_vectors(lib, tmp_path):
+    """P in FP64 and the workspace it is packed through (100 MiB each in these sizes), and 64 MiB for the
+    links and their staging: no copies of P beside them."""
+    import torch
+    dims, nvec = (16, 16, 16, 16), 8
+    p = lib.default_params(dims=dims, blocks=[(4, 4, 4, 4)], nvec=[nvec], inner_prec=lib.F32, setup_init_sweeps=1,
+                           setup_refine_sweeps=0)
+    a, b = lib.Context(p), lib.Context(p)
+    U = dev(inputs.random_gauge(dims, 0.3, 31))
+    a.set_gauge(U)
+    a.setup_seeded(1)
+    path = str(tmp_path / "setup.bin")
+    a.save_setup(path)
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    b.load_setup(path)
+    torch.cuda.synchronize()
+    assert before - torch.cuda.mem_get_info()[0] <= 2 * nvec * 12 * int(np.prod(dims)) * 16 + (64 << 20)
