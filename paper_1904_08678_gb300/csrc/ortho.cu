@@ -12,14 +12,16 @@
 //
 // Accuracy.  With W = L^-1, Q^H Q - 1 = W dG W^H for the error dG of the sums, whose entries
 // are of the order u |a_i| |a_j|: column i of Q is off by u e_i, e_i = sum_j |W_ij|^2 |a_j|^2.
-// Measured on 24 and 32 columns of 1536 rows with e from 4 to 1e10: max |Q^H Q - 1| is 1.3e-15
-// to 6.3e-15 times max e_i (1e-14 below e = 4).  A panel is therefore taken here only if no
-// e_i exceeds CQ_AMP = 8, where 24 and 32 columns are orthonormal to 1.8e-14 and 2.3e-14 (by
-// Gram-Schmidt 1.6e-14 and 1.1e-14); the others are flagged and the Gram-Schmidt kernel does
-// them.  The pivots alone do not bound e: 24 columns that each keep
+// Measured on 24 and 32 columns of 1536 rows with e from 3 to 1e10: max |Q^H Q - 1| is 0.8e-15
+// to 6e-15 times max e_i (1e-14 below).  A panel is therefore taken here only if no e_i exceeds
+// CQ_AMP = 8, where 24 and 32 columns are orthonormal to 1.4e-14 and 2.5e-14 from FP64 and to
+// 2.5e-14 and 3.5e-14 from FP32 input (by Gram-Schmidt 1.1e-14); the others are flagged and the
+// Gram-Schmidt kernel does them.  The pivots alone do not bound e: 24 columns that each keep
 // 0.36 of their squared norm can have e = 3e6.  Near-null candidates have e below 4 after the
 // initial sweeps and below 8 after two refinement sweeps on 32^3x64 (2823 of 16384 panels above
-// 4).  Error against 64 bits on mixed Gaussian panels (e = 2): 8e-15 (Gram-Schmidt 1.7e-14).
+// 4); more sweeps make them more parallel, and from the fourth on nearly all panels go to
+// Gram-Schmidt.  Error against 64 bits on mixed Gaussian panels (e = 2): 8e-15 (Gram-Schmidt
+// 1.7e-14).
 //
 // 1024 panels of 1536 x 24 (16^3x32): 3.35 ms by Gram-Schmidt; now 1.10 + 0.10 + 1.23 ms from
 // FP64 and 0.83 + 0.10 + 0.94 ms from FP32 input (Gram, factor, product).  The arithmetic
@@ -45,7 +47,7 @@ __device__ __forceinline__ long long cq_addr(bool fine, int blk, int e, int s, i
 }
 // Packed double-float: the (re, im) pair of one complex value in two-lane FP32 registers, so
 // that one instruction does both components of a step (the scalar form left the FMA pipe
-// half idle behind the issue slots and register reads).  The same roundings as dfc_mac.
+// half idle behind the issue slots and register reads).
 using f2 = unsigned long long;
 __device__ __forceinline__ f2 f2_mk(float a, float b) {
   f2 r;
@@ -79,7 +81,9 @@ __device__ __forceinline__ f2 f2_fma(f2 a, f2 b, f2 c) {
 }
 struct dfp { f2 h, l; };  // lanes: (re, im)
 __device__ __forceinline__ dfp dfp_zero() { return {0ULL, 0ULL}; }
-// acc += x y lane by lane; XS, YS: x, y have zero low parts
+// acc += x y lane by lane; XS, YS: x, y have zero low parts.  The two error terms join the low
+// part one after the other: the error of an FP32 entry's square has fixed last bits, and added
+// to e first its rounding was biased (e = 8, 32 columns from FP32: 5.6e-14, now 3.5e-14).
 template <bool XS, bool YS>
 __device__ __forceinline__ void dfp_mac(dfp& acc, const dfp& x, const dfp& y) {
   const f2 p = f2_mul(x.h, y.h);
@@ -89,7 +93,7 @@ __device__ __forceinline__ void dfp_mac(dfp& acc, const dfp& x, const dfp& y) {
   const f2 s = f2_add(acc.h, p), v = f2_sub(s, acc.h);
   const f2 e = f2_add(f2_sub(acc.h, f2_sub(s, v)), f2_sub(p, v));
   acc.h = s;
-  acc.l = f2_add(acc.l, f2_add(e, pe));
+  acc.l = f2_add(f2_add(acc.l, pe), e);
 }
 __device__ __forceinline__ dfp dfp_norm(const dfp& a) {
   const f2 h = f2_add(a.h, a.l);

@@ -98,3 +98,23 @@ def test_chained_columns_stay_orthonormal(nvec, keep):
         q = a.reshape(nvec, 256, 2, 6)[:, :, s].reshape(nvec, -1)
         assert np.abs(q.conj() @ q.T - np.eye(nvec)).max() < 2e-14 * cond
     assert rel(a, b) < 2e-14 * cond
+
+
+@pytest.mark.parametrize("nvec,keep", [(32, 0.8), (24, 0.75), (24, 0.6), (10, 0.283)])
+def test_chained_columns_from_fp32(nvec, keep):
+    """The set-up's FP32 vectors (no sweeps): the same bound for the factor of the rounded columns,
+    whose condition number the rounding changes by less than 1e-6 x condition."""
+    from paper_1904_08678_gb300 import wcmg
+    dims, block = (4, 4, 4, 8), (4, 4, 4, 4)
+    v, cond = chained_panels(nvec, keep)
+    v = np.concatenate([v, v[:, ::-1]], axis=1).astype(np.complex64).astype(complex)  # two aggregates along t
+    ctx = wcmg.Context(wcmg.default_params(dims=dims, blocks=[block], nvec=[nvec], ortho_df=1, inner_prec=wcmg.F32,
+                                           setup_init_sweeps=0, setup_refine_sweeps=0))
+    ctx.set_gauge(dev(inputs.random_gauge(dims, 0.3, 36)))
+    ctx.setup(dev(v))
+    out = dev(np.full(v.shape, np.nan, dtype=complex))
+    ctx.get_nullvecs(0, out)
+    a, b = host(out), q_factor(dims, block, nvec, v, 0)
+    for q in (a.reshape(nvec, 2, 256, 2, 6)[:, i, :, s].reshape(nvec, -1) for i in (0, 1) for s in (0, 1)):
+        assert np.abs(q.conj() @ q.T - np.eye(nvec)).max() < 2e-14 * cond
+    assert rel(a, b) < 2e-14 * cond
