@@ -16,8 +16,8 @@
 // for the mixing, where transporting every field's 9 hops costs 3888 more.  The backward
 // passes are the same two kernels with the hops reversed and the weights conjugate-transposed
 // (T_h^dag = T_{opp h}).  Bound by the FP32 pipe (22 k multiply-adds per site and layer).
-// Forward and backward of four fields on 16^3x32, seven layer passes: 8.7 ms before, 5.8 ms
-// now (per pass: expanding 0.69 ms, contracting 0.78, weight gradients 0.91 + 0.06; before:
+// Forward and backward of four fields on 16^3x32, seven layer passes: 8.7 ms before, 5.6 ms
+// now (per pass: expanding 0.69 ms, contracting 0.78, weight gradients 0.78 + 0.06; before:
 // forward 0.68 and 0.85, backward 1.2, gradients 1.65 + 0.23).
 #include "kernels.h"
 
@@ -70,8 +70,8 @@ __device__ __forceinline__ void ptc_load_weights(float2* Ws, const float2* __res
   __syncthreads();
 }
 // acc += W t, a 4 x 4 spin matrix from shared memory.  The four products are summed before they
-// join acc: one chain over all hops and fields (5.79 instead of 5.84 ms for the seven passes
-// above) was half as much further from the FP64 result (2.8e-7, now 1.9e-7).
+// join acc: one chain over all hops and fields (45 us less in the seven passes above) was half
+// as much further from the FP64 result (2.8e-7, now 1.9e-7).
 __device__ __forceinline__ void spin_mix(float2 (&acc)[12], const float2* __restrict__ w, const float2 (&t)[12]) {
 #pragma unroll
   for (int a = 0; a < 4; ++a) {
@@ -196,18 +196,21 @@ __global__ void __launch_bounds__(128) k_ptc_contract(float2* __restrict__ out, 
 // colour c, three columns at a time (14 shared reads per 24 complex multiply-adds, against one
 // warp reduction of 16 values per 48 before).  The sums are in two levels, WG_CH sites and then
 // the CTA's WG_TILES tiles: one chain over all of its 128 sites was twice as far from the FP64
-// result (3.4e-7, now 1.75e-7; 0.84 instead of 0.91 ms on the sizes above).
-// Three CTAs per SM: one stages while the others multiply.  The colours are added in a fixed
-// order and written as one partial per CTA; k_ptc_wgrad_sum and _final add the partials in FP64.
+// result (3.4e-7, now 1.75e-7).  Two CTAs per SM, one of which stages while the other multiplies:
+// a quarter of the SM's registers holds five warps of 96, and three CTAs would put six on some
+// of them, so the threads take 126 (96 spilled: 0.91 against 0.78 ms per gradient on the sizes
+// above).  The colours are added in a fixed order and written as one partial per CTA;
+// k_ptc_wgrad_sum and _final add the partials in FP64.
 constexpr int WG_S = 32, WG_TILES = 4, WG_P = 3 * WG_S + 1;
 constexpr int WG_CH = 16;    // sites per first-level sum
 constexpr int WG_COLS = 36;  // 9 hops x 4 spins
 constexpr int WG_T = 224;    // 3 colours x 12 x 6 threads multiply, all stage
-__global__ void __maxnreg__(96) k_ptc_wgrad_partial(float2* __restrict__ partial, const float2* __restrict__ mf,
-                                                           const float2* __restrict__ sf,
-                                                           const float2* __restrict__ U,
-                                                           const int* __restrict__ nbr, int V, int nf, int nrhs,
-                                                           bool adj) {
+__global__ void __launch_bounds__(WG_T, 2) k_ptc_wgrad_partial(float2* __restrict__ partial,
+                                                               const float2* __restrict__ mf,
+                                                               const float2* __restrict__ sf,
+                                                               const float2* __restrict__ U,
+                                                               const int* __restrict__ nbr, int V, int nf, int nrhs,
+                                                               bool adj) {
   extern __shared__ float2 sm[];
   float2* Ms = sm;                   // [4 nf][WG_P]
   float2* Ts = sm + 4 * nf * WG_P;   // [36][WG_P]
