@@ -23,9 +23,10 @@
 // Gram-Schmidt.  Error against 64 bits on mixed Gaussian panels (e = 2): 8e-15 (Gram-Schmidt
 // 1.7e-14).
 //
-// 1024 panels of 1536 x 24 (16^3x32): 3.35 ms by Gram-Schmidt; now 1.10 + 0.10 + 1.23 ms from
-// FP64 and 0.83 + 0.10 + 0.94 ms from FP32 input (Gram, factor, product).  The arithmetic
-// alone is 0.6 ms per product at the FP32 pipe's rate; the pipe is 55 % busy, the rest goes to
+// 1024 panels of 1536 x 24 (16^3x32): 3.35 ms by Gram-Schmidt; now 1.10 + 0.11 + 1.22 ms from
+// FP64 and 0.83 + 0.11 + 0.94 ms from FP32 input (Gram, factor, product).  The arithmetic
+// alone is 0.6 ms per product at the FP32 pipe's rate; the pipe is 68 % busy in the Gram kernel
+// and 55 % in the product (whose conversions to FP64 keep that unit 62 % busy), the rest goes to
 // its latency at 4 to 6 warps per scheduler.
 #include <algorithm>
 

@@ -15,9 +15,10 @@
 // the 9 sums.  Either way 9 transports per site (324 complex multiply-adds) join 5184
 // for the mixing, where transporting every field's 9 hops costs 3888 more.  The backward
 // passes are the same two kernels with the hops reversed and the weights conjugate-transposed
-// (T_h^dag = T_{opp h}).  Bound by the FP32 pipe (22 k multiply-adds per site and layer).
+// (T_h^dag = T_{opp h}).  Bound by the FP32 pipe (22 k multiply-adds per site and
+// layer; 43 to 55 % busy, its three-operand instructions' register reads allow 63 %).
 // Forward and backward of four fields on 16^3x32, seven layer passes: 8.7 ms before, 5.6 ms
-// now (per pass: expanding 0.69 ms, contracting 0.78, weight gradients 0.78 + 0.06; before:
+// now (per pass: expanding 0.69 ms, contracting 0.78, weight gradients 0.80 + 0.06; before:
 // forward 0.68 and 0.85, backward 1.2, gradients 1.65 + 0.23).
 #include "kernels.h"
 
@@ -198,7 +199,7 @@ __global__ void __launch_bounds__(128) k_ptc_contract(float2* __restrict__ out, 
 // the CTA's WG_TILES tiles: one chain over all of its 128 sites was twice as far from the FP64
 // result (3.4e-7, now 1.75e-7).  Two CTAs per SM, one of which stages while the other multiplies:
 // a quarter of the SM's registers holds five warps of 96, and three CTAs would put six on some
-// of them, so the threads take 126 (96 spilled: 0.91 against 0.78 ms per gradient on the sizes
+// of them, so the threads take 126 (96 spilled: 0.91 against 0.80 ms per gradient on the sizes
 // above).  The colours are added in a fixed order and written as one partial per CTA;
 // k_ptc_wgrad_sum and _final add the partials in FP64.
 constexpr int WG_S = 32, WG_TILES = 4, WG_P = 3 * WG_S + 1;

@@ -440,8 +440,8 @@ __global__ void __launch_bounds__(8 * TR) k_restrict_gemm(cplx<R>* __restrict__ 
     }
 }
 
-// 4 to 15 FP32 rhs.  The vectors are read once for all rhs; bound by the FP32 lanes' register reads
-// and the L2 latency that three chunks per warp leave (0.49 of the copy rate).  The CTA's four warps split the aggregate's elements
+// 4 to 15 FP32 rhs.  The vectors are read once for all rhs.  No unit is full (12 rhs on 16^3x32: L1
+// and shared memory 63 %, issue 59 %, FMA 47 %, DRAM 43 %).  The CTA's four warps split the aggregate's elements
 // (warp w takes the chunks w, w + 4, ... of RT_KT elements) and each forms the whole M x N
 // tile (M = LX VI vectors, N = LT NT rhs) of its share: lane (ti, tr) of the LX x LT lane
 // grid owns vectors ti + LX q and rhs tr + LT p.  Each warp stages its own chunks with
